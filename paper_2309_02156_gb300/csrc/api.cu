@@ -53,13 +53,19 @@ struct seq_ctx {
     KState* ks = nullptr;            // outer / FP64 solve state
     KState* ks_in = nullptr;         // inner solve state
     KState* h_ks = nullptr;          // pinned mirror of the state tail
-    int* sell_width = nullptr;       // SELL-32 copy of A used by the GMRES cycles
+    int* sell_width = nullptr;       // SELL-32 copy of A used by the solves' products
     int* sell_off = nullptr;
     int* sell_col = nullptr;
     void* sell_val = nullptr;
-    size_t sell_cap = 0;             // entries allocated
-    int* h_int = nullptr;            // pinned scratch words (SELL total and widest slice)
-    bool sell_ok = false;
+    int2* slot = nullptr;            // slot form of A: (offset, row mask) of every slot
+    size_t sell_cap = 0;             // values, columns and slot words allocated
+    size_t col_cap = 0;
+    size_t slot_cap = 0;
+    unsigned long long* d_stats = nullptr;   // totals of the matrix copy (slot_stats_kernel)
+    unsigned long long* h_stats = nullptr;   // pinned
+    bool sell_ok = false;            // a copy of this solve's matrix exists
+    int slot_w = 0;                  // slots per slice (0: not in slot form)
+    double copy_bytes = 0.0;         // bytes of the copy that a product reads
     int sell_w = 0;                  // uniform SELL slice width (0: slices differ)
     int sell_keep = 0;               // SELL arrays small enough to keep in L2 (evict-last loads)
     double* yring = nullptr;         // last four coefficient vectors (newest first)
@@ -154,7 +160,9 @@ int set_args(seq_ctx* ctx, const seq_csr* A, const double* b, double* x, double 
     h->x = x;
     h->d = ctx->d;
     h->rhs32 = ctx->rhs32;
-    h->sell_off = ctx->sell_ok ? ctx->sell_off : nullptr;
+    h->sell_off = ctx->sell_ok && !ctx->slot_w ? ctx->sell_off : nullptr;
+    h->slot = ctx->sell_ok && ctx->slot_w ? ctx->slot : nullptr;
+    h->slot_w = ctx->sell_ok ? ctx->slot_w : 0;
     h->sell_col = ctx->sell_ok ? ctx->sell_col : nullptr;
     h->sell_val = ctx->sell_ok ? ctx->sell_val : nullptr;
     h->sell_w = ctx->sell_ok ? ctx->sell_w : 0;
@@ -187,62 +195,93 @@ int ensure_val32(seq_ctx* ctx, const seq_csr* A) {
     return SEQ_OK;
 }
 
-// SELL-32 copy of the matrix for the GMRES cycles (values in FP64, or the
-// FP32 copy in mixed precision).  Sized with one small synchronisation; kept
-// off (CSR is used) when padding would more than double the storage.
+// Device arrays of the matrix copy: values (and, for SELL-32, column indices)
+// of `entries` entries, `slots` slot words.  Kept for the context's next matrix.
+int reserve_copy(seq_ctx* ctx, size_t entries, bool columns, size_t slots) {
+    const size_t el = ctx->mixed ? sizeof(float) : sizeof(double);
+    auto grow = [&](void** p, size_t* cap, size_t want, size_t size) {
+        if (want <= *cap) return true;
+        if (*p) cudaFree(*p);
+        *p = nullptr;
+        *cap = 0;
+        if (cudaMalloc(p, size * want) != cudaSuccess) return false;
+        *cap = want;
+        return true;
+    };
+    if (!grow(&ctx->sell_val, &ctx->sell_cap, entries, el) ||
+        (columns && !grow((void**)&ctx->sell_col, &ctx->col_cap, entries, sizeof(int))) ||
+        !grow((void**)&ctx->slot, &ctx->slot_cap, slots, sizeof(int2))) {
+        cudaGetLastError();
+        return fail(ctx, SEQ_ENOMEM, "cannot allocate the matrix copy of the solve");
+    }
+    return SEQ_OK;
+}
+
+// Copy of the matrix for this solve's products (values in FP64, or the FP32
+// copy in mixed precision), sized with one small synchronisation.  Slot form
+// when it exists and has at most a quarter more entries than SELL-32 (it
+// stores no columns: 10.0 bytes per FP64 entry and 5.3 per FP32 one with that
+// padding, against 12 and 8); else SELL-32; neither (CSR is used) when
+// padding would more than double the storage.
 int build_sell(seq_ctx* ctx, const seq_csr* A) {
     ctx->sell_ok = false;
+    ctx->slot_w = 0;
     const int n = A->n, ns = (n + 31) / 32;
-    launch_sell_layout(A->rowptr, n, A->nnz, ctx->sell_width, ctx->sell_off, ctx->stream);
+    launch_slot_stats(A->rowptr, A->colind, n, A->nnz, ctx->sell_width, ctx->d_stats, ctx->stream);
+    ctx->launches += 1;
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(ctx->h_int, ctx->sell_off + ns, 2 * sizeof(int), cudaMemcpyDeviceToHost,
-                       ctx->stream));
+    CK(cudaMemcpyAsync(ctx->h_stats, ctx->d_stats, 4 * sizeof(unsigned long long),
+                       cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    long long total = ctx->h_int[0];
-    const long long wmax = ctx->h_int[1];
+    long long total = (long long)ctx->h_stats[0];
+    const long long wmax = (long long)ctx->h_stats[1], slots = (long long)ctx->h_stats[2];
     ctx->sell_w = 0;
     if (total <= 0 || total >= 0x7fffffffLL || total > 2LL * A->nnz + 64LL * ns) return SEQ_OK;
-    // When padding every slice to the widest costs at most 5% more storage,
-    // use one width: the products then compute slice offsets instead of
-    // loading them (one dependent load less per slice).
-    if (wmax > 0 && 32LL * ns * wmax <= total + total / 20 && 32LL * ns * wmax < 0x7fffffffLL) {
-        launch_sell_uniform(n, (int)wmax, ctx->sell_off, ctx->stream);
-        ctx->launches += 1;
-        total = 32LL * ns * wmax;
-        ctx->h_int[0] = (int)total;
-        ctx->sell_w = (int)wmax;
-    }
     const size_t el = ctx->mixed ? sizeof(float) : sizeof(double);
-    if ((size_t)total > ctx->sell_cap) {
-        if (ctx->sell_col) cudaFree(ctx->sell_col);
-        if (ctx->sell_val) cudaFree(ctx->sell_val);
-        ctx->sell_col = nullptr;
-        ctx->sell_val = nullptr;
-        ctx->sell_cap = 0;
-        if (cudaMalloc(&ctx->sell_col, sizeof(int) * (size_t)total) != cudaSuccess ||
-            cudaMalloc(&ctx->sell_val, el * (size_t)total) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(ctx, SEQ_ENOMEM, "cannot allocate the SELL-32 copy of A");
-        }
-        ctx->sell_cap = (size_t)total;
-    }
-    if (ctx->mixed) {
-        const float* v32 = A->values_f32 ? A->values_f32 : ctx->val32;
-        launch_sell_fill_f32(A->rowptr, A->colind, v32, n, A->nnz, ctx->sell_off, ctx->sell_col,
-                             (float*)ctx->sell_val, ctx->stream);
+    const float* v32 = A->values_f32 ? A->values_f32 : ctx->val32;
+    if (slots > 0 && slots <= kMaxSlots && 32LL * ns * slots <= total + total / 4 &&
+        32LL * ns * slots < 0x7fffffffLL) {
+        total = 32LL * ns * slots;
+        int rc = reserve_copy(ctx, (size_t)total, false, (size_t)ns * slots);
+        if (rc) return rc;
+        ctx->slot_w = (int)slots;
+        ctx->copy_bytes = (double)el * (double)total + 8.0 * (double)ns * (double)slots;
+        if (ctx->mixed)
+            launch_slot_fill_f32(A->rowptr, A->colind, v32, n, A->nnz, ctx->slot_w, ctx->slot,
+                                 (float*)ctx->sell_val, ctx->stream);
+        else
+            launch_slot_fill_f64(A->rowptr, A->colind, A->values, n, A->nnz, ctx->slot_w, ctx->slot,
+                                 (double*)ctx->sell_val, ctx->stream);
+        ctx->launches += 1;
     } else {
-        launch_sell_fill_f64(A->rowptr, A->colind, A->values, n, A->nnz, ctx->sell_off,
-                             ctx->sell_col, (double*)ctx->sell_val, ctx->stream);
+        // When padding every slice to the widest costs at most 5% more storage,
+        // use one width: the products then compute slice offsets instead of
+        // loading them (one dependent load less per slice).
+        if (wmax > 0 && 32LL * ns * wmax <= total + total / 20 && 32LL * ns * wmax < 0x7fffffffLL) {
+            launch_sell_uniform(n, (int)wmax, ctx->sell_off, ctx->stream);
+            total = 32LL * ns * wmax;
+            ctx->sell_w = (int)wmax;
+        } else {
+            launch_sell_scan(ctx->sell_width, n, ctx->sell_off, ctx->stream);
+        }
+        int rc = reserve_copy(ctx, (size_t)total, true, 0);
+        if (rc) return rc;
+        ctx->copy_bytes = (4.0 + (double)el) * (double)total + 4.0 * (ns + 1);
+        if (ctx->mixed)
+            launch_sell_fill_f32(A->rowptr, A->colind, v32, n, A->nnz, ctx->sell_off, ctx->sell_col,
+                                 (float*)ctx->sell_val, ctx->stream);
+        else
+            launch_sell_fill_f64(A->rowptr, A->colind, A->values, n, A->nnz, ctx->sell_off,
+                                 ctx->sell_col, (double*)ctx->sell_val, ctx->stream);
+        ctx->launches += 2;
     }
-    ctx->launches += 3;
     CK(cudaGetLastError());
     ctx->sell_ok = true;
     // Every Arnoldi step reads the matrix several times (the product and, when
     // preconditioned, every sweep): keep it in L2 when it takes at most half.
     int l2 = 0;
     cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, ctx->dev);
-    const double sell_bytes = (4.0 + (double)el) * (double)total + 4.0 * (ns + 1);
-    ctx->sell_keep = l2 > 0 && sell_bytes <= 0.5 * (double)l2;
+    ctx->sell_keep = l2 > 0 && ctx->copy_bytes <= 0.5 * (double)l2;
     return SEQ_OK;
 }
 
@@ -305,10 +344,9 @@ void add_stat(seq_ctx* ctx, int kind, int ev0, double bytes, double flops, int l
 void account_cycle(seq_ctx* ctx, bool f32, int jd, bool updated, int nnz) {
     const double n = ctx->cfg.n, E = f32 ? 4.0 : 8.0, R = ctx->cfg.restart;
     const double csr = 4.0 * (n + 1) + (4.0 + E) * nnz;
-    // The cycle's products read the SELL-32 copy when it exists (padded index
-    // and value arrays plus the slice offsets), the CSR arrays otherwise.
-    const double ns = (ctx->cfg.n + 31) / 32;
-    const double spmv_mat = ctx->sell_ok ? 4.0 * (ns + 1) + (4.0 + E) * (double)*ctx->h_int : csr;
+    // The cycle's products read the copy of the matrix when it exists (padded
+    // arrays included), the CSR arrays otherwise.
+    const double spmv_mat = ctx->sell_ok ? ctx->copy_bytes : csr;
     const int sw = ctx->cfg.precond_sweeps;
     const int pk = precond_kernels(sw);
     const int pm = sw > 0 ? 1 : 0;                   // one mark per preconditioner application
@@ -545,7 +583,8 @@ int seq_create(const seq_config* cfg, void* cuda_stream, seq_ctx** out) {
         ok = ok && cudaMalloc(&ctx->sell_width, sizeof(int) * (size_t)ns) == cudaSuccess;
         ok = ok && cudaMalloc(&ctx->sell_off, sizeof(int) * (size_t)(ns + 2)) == cudaSuccess;
     }
-    ok = ok && cudaMallocHost(&ctx->h_int, 2 * sizeof(int)) == cudaSuccess;
+    ok = ok && cudaMalloc(&ctx->d_stats, 4 * sizeof(unsigned long long)) == cudaSuccess;
+    ok = ok && cudaMallocHost(&ctx->h_stats, 4 * sizeof(unsigned long long)) == cudaSuccess;
     {
         const int in = 4 * M + s, stride = in + M + M * M + 1;
         ok = ok && cudaMalloc(&ctx->yring, sizeof(double) * 4 * kMaxM) == cudaSuccess;
@@ -612,13 +651,13 @@ int seq_destroy(seq_ctx* ctx) {
     void* dev_ptrs[] = {ctx->X, ctx->sk_partial, ctx->W, ctx->lsq, ctx->kpartial,
                         ctx->V, ctx->w, ctx->r, ctx->p, ctx->q, ctx->val32, ctx->rhs32, ctx->r64, ctx->d,
                         ctx->d_args, ctx->d_args_in, ctx->ks, ctx->ks_in, ctx->sell_width,
-                        ctx->sell_off, ctx->sell_col, ctx->sell_val, ctx->yring, ctx->sample,
+                        ctx->sell_off, ctx->sell_col, ctx->sell_val, ctx->slot, ctx->d_stats, ctx->yring, ctx->sample,
                         ctx->yhat, ctx->used_net, ctx->Om, ctx->Zs, ctx->gpart, ctx->gcount,
                         ctx->G, ctx->Vk, ctx->lam, ctx->sweeps, ctx->Wp, ctx->lsq_red,
                         ctx->dinv, ctx->za, ctx->zb, ctx->tprec, ctx->pc_d, ctx->pc_tab};
     for (void* p : dev_ptrs)
         if (p) cudaFree(p);
-    void* host_ptrs[] = {ctx->lsq_host, ctx->h_args, ctx->h_args_in, ctx->h_ks, ctx->h_int,
+    void* host_ptrs[] = {ctx->lsq_host, ctx->h_args, ctx->h_args_in, ctx->h_ks, ctx->h_stats,
                          ctx->h_used};
     for (void* p : host_ptrs)
         if (p) cudaFreeHost(p);

@@ -58,11 +58,7 @@ __device__ __forceinline__ void cg_product(const DevArgs* __restrict__ a, KState
                                            const Epi& epi) {
     using T = typename Sys::T;
     const int n = a->n;
-    if (a->sell_off) {
-        sell_rows<T>(a->sell_off, a->sell_col, reinterpret_cast<const T*>(a->sell_val), x, n, lo,
-                     hi, kWarps, a->sell_w, a->sell_keep, &ks->bad_index, epi);
-        return;
-    }
+    if (copy_rows<T>(a, x, lo, hi, kWarps, &ks->bad_index, epi)) return;
     const T* val = Sys::val(a);
     int flag = 0;
     for (int r = lo + threadIdx.x; r < hi; r += blockDim.x) {

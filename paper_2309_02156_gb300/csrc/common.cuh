@@ -38,12 +38,14 @@ struct DevArgs {
     const int* sell_off;   // SELL-32 copy of the matrix used inside GMRES cycles
     const int* sell_col;   // (slice offsets, column indices, values; NULL: use CSR)
     const void* sell_val;
+    const int2* slot;      // slot form of the copy: (offset, row mask) of every slot of every
+                           // slice; sell_val then holds the slots' values (NULL: SELL or CSR)
     int n;
     int nnz;
     int max_iters;
     int sell_w;         // every SELL slice has this width (offsets = 32 w s); 0: read them
     int sell_keep;      // 1: load the SELL arrays with L2 evict-last priority (they fit in L2)
-    int pad1;
+    int slot_w;         // slots per slice (slot form)
     double tol;         // relative tolerance of this solve
 };
 

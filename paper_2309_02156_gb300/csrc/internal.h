@@ -151,6 +151,17 @@ void launch_cgg_true_residual_f64(const DevArgs* a, KState* ks, double* r, doubl
                                   double* partial, int nblk, int check, cudaStream_t st);
 void launch_cgg_true_residual_f32(const DevArgs* a, KState* ks, float* r, float* p,
                                   float* partial, int nblk, int check, cudaStream_t st);
+// Slot form: widths of the slices and four totals (SELL entries, widest slice,
+// most slots of a slice or kMaxSlots + 1, largest |column - row|), then the fill.
+constexpr int kMaxSlots = 24;
+void launch_slot_stats(const int* rowptr, const int* colind, int n, int nnz, int* width,
+                       unsigned long long* stats, cudaStream_t st);
+void launch_slot_fill_f64(const int* rowptr, const int* colind, const double* val, int n, int nnz,
+                          int W, int2* slot, double* v, cudaStream_t st);
+void launch_slot_fill_f32(const int* rowptr, const int* colind, const float* val, int n, int nnz,
+                          int W, int2* slot, float* v, cudaStream_t st);
+// Exclusive scan of 32 x width: off[ns] = total, off[ns + 1] = widest slice.
+void launch_sell_scan(const int* width, int n, int* off, cudaStream_t st);
 // CSR -> SELL-32 (slice widths and offsets, then the padded arrays).
 // off needs (n + 31) / 32 + 2 entries: off[ns] = total, off[ns + 1] = widest slice.
 void launch_sell_layout(const int* rowptr, int n, int nnz, int* width, int* off, cudaStream_t st);

@@ -95,6 +95,112 @@ void launch_diag_inv_f64(const DevArgs* a, double* dinv, int n, cudaStream_t st,
 // products on the same matrix).  Slice s holds rows 32 s .. 32 s + 31; its
 // width is its longest row; entry k of row 32 s + l sits at
 // off[s] + 32 k + l.  Padding entries have column -1 and value 0.
+//
+// Slot form: where the rows of a slice share their column offsets (stencils,
+// bands), the slice is stored by offset instead: slot k holds one offset and
+// the mask of the rows that have an entry at it, values at (W s + k) 32 + l, W
+// slots in every slice.  It needs every row's columns to ascend strictly and
+// lie in [0, n) (a row's entries then meet their slots in CSR order).
+
+// The next slot of a slice: the smallest offset column - row that a lane has
+// not passed yet (kNoSlot: none), called by all lanes; e is advanced in the
+// lanes that have an entry there.  *ok: the lane's columns ascend in range.
+constexpr int kNoSlot = 0x7fffffff;
+__device__ __forceinline__ int next_slot(const int* __restrict__ colind, int row, int n, int re,
+                                         int& e, int& prev, bool& mine, bool& ok) {
+    int off = kNoSlot;
+    if (e < re) {
+        const int c = colind[e];
+        ok = ok && c > prev && c < n;
+        off = c - row;
+        prev = c;
+    }
+    const int o = __reduce_min_sync(0xffffffffu, ok ? off : -kNoSlot);
+    mine = off == o && o != kNoSlot;
+    if (mine) ++e;
+    else if (off != kNoSlot) prev = -1;
+    return o;
+}
+
+// Per slice its width (longest row) into width[s]; over the matrix: stats[0]
+// the SELL entries (32 x the widths), [1] the widest slice, [2] the most slots
+// of a slice (kMaxSlots + 1: no slot form), [3] the largest |offset|.
+__global__ void __launch_bounds__(256)
+slot_stats_kernel(const int* __restrict__ rowptr, const int* __restrict__ colind, int n, int nnz,
+                  int* width, unsigned long long* stats) {
+    __shared__ unsigned long long tot[8];
+    __shared__ int wmax[8], smax[8], reach[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int s = blockIdx.x * 8 + warp, ns = (n + 31) >> 5;
+    int len = 0, slots = 0, far = 0;
+    if (s < ns) {
+        const int row = s * 32 + lane;
+        int rs = 0, re = 0;
+        if (row < n) {
+            rs = max(0, min(rowptr[row], nnz));
+            re = max(rs, min(rowptr[row + 1], nnz));
+        }
+        len = __reduce_max_sync(0xffffffffu, re - rs);
+        int e = rs, prev = -1;
+        bool ok = true, mine;
+        while (slots <= kMaxSlots) {
+            const int o = next_slot(colind, row, n, re, e, prev, mine, ok);
+            if (o == kNoSlot) break;
+            if (o == -kNoSlot) {
+                slots = kMaxSlots + 1;
+                break;
+            }
+            ++slots;
+            far = max(far, abs(o));
+        }
+        if (lane == 0) width[s] = len;
+    }
+    if (lane == 0) {
+        tot[warp] = 32ull * len;
+        wmax[warp] = len;
+        smax[warp] = slots;
+        reach[warp] = far;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) {
+            tot[0] += tot[w];
+            wmax[0] = max(wmax[0], wmax[w]);
+            smax[0] = max(smax[0], smax[w]);
+            reach[0] = max(reach[0], reach[w]);
+        }
+        atomicAdd(stats, tot[0]);
+        atomicMax(stats + 1, (unsigned long long)wmax[0]);
+        atomicMax(stats + 2, (unsigned long long)smax[0]);
+        atomicMax(stats + 3, (unsigned long long)reach[0]);
+    }
+}
+
+template <typename VT>
+__global__ void __launch_bounds__(256)
+slot_fill_kernel(const int* __restrict__ rowptr, const int* __restrict__ colind,
+                 const VT* __restrict__ val, int n, int nnz, int W, int2* slot,
+                 VT* __restrict__ val_out) {
+    const int lane = threadIdx.x & 31;
+    const int s = blockIdx.x * 8 + (threadIdx.x >> 5), ns = (n + 31) >> 5;
+    if (s >= ns) return;
+    const int row = s * 32 + lane;
+    int rs = 0, re = 0;
+    if (row < n) {
+        rs = max(0, min(rowptr[row], nnz));
+        re = max(rs, min(rowptr[row + 1], nnz));
+    }
+    int e = rs, prev = -1;
+    bool ok = true, mine;
+    for (int k = 0; k < W; ++k) {
+        const int at = e;
+        const int o = next_slot(colind, row, n, re, e, prev, mine, ok);
+        const unsigned mask = __ballot_sync(0xffffffffu, mine);
+        if (lane == 0) slot[s * W + k] = mask ? make_int2(o, (int)mask) : make_int2(0, 0);
+        val_out[(s * W + k) * 32 + lane] = mine ? val[at] : (VT)0;
+    }
+}
+
 __global__ void sell_width_kernel(const int* __restrict__ rowptr, int n, int nnz, int* width) {
     const int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -187,6 +293,29 @@ void launch_sell_layout(const int* rowptr, int n, int nnz, int* width, int* off,
     const int ns = (n + 31) / 32;
     sell_width_kernel<<<(ns + 7) / 8, 256, 0, st>>>(rowptr, n, nnz, width);
     sell_scan_kernel<<<1, 1024, 0, st>>>(width, ns, off);
+}
+
+void launch_slot_stats(const int* rowptr, const int* colind, int n, int nnz, int* width,
+                       unsigned long long* stats, cudaStream_t st) {
+    cudaMemsetAsync(stats, 0, 4 * sizeof(unsigned long long), st);
+    const int ns = (n + 31) / 32;
+    slot_stats_kernel<<<(ns + 7) / 8, 256, 0, st>>>(rowptr, colind, n, nnz, width, stats);
+}
+
+void launch_slot_fill_f64(const int* rowptr, const int* colind, const double* val, int n, int nnz,
+                          int W, int2* slot, double* v, cudaStream_t st) {
+    slot_fill_kernel<double><<<((n + 31) / 32 + 7) / 8, 256, 0, st>>>(rowptr, colind, val, n, nnz,
+                                                                     W, slot, v);
+}
+
+void launch_slot_fill_f32(const int* rowptr, const int* colind, const float* val, int n, int nnz,
+                          int W, int2* slot, float* v, cudaStream_t st) {
+    slot_fill_kernel<float><<<((n + 31) / 32 + 7) / 8, 256, 0, st>>>(rowptr, colind, val, n, nnz,
+                                                                    W, slot, v);
+}
+
+void launch_sell_scan(const int* width, int n, int* off, cudaStream_t st) {
+    sell_scan_kernel<<<1, 1024, 0, st>>>(width, (n + 31) / 32, off);
 }
 
 void launch_sell_uniform(int n, int w, int* off, cudaStream_t st) {

@@ -150,11 +150,7 @@ f32_spmv_dot_kernel(const DevArgs* __restrict__ a, KState* ks, const float* __re
     const float* vj = src ? src : V + (size_t)j * ldv;
     int lo, hi;
     block_rows(n, gridDim.x, blockIdx.x, lo, hi);
-    if (a->sell_off) {
-        sell_spmv_rows<float>(a->sell_off, a->sell_col, reinterpret_cast<const float*>(a->sell_val),
-                              vj, n, lo, hi, sig, w, kWarps, a->sell_w, a->sell_keep,
-                              &ks->bad_index);
-    } else {                                      // no SELL copy: CSR, one row per thread
+    if (!copy_rows<float>(a, vj, lo, hi, kWarps, &ks->bad_index, ScaleEpi<float>{w, sig})) {                                      // no copy: CSR, one row per thread
         const float* val = a->val32;
         int flag = 0;
         for (int r = lo + threadIdx.x; r < hi; r += blockDim.x) {

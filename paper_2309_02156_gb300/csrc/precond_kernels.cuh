@@ -203,11 +203,7 @@ __device__ __forceinline__ void precond_rows(const DevArgs* __restrict__ a, KSta
     const int n = a->n;
     int lo, hi;
     block_rows(n, gridDim.x, blockIdx.x, lo, hi);
-    if (a->sell_off) {
-        sell_rows<T>(a->sell_off, a->sell_col, reinterpret_cast<const T*>(a->sell_val), zin, n, lo,
-                     hi, (int)(blockDim.x >> 5), a->sell_w, a->sell_keep, &ks->bad_index, epi);
-        return;
-    }
+    if (copy_rows<T>(a, zin, lo, hi, (int)(blockDim.x >> 5), &ks->bad_index, epi)) return;
     const T* val = Sys::val(a);
     const T* x2 = gather_x2<Epi, T>(epi);
     int flag = 0;
