@@ -176,13 +176,17 @@ int seq_guess(seq_ctx* ctx, const seq_csr* A, const double* b_dev,
  * CG or GMRES(restart) with CGS2 per the config, optionally right-
  * preconditioned (precond_sweeps); the mixed precisions run FP32 inner solves
  * inside FP64 iterative refinement of the true residual (a GMRES inner solve
- * is one restart cycle).  CG runs in one thread block for n < 65,536 and on
- * the whole GPU above (three kernels per iteration, captured as a CUDA graph
- * of 16 iterations); the algorithm and its stopping test are the same.  With b = 0 the
+ * is one restart cycle).  CG runs as one launch with its vectors on the chip
+ * where the matrix's rows share their column offsets (stencils, bands): a
+ * thread-block cluster for small n, a cooperative grid above.  Other matrices
+ * take one thread block for n < 65,536 and the whole GPU above (three kernels
+ * per iteration, captured as a CUDA graph of 16 iterations); the algorithm and
+ * its stopping test are the same.  With b = 0 the
  * test is ||b - A x|| <= 0 and x = 0 passes it.  Does not push x.
  * Synchronises.
  * Errors: SEQ_EINVAL, SEQ_EBREAKDOWN (CG p^T A p <= 0, singular Hessenberg),
- * SEQ_ENONFINITE (NaN or Inf met), SEQ_ETIMEOUT (host cycle bound), SEQ_ECUDA. */
+ * SEQ_ENONFINITE (NaN or Inf met), SEQ_ETIMEOUT (host cycle bound, or a bounded
+ * wait between thread blocks ran out), SEQ_ECUDA. */
 int seq_solve(seq_ctx* ctx, const seq_csr* A, const double* b_dev, double tol,
               double* x_dev, seq_info* info);
 

@@ -65,6 +65,8 @@ struct seq_ctx {
     unsigned long long* h_stats = nullptr;   // pinned
     bool sell_ok = false;            // a copy of this solve's matrix exists
     int slot_w = 0;                  // slots per slice (0: not in slot form)
+    int slot_reach = 0;              // largest |column - row| (slot form)
+    TeamSlot* team = nullptr;        // posted partials of the resident CG's grid team
     double copy_bytes = 0.0;         // bytes of the copy that a product reads
     int sell_w = 0;                  // uniform SELL slice width (0: slices differ)
     int sell_keep = 0;               // SELL arrays small enough to keep in L2 (evict-last loads)
@@ -163,6 +165,7 @@ int set_args(seq_ctx* ctx, const seq_csr* A, const double* b, double* x, double 
     h->sell_off = ctx->sell_ok && !ctx->slot_w ? ctx->sell_off : nullptr;
     h->slot = ctx->sell_ok && ctx->slot_w ? ctx->slot : nullptr;
     h->slot_w = ctx->sell_ok ? ctx->slot_w : 0;
+    h->slot_reach = ctx->slot_reach;
     h->sell_col = ctx->sell_ok ? ctx->sell_col : nullptr;
     h->sell_val = ctx->sell_ok ? ctx->sell_val : nullptr;
     h->sell_w = ctx->sell_ok ? ctx->sell_w : 0;
@@ -245,6 +248,7 @@ int build_sell(seq_ctx* ctx, const seq_csr* A) {
         int rc = reserve_copy(ctx, (size_t)total, false, (size_t)ns * slots);
         if (rc) return rc;
         ctx->slot_w = (int)slots;
+        ctx->slot_reach = (int)ctx->h_stats[3];
         ctx->copy_bytes = (double)el * (double)total + 8.0 * (double)ns * (double)slots;
         if (ctx->mixed)
             launch_slot_fill_f32(A->rowptr, A->colind, v32, n, A->nnz, ctx->slot_w, ctx->slot,
@@ -507,6 +511,41 @@ int run_cg_grid(seq_ctx* ctx, bool f32) {
     return read_tail(ctx, ks);
 }
 
+// One CG solve on the system bound to (args, ks): by a resident team when the
+// matrix is in slot form and its reach fits on the chip, else grid-wide from
+// kGridCgMinRows rows on, else in one block.
+int run_cg(seq_ctx* ctx, bool f32) {
+    KState* ks = f32 ? ctx->ks_in : ctx->ks;
+    const DevArgs* args = f32 ? ctx->d_args_in : ctx->d_args;
+    const int n = ctx->cfg.n;
+    if (ctx->sell_ok && ctx->slot_w) {
+        cudaError_t e = cudaSuccess;
+        const bool taken =
+            f32 ? launch_resident_cg_f32(args, ks, (float*)ctx->r, (float*)ctx->q, ctx->team, n,
+                                         ctx->slot_w, ctx->slot_reach, ctx->stream, &e)
+                : launch_resident_cg_f64(args, ks, (double*)ctx->r, (double*)ctx->q, ctx->team, n,
+                                         ctx->slot_w, ctx->slot_reach, ctx->stream, &e);
+        if (taken) {
+            ctx->launches += 1;
+            CK(e);
+            CK(cudaGetLastError());
+            const int rc = read_tail(ctx, ks);
+            if (rc) return rc;
+            if (ctx->h_ks->status == SEQ_ETIMEOUT)
+                return fail(ctx, SEQ_ETIMEOUT, "CG: a wait between blocks ran out");
+            return SEQ_OK;
+        }
+    }
+    if (n >= kGridCgMinRows) return run_cg_grid(ctx, f32);
+    if (f32)
+        launch_cg_block_f32(args, ks, (float*)ctx->r, (float*)ctx->p, (float*)ctx->q, ctx->stream);
+    else
+        launch_cg_block_f64(args, ks, (double*)ctx->r, (double*)ctx->p, (double*)ctx->q, ctx->stream);
+    ctx->launches += 1;
+    CK(cudaGetLastError());
+    return read_tail(ctx, ks);
+}
+
 void fill_info(seq_info* info, const KState* t) {
     if (!info) return;
     info->guess_relres = t->first_relres;
@@ -572,13 +611,14 @@ int seq_create(const seq_config* cfg, void* cuda_stream, seq_ctx** out) {
         ok = ok && cudaMalloc(&ctx->r, el * (size_t)n) == cudaSuccess;
         ok = ok && cudaMalloc(&ctx->p, el * (size_t)n) == cudaSuccess;
         ok = ok && cudaMalloc(&ctx->q, el * (size_t)n) == cudaSuccess;
+        ok = ok && cudaMalloc((void**)&ctx->team, kTeamSlotBytes) == cudaSuccess;
     }
     if (ctx->mixed) {
         ok = ok && cudaMalloc(&ctx->rhs32, sizeof(float) * (size_t)n) == cudaSuccess;
         ok = ok && cudaMalloc(&ctx->r64, sizeof(double) * (size_t)n) == cudaSuccess;
         ok = ok && cudaMalloc(&ctx->d, sizeof(float) * (size_t)n) == cudaSuccess;
     }
-    if (c.krylov == SEQ_GMRES || n >= kGridCgMinRows) {     // SELL-32 copy for the cycles
+    {                                                       // matrix copy of the solves
         const int ns = (n + 31) / 32;
         ok = ok && cudaMalloc(&ctx->sell_width, sizeof(int) * (size_t)ns) == cudaSuccess;
         ok = ok && cudaMalloc(&ctx->sell_off, sizeof(int) * (size_t)(ns + 2)) == cudaSuccess;
@@ -651,7 +691,7 @@ int seq_destroy(seq_ctx* ctx) {
     void* dev_ptrs[] = {ctx->X, ctx->sk_partial, ctx->W, ctx->lsq, ctx->kpartial,
                         ctx->V, ctx->w, ctx->r, ctx->p, ctx->q, ctx->val32, ctx->rhs32, ctx->r64, ctx->d,
                         ctx->d_args, ctx->d_args_in, ctx->ks, ctx->ks_in, ctx->sell_width,
-                        ctx->sell_off, ctx->sell_col, ctx->sell_val, ctx->slot, ctx->d_stats, ctx->yring, ctx->sample,
+                        ctx->sell_off, ctx->sell_col, ctx->sell_val, ctx->slot, ctx->d_stats, ctx->team, ctx->yring, ctx->sample,
                         ctx->yhat, ctx->used_net, ctx->Om, ctx->Zs, ctx->gpart, ctx->gcount,
                         ctx->G, ctx->Vk, ctx->lam, ctx->sweeps, ctx->Wp, ctx->lsq_red,
                         ctx->dinv, ctx->za, ctx->zb, ctx->tprec, ctx->pc_d, ctx->pc_tab};
@@ -984,11 +1024,8 @@ int seq_solve(seq_ctx* ctx, const seq_csr* A, const double* b_dev, double tol, d
     CK(cudaMemsetAsync(ctx->ks_in, 0, sizeof(KState), ctx->stream));
     rc = ensure_val32(ctx, A);
     if (rc) return rc;
-    const bool grid_cg = c.krylov == SEQ_CG && c.n >= kGridCgMinRows;
-    if (c.krylov == SEQ_GMRES || grid_cg) {
-        rc = build_sell(ctx, A);
-        if (rc) return rc;
-    }
+    rc = build_sell(ctx, A);
+    if (rc) return rc;
     rc = set_args(ctx, A, b_dev, x_dev, tol, c.max_iters);
     if (rc) return rc;
     if (c.precond_sweeps > 0) {
@@ -1011,15 +1048,8 @@ int seq_solve(seq_ctx* ctx, const seq_csr* A, const double* b_dev, double tol, d
         if (c.krylov == SEQ_GMRES) {
             rc = run_gmres(ctx, false);
             if (rc) return rc;
-        } else if (grid_cg) {
-            rc = run_cg_grid(ctx, false);
-            if (rc) return rc;
         } else {
-            launch_cg_block_f64(ctx->d_args, ctx->ks, (double*)ctx->r, (double*)ctx->p,
-                                (double*)ctx->q, ctx->stream);
-            ctx->launches += 1;
-            CK(cudaGetLastError());
-            rc = read_tail(ctx, ctx->ks);
+            rc = run_cg(ctx, false);
             if (rc) return rc;
         }
         fill_info(info, ctx->h_ks);
@@ -1064,15 +1094,8 @@ int seq_solve(seq_ctx* ctx, const seq_csr* A, const double* b_dev, double tol, d
             if (c.krylov == SEQ_GMRES) {
                 rc = run_gmres(ctx, true);
                 if (rc) return rc;
-            } else if (grid_cg) {
-                rc = run_cg_grid(ctx, true);
-                if (rc) return rc;
             } else {
-                launch_cg_block_f32(ctx->d_args_in, ctx->ks_in, (float*)ctx->r, (float*)ctx->p,
-                                    (float*)ctx->q, ctx->stream);
-                ctx->launches += 1;
-                CK(cudaGetLastError());
-                rc = read_tail(ctx, ctx->ks_in);
+                rc = run_cg(ctx, true);
                 if (rc) return rc;
             }
             bad |= ctx->h_ks->bad_index;

@@ -46,6 +46,8 @@ struct DevArgs {
     int sell_w;         // every SELL slice has this width (offsets = 32 w s); 0: read them
     int sell_keep;      // 1: load the SELL arrays with L2 evict-last priority (they fit in L2)
     int slot_w;         // slots per slice (slot form)
+    int slot_reach;     // largest |column - row| (slot form)
+    int pad1;
     double tol;         // relative tolerance of this solve
 };
 

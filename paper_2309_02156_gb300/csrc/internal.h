@@ -134,6 +134,20 @@ void launch_cg_block_f64(const DevArgs* a, KState* ks, double* r, double* p, dou
 void launch_cg_block_f32(const DevArgs* a, KState* ks, float* r, float* p, float* q,
                          cudaStream_t st);
 void launch_round_f32(const double* src, float* dst, int n, cudaStream_t st);
+// CG by a resident team (resident_cg.cuh; matrices in slot form).  Up to these
+// many rows the team is one cluster of 16 (or 8) blocks, above it the grid: a
+// cluster's reduction is faster (0.9 against 2.1 us), a grid's blocks hold
+// fewer rows.  Measured per iteration (cluster, grid): FP64 15,876 rows 7.5 us,
+// 16,900 rows 8.3; FP32 32,761 rows 4.8 us (cluster), 44,100 rows 6.4 (grid)
+// with the cluster extrapolating to 5.7 there and meeting it near 57,000.
+constexpr int kClusterCgRows64 = 16384;
+constexpr int kClusterCgRows32 = 57344;
+struct TeamSlot;
+constexpr size_t kTeamSlotBytes = 16 * 2 * 160 + 128;   // slots, counter
+bool launch_resident_cg_f64(const DevArgs* a, KState* ks, double* r, double* q, TeamSlot* slots,
+                            int n, int W, int reach, cudaStream_t st, cudaError_t* launched);
+bool launch_resident_cg_f32(const DevArgs* a, KState* ks, float* r, float* q, TeamSlot* slots,
+                            int n, int W, int reach, cudaStream_t st, cudaError_t* launched);
 // Grid-wide CG for large systems (all SMs; three kernels per iteration): the
 // start (FP32: from x = 0), `iters` iterations (the body of a CUDA graph), and
 // the true residual (check != 0: convergence check and restart).

@@ -4,6 +4,7 @@
 
 #include "krylov_kernels.cuh"
 #include "cg_kernels.cuh"
+#include "resident_cg.cuh"
 
 namespace sa {
 
@@ -564,6 +565,15 @@ void launch_cg_block_f64(const DevArgs* a, KState* ks, double* r, double* p, dou
 void launch_cg_block_f32(const DevArgs* a, KState* ks, float* r, float* p, float* q,
                          cudaStream_t st) {
     cg_block_kernel<SysF32><<<1, 1024, 0, st>>>(a, ks, r, p, q);
+}
+
+bool launch_resident_cg_f64(const DevArgs* a, KState* ks, double* r, double* q, TeamSlot* slots,
+                            int n, int W, int reach, cudaStream_t st, cudaError_t* launched) {
+    return launch_resident_cg<SysF64>(a, ks, r, q, slots, n, W, reach, st, launched);
+}
+bool launch_resident_cg_f32(const DevArgs* a, KState* ks, float* r, float* q, TeamSlot* slots,
+                            int n, int W, int reach, cudaStream_t st, cudaError_t* launched) {
+    return launch_resident_cg<SysF32>(a, ks, r, q, slots, n, W, reach, st, launched);
 }
 
 void launch_cgg_start_f64(const DevArgs* a, KState* ks, double* r, double* p, double* partial,

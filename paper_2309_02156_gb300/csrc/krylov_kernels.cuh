@@ -32,7 +32,7 @@
 
 namespace sa {
 
-enum { ST_OK = 0, ST_NOT_CONVERGED = 1, ST_BREAKDOWN = -4, ST_NONFINITE = -5 };
+enum { ST_OK = 0, ST_NOT_CONVERGED = 1, ST_BREAKDOWN = -4, ST_NONFINITE = -5, ST_TIMEOUT = -6 };
 enum { CNT_START = 0, CNT_DOT = 1, CNT_PASS2 = 2, CNT_PASS3 = 3, CNT_RES = 4, CNT_REFINE = 5 };
 
 struct SysF64 {

@@ -1,0 +1,353 @@
+// Conjugate gradients with the iteration's vectors on the chip (matrices in
+// slot form; see resident.cuh): one launch per solve, two team reductions per
+// iteration.  An iteration is one product; when the recursive residual passes
+// the test the true residual b - A x is formed and the solve either ends or
+// restarts from it; p^T A p <= 0 is a breakdown.
+//
+// What bounds it: at small sizes the two reductions (0.9 us each in a cluster
+// of 16, 2.1 in a grid of 152, plus their FP64 sums), above about 200,000 rows
+// in FP64 the FP64 pipe (ten multiply-adds per row, 0.53 T/s: 5 us of the 13 us
+// per iteration at 262,144 rows).  Per iteration, before (one block below
+// 65,536 rows, three graph kernels above) and now: FP64 4,096 rows 42 -> 5.2 us,
+// 262,144 rows 22.4 -> 13.2 us; FP32 32,761 rows 58 -> 4.8 us.
+#pragma once
+
+#include "krylov_kernels.cuh"
+#include "resident.cuh"
+
+namespace sa {
+
+constexpr int kResThreads = 512;
+
+template <class Sys, class Team>
+__device__ __forceinline__ void resident_cg(const DevArgs* __restrict__ a, KState* ks,
+                                            typename Sys::T* rg, typename Sys::T* qg, Team& tm,
+                                            const ResLayout& L) {
+    using T = typename Sys::T;
+    extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ T scratch[33];
+    __shared__ T s_alpha, s_beta, s_rr;
+    __shared__ int s_go;
+    __shared__ double s_target, s_bnorm, s_first;
+    const int n = a->n, W = a->slot_w, ns = (n + 31) >> 5;
+    const int tid = threadIdx.x, bd = blockDim.x;
+    const int s_lo = min(ns, tm.rank() * L.per), s_hi = min(ns, s_lo + L.per);
+    const int nsl = s_hi - s_lo;
+    const int r_lo = s_lo * 32, r_hi = min(n, s_hi * 32), rows = max(0, r_hi - r_lo);
+    const int reach = a->slot_reach;
+    const int e_lo = max(0, r_lo - reach), e_hi = min(n, r_hi + reach);
+    const int base = r_lo - e_lo;              // own rows start here in the gathered array
+    const int above = nsl > 0 ? e_hi - r_hi : 0, below = nsl > 0 ? base : 0;
+    T* x = Sys::x(a);
+    const T* b = Sys::rhs(a);
+    const bool zero_x = sizeof(T) == 4;        // the FP32 inner solve starts from d = 0
+    // Shared arrays.
+    T* p = reinterpret_cast<T*>(dsm);
+    T* next = p + L.ext;
+    const int cap = 32 * L.per;
+    T* r = L.r_in ? next : rg + r_lo;
+    next += L.r_in ? cap : 0;
+    T* q = L.q_in ? next : qg + r_lo;
+    next += L.q_in ? cap : 0;
+    T* xs = L.x_in ? next : x + r_lo;
+    next += L.x_in ? cap : 0;
+    T* sval = next;
+    next += (size_t)L.nval * 32 * W;
+    int2* sslot = reinterpret_cast<int2*>(dsm + ((((size_t)((unsigned char*)next - dsm)) + 7) & ~(size_t)7));
+    const T* gval = reinterpret_cast<const T*>(a->sell_val) + (size_t)s_lo * W * 32;
+    const int nval = min(L.nval, nsl);
+    for (int i = tid; i < nsl * W; i += bd) sslot[i] = __ldg(a->slot + s_lo * W + i);
+    for (int i = tid; i < nval * W * 32; i += bd) sval[i] = __ldg(gval + i);
+    __syncthreads();
+    // Rows that other blocks gather go to rg (all own rows when r lies there).
+    auto edge = [&](int i) { return i < reach || i >= rows - reach; };
+    auto product = [&](const T* vec, int at, const auto& epi) {
+        if (W <= 5) res_product<T, 5>(sslot, sval, gval, vec, at, nsl, nval, W, rows, epi);
+        else if (W <= 9) res_product<T, 9>(sslot, sval, gval, vec, at, nsl, nval, W, rows, epi);
+        else res_product<T, 0>(sslot, sval, gval, vec, at, nsl, nval, W, rows, epi);
+    };
+    // r = b - A x over the global iterate, |r|^2; the edge rows are published.
+    // ldcg: other blocks wrote their rows of x during this launch.
+    auto residual = [&](bool start) {
+        T acc = 0;
+        auto take = [&](int i, T ax, bool live) {
+            if (!live) return;
+            const T ri = b[r_lo + i] - ax;
+            r[i] = ri;
+            if (L.r_in && edge(i)) rg[r_lo + i] = ri;
+            p[base + i] = ri;
+            acc = fma(ri, ri, acc);
+        };
+        if (start && zero_x) {
+            for (int i = tid; i < rows; i += bd) take(i, (T)0, true);
+        } else {
+            const int lane = tid & 31, warp = tid >> 5, nw = bd >> 5;
+            for (int s = warp; s < nsl; s += nw) {
+                const int i = s * 32 + lane;
+                T ax = 0;
+                for (int k = 0; k < W; ++k) {
+                    const int2 m = sslot[s * W + k];
+                    if ((m.y >> lane) & 1)
+                        ax = fma(gval[((size_t)s * W + k) * 32 + lane],
+                                 __ldcg(x + r_lo + i + m.x), ax);
+                }
+                take(i, ax, i < rows);
+            }
+        }
+        return acc;
+    };
+    auto fetch_halo = [&](T beta, bool fresh) {    // p = r (fresh) or r + beta p outside own rows
+        for (int i = tid; i < below + above; i += bd) {
+            const int at = i < below ? i : base + rows + (i - below);
+            const T ri = __ldcg(rg + e_lo + at);
+            p[at] = fresh ? ri : fma(beta, p[at], ri);
+        }
+    };
+    int it = 0, status = ST_OK;
+    T bb = 0;
+    for (int i = tid; i < rows; i += bd) {
+        const T bi = b[r_lo + i];
+        bb = fma(bi, bi, bb);
+        xs[i] = zero_x ? (T)0 : x[r_lo + i];
+    }
+    tm.total(bb, scratch, [&](T t) {
+        s_bnorm = sqrt((double)t);
+        s_target = a->tol * s_bnorm;
+    });
+    tm.total(residual(true), scratch, [&](T t) {
+        const double rn = sqrt((double)t);
+        s_rr = t;
+        s_first = rel_residual(rn, s_bnorm);
+        s_go = isfinite((double)t) && isfinite(s_bnorm) ? (rn <= s_target ? 0 : 1) : ST_NONFINITE;
+    });
+    const double target = s_target, t2 = target * target * (1.0 + 1e-12);
+    T rr = s_rr;
+    bool known = false;                            // rr is the true residual of the final x
+    if (s_go == ST_NONFINITE) status = ST_NONFINITE;
+    known = s_go == 0;
+    if (s_go == 1 && !tm.late) {
+        const int cap_it = a->max_iters;
+        fetch_halo((T)0, true);
+        for (;;) {
+            if (it >= cap_it) {
+                status = ST_NOT_CONVERGED;
+                break;
+            }
+            __syncthreads();
+            T acc = 0;
+            product(p, base, [&](int i, T ax, bool live) {
+                if (!live) return;
+                q[i] = ax;
+                acc = fma(p[base + i], ax, acc);
+            });
+            tm.total(acc, scratch, [&](T pq) {
+                s_alpha = rr / pq;
+                s_go = pq > 0 ? 1 : (isfinite((double)pq) ? ST_BREAKDOWN : ST_NONFINITE);
+            });
+            if (tm.late) break;
+            if (s_go != 1) {
+                status = s_go;
+                break;
+            }
+            const T alpha = s_alpha;
+            T rn = 0;
+            const int lane = tid & 31, warp = tid >> 5, nw = bd >> 5;
+            for (int s = warp; s < nsl; s += nw) {
+                const int i = s * 32 + lane;
+                if (i < rows) {
+                    const T ri = fma(-alpha, q[i], r[i]);
+                    r[i] = ri;
+                    if (L.r_in && edge(i)) rg[r_lo + i] = ri;
+                    rn = fma(ri, ri, rn);
+                }
+            }
+            tm.total(rn, scratch, [&](T t) {
+                s_beta = t / rr;
+                s_rr = t;
+                s_go = !isfinite((double)t) ? ST_NONFINITE
+                       : ((double)t <= t2 && sqrt((double)t) <= target) ? 0 : 1;
+            }, [&](int w0, int step) {             // x += alpha p while the total is on its way
+                for (int s = w0; s < nsl; s += step) {
+                    const int i = s * 32 + lane;
+                    if (i < rows) xs[i] = fma(alpha, p[base + i], xs[i]);
+                }
+            });
+            if (tm.late) break;
+            ++it;
+            if (s_go == ST_NONFINITE) {
+                status = ST_NONFINITE;
+                break;
+            }
+            if (s_go == 0) {                       // the true residual decides
+                if (L.x_in)
+                    for (int i = tid; i < rows; i += bd) x[r_lo + i] = xs[i];
+                tm.total((T)0, scratch, [&](T) {});
+                if (tm.late) break;
+                tm.total(residual(false), scratch, [&](T t) {
+                    s_rr = t;
+                    s_go = sqrt((double)t) <= target ? 0 : 1;
+                });
+                if (tm.late) break;
+                rr = s_rr;
+                if (s_go == 0) {
+                    known = true;
+                    break;
+                }
+                fetch_halo((T)0, true);
+                continue;
+            }
+            const T beta = s_beta;
+            rr = s_rr;
+            // The neighbours' rows of r are on their way while the own rows of
+            // the direction are formed.
+            constexpr int kAhead = 4;
+            T ahead[kAhead];
+            const bool few = below + above <= kAhead * bd;
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                const int i = tid + u * bd;
+                ahead[u] = few && i < below + above
+                               ? __ldcg(rg + e_lo + (i < below ? i : rows + i)) : (T)0;
+            }
+            for (int s = warp; s < nsl; s += nw) {
+                const int i = s * 32 + lane;
+                if (i < rows) p[base + i] = fma(beta, p[base + i], r[i]);
+            }
+            if (few) {
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    const int i = tid + u * bd;
+                    if (i < below + above) {
+                        const int at = i < below ? i : rows + i;
+                        p[at] = fma(beta, p[at], ahead[u]);
+                    }
+                }
+            } else {
+                fetch_halo(beta, false);
+            }
+        }
+    }
+    // The final iterate and its true residual (reported, and used by the
+    // refinement loop).
+    __syncthreads();
+    if (L.x_in)
+        for (int i = tid; i < rows; i += bd) x[r_lo + i] = xs[i];
+    if (!known && !tm.late) {
+        tm.total((T)0, scratch, [&](T) {});
+        if (!tm.late) tm.total(residual(false), scratch, [&](T t) { s_rr = t; });
+        rr = s_rr;
+    }
+    if (tm.rank() == 0 && tid == 0) {
+        ks->iters = it;
+        ks->status = tm.late ? ST_TIMEOUT : status;
+        ks->bnorm = s_bnorm;
+        ks->target = target;
+        ks->first_relres = s_first;
+        ks->beta = sqrt((double)rr);
+        ks->finished = 1;
+        ks->cycle_over = 1;
+    }
+}
+
+template <class Sys>
+__global__ void __launch_bounds__(kResThreads, 1)
+resident_cg_grid_kernel(const DevArgs* __restrict__ a, KState* ks, typename Sys::T* r,
+                        typename Sys::T* q, TeamSlot* slots, const ResLayout L) {
+    __shared__ int bad;
+    if (threadIdx.x == 0) bad = 0;
+    __syncthreads();
+    GridTeam<typename Sys::T> tm;
+    tm.slots = slots;
+    tm.count = reinterpret_cast<unsigned*>(slots + 2 * kTeamMax);
+    tm.bad = &bad;
+    resident_cg<Sys>(a, ks, r, q, tm, L);
+}
+
+template <class Sys>
+__global__ void __launch_bounds__(kResThreads, 1)
+resident_cg_cluster_kernel(const DevArgs* __restrict__ a, KState* ks, typename Sys::T* r,
+                           typename Sys::T* q, const ResLayout L) {
+    __shared__ typename Sys::T box[32];
+    ClusterTeam<typename Sys::T> tm;
+    tm.box = box;
+    tm.sync();                                     // every block has started before a remote store
+    resident_cg<Sys>(a, ks, r, q, tm, L);
+    tm.sync();                                     // no block leaves while another may store to it
+}
+
+// Launch of one CG solve by a resident team; false when none fits (the caller
+// takes the streaming kernels).  *launched: the launch's own status.
+template <class Sys>
+static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r, typename Sys::T* q,
+                               TeamSlot* slots, int n, int W, int reach, cudaStream_t st,
+                               cudaError_t* launched) {
+    using T = typename Sys::T;
+    int dev = 0, sms = 0, optin = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (sms > kTeamMax) sms = kTeamMax;
+    const size_t budget = (size_t)optin - 2048;    // the kernel's static shared memory
+    const int ns = (n + 31) / 32;
+    // A warp per slice; in FP64 eight warps fill the FP64 pipe and more only
+    // add to the reductions.
+    auto threads = [](int per) {
+        const int t = 32 * per, most = sizeof(T) == 8 ? kResThreads / 2 : kResThreads;
+        return t < 128 ? 128 : (t > most ? most : t);
+    };
+    ResLayout L;
+    if (n <= (sizeof(T) == 8 ? kClusterCgRows64 : kClusterCgRows32)) {
+        for (int c = 16; c >= 8; c >>= 1) {
+            if (!res_layout(n, W, reach, c, sizeof(T), budget, &L)) continue;
+            auto k = resident_cg_cluster_kernel<Sys>;
+            const size_t bytes = res_bytes(L, W, sizeof(T));
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess ||
+                (c > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+                cudaGetLastError();
+                continue;
+            }
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = c;
+            at[0].val.clusterDim.y = 1;
+            at[0].val.clusterDim.z = 1;
+            cfg.gridDim = dim3(c);
+            cfg.blockDim = dim3(threads(L.per));
+            cfg.dynamicSmemBytes = bytes;
+            cfg.stream = st;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            int fit = 0;
+            if (cudaOccupancyMaxActiveClusters(&fit, (const void*)k, &cfg) != cudaSuccess || fit < 1) {
+                cudaGetLastError();
+                continue;
+            }
+            *launched = cudaLaunchKernelEx(&cfg, k, a, ks, r, q, (const ResLayout)L);
+            return true;
+        }
+    }
+    // At least four slices per block: the reductions cost more than rows save.
+    int nblk = (ns + 3) / 4;
+    if (nblk > sms) nblk = sms;
+    if (!res_layout(n, W, reach, nblk, sizeof(T), budget, &L)) return false;
+    nblk = (ns + L.per - 1) / L.per;
+    auto k = resident_cg_grid_kernel<Sys>;
+    const size_t bytes = res_bytes(L, W, sizeof(T));
+    int per_sm = 0, coop = 0;
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    if (!coop ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads(L.per), bytes) != cudaSuccess ||
+        per_sm * sms < nblk) {
+        cudaGetLastError();
+        return false;
+    }
+    cudaMemsetAsync(slots, 0, kTeamSlotBytes, st);
+    void* args[] = {(void*)&a, (void*)&ks, (void*)&r, (void*)&q, (void*)&slots, (void*)&L};
+    *launched = cudaLaunchCooperativeKernel((const void*)k, dim3(nblk), dim3(threads(L.per)), args,
+                                            bytes, st);
+    return true;
+}
+
+}  // namespace sa

@@ -1,0 +1,87 @@
+"""Solves whose vectors stay on the chip (one cluster or one cooperative grid):
+block counts and row splits at their edges, reaches longer than a block's rows,
+more slots than the unrolled products take, and reaches too long for the chip,
+which take the streaming kernels.
+
+Matrices are symmetric with 1 <= a_ii <= 2 and off-diagonal row sums of at most
+a_ii / 2, so A has its eigenvalues in [1/2, 3] and condition number at most 6: a
+solution with relative residual 1e-12 lies within 6e-12 of the exact one."""
+import numpy as np
+import pytest
+import scipy.sparse as sp
+import scipy.sparse.linalg as spl
+import torch
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _spd(n, offsets, rng):
+    """Diagonally dominant symmetric matrix with entries at +-offsets."""
+    offs = [o for o in offsets if 0 < o < n]
+    bands = [rng.uniform(-1, 1, n - o) * 0.25 / max(len(offs), 1) for o in offs]
+    return sp.diags([rng.uniform(1, 2, n)] + bands + bands, [0] + offs + [-o for o in offs],
+                    format="csr")
+
+
+def _dev(A, b):
+    import paper_2309_02156_gb300 as sa
+    A.sort_indices()
+    t = lambda a, d: torch.from_numpy(np.ascontiguousarray(a, dtype=d)).to(DEV)
+    return sa.CSR(t(A.indptr, np.int32), t(A.indices, np.int32), t(A.data, np.float64)), \
+        t(b, np.float64)
+
+
+def _solve(A, b, tol, max_iters=2000, **kw):
+    import paper_2309_02156_gb300 as sa
+    n = A.shape[0]
+    seq = sa.Sequence(n, 2, 8, zeta=2, guess="zero", max_iters=max_iters, **kw)
+    Ad, bd = _dev(A, b)
+    x = torch.zeros(n, dtype=torch.float64, device=DEV)
+    infos = [seq.solve(Ad, bd, tol, x.zero_()) for _ in range(2)]
+    seq.close()
+    assert infos[0] == infos[1]           # the same solve again gives the same bits
+    return infos[0], x.cpu().numpy()
+
+
+# n: below a warp, ragged, the last cluster sizes and the first grid sizes of
+# both precisions (16,384 and 57,344 rows), several slices per warp
+@pytest.mark.parametrize("precision", ["f64", "mixed_krylov"])
+@pytest.mark.parametrize("n,offsets", [
+    (1, []), (31, [1, 7]), (33, [1, 7]), (700, [1, 300]), (4097, [1, 64]), (16384, [1, 128]),
+    (16385, [1, 128]), (57344, [1, 239]), (57345, [1, 239]), (131071, [1, 362]),
+    (5000, list(range(1, 5))), (5000, list(range(1, 12))), (20011, list(range(1, 12))),
+    (20000, [1, 9999]), (200003, [1, 100001])])
+def test_cg_matches_direct_solve(n, offsets, precision):
+    rng = np.random.default_rng(n + len(offsets))
+    A = _spd(n, offsets, rng)
+    b = rng.standard_normal(n)
+    info, x = _solve(A, b, 1e-12, krylov="cg", precision=precision)
+    assert info["status"] == 0 and info["final_relres"] <= 1e-12
+    assert np.linalg.norm(b - A @ x) <= 1.01e-12 * np.linalg.norm(b)
+    if n <= 60000:
+        ref = spl.spsolve(A.tocsc(), b) if n > 1 else b / A.toarray()[0]
+        assert np.linalg.norm(x - ref) <= 6e-12 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n", [500, 30000])
+def test_cg_status_codes(n):
+    """Iteration cap, breakdown and a NaN right-hand side on cluster and grid."""
+    import paper_2309_02156_gb300 as sa
+    rng = np.random.default_rng(n)
+    A = _spd(n, [1, 50], rng)
+    b = rng.standard_normal(n)
+    info, _ = _solve(A, b, 1e-12, max_iters=3, krylov="cg")
+    assert info["status"] == 1 and info["iters"] == 3
+    assert 1e-12 < info["final_relres"] < 1.0
+    for bad, code in ((-A, -4), (A, -5)):
+        seq = sa.Sequence(n, 2, 8, zeta=2, guess="zero", krylov="cg")
+        bb = b.copy()
+        if code == -5:
+            bb[n // 2] = np.nan
+        Ad, bd = _dev(bad.tocsr(), bb)
+        with pytest.raises(sa.SeqError) as e:
+            x = torch.zeros(n, dtype=torch.float64, device=DEV)
+            info = seq.solve(Ad, bd, 1e-10, x)
+        assert e.value.code == code
+        seq.close()
