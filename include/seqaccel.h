@@ -404,8 +404,11 @@ int seq_batch_set_schedule(seq_batch* batch, int32_t threads, int32_t blocks_per
  * sequence's rows; block sums are combined over the cluster through
  * distributed shared memory (same steps and arithmetic, rows split).  Fewer
  * sequences are in flight at once, so their working sets stay in L2 between
- * CG iterations.  ctas = 1 is the one-block schedule with `threads`.  The
- * autotuner also tries clusters of 4 and 8 (512 and 1024 threads). */
+ * CG iterations, or in the CTAs' shared memory where the patterns' rows share
+ * their column offsets and the CTAs have room.  ctas = 1 is the one-block
+ * schedule with `threads`.  The autotuner also tries clusters of 4 and 8 (512
+ * and 1024 threads).  In every schedule blocks whose patterns share their
+ * column offsets run at most 512 threads per SM. */
 int seq_batch_set_cluster(seq_batch* batch, int32_t ctas, int32_t threads, int32_t order_kind);
 
 /* The schedule in use: out[0] threads per block, out[1] blocks per SM,

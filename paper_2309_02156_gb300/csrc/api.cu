@@ -61,11 +61,10 @@ struct seq_ctx {
     size_t sell_cap = 0;             // values, columns and slot words allocated
     size_t col_cap = 0;
     size_t slot_cap = 0;
-    unsigned long long* d_stats = nullptr;   // totals of the matrix copy (slot_stats_kernel)
-    unsigned long long* h_stats = nullptr;   // pinned
+    SlotStats* d_stats = nullptr;    // totals of the matrix (launch_slot_stats)
+    SlotStats* h_stats = nullptr;    // pinned
     bool sell_ok = false;            // a copy of this solve's matrix exists
-    int slot_w = 0;                  // slots per slice (0: not in slot form)
-    int slot_reach = 0;              // largest |column - row| (slot form)
+    SlotPlan plan = {};              // slot form of this solve's matrix (W = 0: none)
     TeamSlot* team = nullptr;        // posted partials of the resident CG's grid team
     double copy_bytes = 0.0;         // bytes of the copy that a product reads
     int sell_w = 0;                  // uniform SELL slice width (0: slices differ)
@@ -162,10 +161,11 @@ int set_args(seq_ctx* ctx, const seq_csr* A, const double* b, double* x, double 
     h->x = x;
     h->d = ctx->d;
     h->rhs32 = ctx->rhs32;
-    h->sell_off = ctx->sell_ok && !ctx->slot_w ? ctx->sell_off : nullptr;
-    h->slot = ctx->sell_ok && ctx->slot_w ? ctx->slot : nullptr;
-    h->slot_w = ctx->sell_ok ? ctx->slot_w : 0;
-    h->slot_reach = ctx->slot_reach;
+    h->sell_off = ctx->sell_ok && !ctx->plan.W ? ctx->sell_off : nullptr;
+    h->slot = ctx->sell_ok && ctx->plan.W ? ctx->slot : nullptr;
+    h->slot_w = ctx->sell_ok ? ctx->plan.W : 0;
+    h->slot_reach = ctx->plan.reach;
+    h->slot_off = ctx->plan.list;
     h->sell_col = ctx->sell_ok ? ctx->sell_col : nullptr;
     h->sell_val = ctx->sell_ok ? ctx->sell_val : nullptr;
     h->sell_w = ctx->sell_ok ? ctx->sell_w : 0;
@@ -228,33 +228,32 @@ int reserve_copy(seq_ctx* ctx, size_t entries, bool columns, size_t slots) {
 // padding would more than double the storage.
 int build_sell(seq_ctx* ctx, const seq_csr* A) {
     ctx->sell_ok = false;
-    ctx->slot_w = 0;
+    ctx->plan = SlotPlan{};
     const int n = A->n, ns = (n + 31) / 32;
     launch_slot_stats(A->rowptr, A->colind, n, A->nnz, ctx->sell_width, ctx->d_stats, ctx->stream);
     ctx->launches += 1;
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(ctx->h_stats, ctx->d_stats, 4 * sizeof(unsigned long long),
-                       cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(ctx->h_stats, ctx->d_stats, sizeof(SlotStats), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    long long total = (long long)ctx->h_stats[0];
-    const long long wmax = (long long)ctx->h_stats[1], slots = (long long)ctx->h_stats[2];
+    long long total = (long long)ctx->h_stats->total[0];
+    const long long wmax = (long long)ctx->h_stats->total[1];
     ctx->sell_w = 0;
     if (total <= 0 || total >= 0x7fffffffLL || total > 2LL * A->nnz + 64LL * ns) return SEQ_OK;
     const size_t el = ctx->mixed ? sizeof(float) : sizeof(double);
     const float* v32 = A->values_f32 ? A->values_f32 : ctx->val32;
-    if (slots > 0 && slots <= kMaxSlots && 32LL * ns * slots <= total + total / 4 &&
-        32LL * ns * slots < 0x7fffffffLL) {
-        total = 32LL * ns * slots;
-        int rc = reserve_copy(ctx, (size_t)total, false, (size_t)ns * slots);
+    const SlotPlan plan = plan_slots(*ctx->h_stats, n);
+    if (plan.W) {
+        total = 32LL * ns * plan.W;
+        int rc = reserve_copy(ctx, (size_t)total, false, (size_t)ns * plan.W);
         if (rc) return rc;
-        ctx->slot_w = (int)slots;
-        ctx->slot_reach = (int)ctx->h_stats[3];
-        ctx->copy_bytes = (double)el * (double)total + 8.0 * (double)ns * (double)slots;
+        ctx->plan = plan;
+        ctx->copy_bytes = (double)el * (double)total +
+                          (plan.list.count ? 0.0 : 8.0 * (double)ns * plan.W);
         if (ctx->mixed)
-            launch_slot_fill_f32(A->rowptr, A->colind, v32, n, A->nnz, ctx->slot_w, ctx->slot,
+            launch_slot_fill_f32(A->rowptr, A->colind, v32, n, A->nnz, plan, ctx->slot,
                                  (float*)ctx->sell_val, ctx->stream);
         else
-            launch_slot_fill_f64(A->rowptr, A->colind, A->values, n, A->nnz, ctx->slot_w, ctx->slot,
+            launch_slot_fill_f64(A->rowptr, A->colind, A->values, n, A->nnz, plan, ctx->slot,
                                  (double*)ctx->sell_val, ctx->stream);
         ctx->launches += 1;
     } else {
@@ -518,13 +517,13 @@ int run_cg(seq_ctx* ctx, bool f32) {
     KState* ks = f32 ? ctx->ks_in : ctx->ks;
     const DevArgs* args = f32 ? ctx->d_args_in : ctx->d_args;
     const int n = ctx->cfg.n;
-    if (ctx->sell_ok && ctx->slot_w) {
+    if (ctx->sell_ok && ctx->plan.W) {
         cudaError_t e = cudaSuccess;
         const bool taken =
             f32 ? launch_resident_cg_f32(args, ks, (float*)ctx->r, (float*)ctx->q, ctx->team, n,
-                                         ctx->slot_w, ctx->slot_reach, ctx->stream, &e)
+                                         ctx->plan.W, ctx->plan.reach, ctx->stream, &e)
                 : launch_resident_cg_f64(args, ks, (double*)ctx->r, (double*)ctx->q, ctx->team, n,
-                                         ctx->slot_w, ctx->slot_reach, ctx->stream, &e);
+                                         ctx->plan.W, ctx->plan.reach, ctx->stream, &e);
         if (taken) {
             ctx->launches += 1;
             CK(e);
@@ -623,8 +622,8 @@ int seq_create(const seq_config* cfg, void* cuda_stream, seq_ctx** out) {
         ok = ok && cudaMalloc(&ctx->sell_width, sizeof(int) * (size_t)ns) == cudaSuccess;
         ok = ok && cudaMalloc(&ctx->sell_off, sizeof(int) * (size_t)(ns + 2)) == cudaSuccess;
     }
-    ok = ok && cudaMalloc(&ctx->d_stats, 4 * sizeof(unsigned long long)) == cudaSuccess;
-    ok = ok && cudaMallocHost(&ctx->h_stats, 4 * sizeof(unsigned long long)) == cudaSuccess;
+    ok = ok && cudaMalloc(&ctx->d_stats, sizeof(SlotStats)) == cudaSuccess;
+    ok = ok && cudaMallocHost(&ctx->h_stats, sizeof(SlotStats)) == cudaSuccess;
     {
         const int in = 4 * M + s, stride = in + M + M * M + 1;
         ok = ok && cudaMalloc(&ctx->yring, sizeof(double) * 4 * kMaxM) == cudaSuccess;

@@ -5,8 +5,8 @@
 // by default, the order the autotuner picked otherwise) and runs the whole
 // step of one sequence with block barriers only -- there is no grid-wide
 // wait anywhere, so blocks never spin on one another:
-//   1. guess (Algorithm 1): W = S [A X | b] accumulated in shared
-//      memory (the sparse-sign S generated on the fly from its counters),
+//   1. guess (Algorithm 1): W = S [A X | b] accumulated in shared memory in
+//      exact fixed point (the sparse-sign S generated from its counters),
 //      the column-scaled pivoted Householder least squares in shared memory,
 //      x0 = X y with FP64 accumulation;
 //   2. FP64 iterative refinement around FP32 CG (the solve): r = b - A x in FP64,
@@ -26,13 +26,15 @@
 #include "../../include/seqaccel.h"
 #include "common.cuh"
 #include "internal.h"
+#include "resident.cuh"
+#include "sketch_tile.cuh"
 
 namespace sa {
 namespace {
 
 constexpr int kBatchMaxM = 16;
 constexpr int kBatchMaxS = 64;
-constexpr int kSketchWarps = 8;           // warps with a private copy of W
+constexpr int kSketchTeams = 4;           // teams of four warps that sketch a sequence
 constexpr double kTheta = 0.5;
 constexpr int kOk = 0;
 
@@ -47,6 +49,9 @@ struct BatchSeq {
     const int* soff;                       // SELL-32 copy of the pattern for the FP32 CG:
     const int* scol;                       //   slice offsets, padded column indices,
     float* sval;                           //   values refreshed every step (FP32)
+    const int2* slot;                      // slot form of the pattern (NULL: SELL-32 above); sval
+    int slot_w, reach;                     //   then holds the slots' values; max |column - row|
+    OffsetList list;                       //   the offsets of every slice (count 0: they differ)
     float *r, *p, *q, *d;                  // FP32 CG vectors (16-byte aligned, stride nv)
     // per step
     const double* val;
@@ -94,84 +99,54 @@ __device__ __forceinline__ Acc row_dot(const int* __restrict__ rowptr, const int
     return acc;
 }
 
-__device__ void sketch_column_b(int j, int s, int zeta, uint64_t seed, uint16_t* out) {
-    int rows[kMaxZeta];
-    int cnt = 0;
-    for (int c = 0; c < 256 && cnt < zeta; ++c) {
-        const uint64_t h = mix64(seed + ((uint64_t)j * 256ull + (uint64_t)(c + 1)) *
-                                            0x9E3779B97F4A7C15ull);
-        const int q = (int)(((h >> 32) * (uint64_t)s) >> 32);
-        bool dup = false;
-        for (int k = 0; k < cnt; ++k) dup |= rows[k] == q;
-        if (!dup) {
-            rows[cnt] = q;
-            out[cnt] = (uint16_t)(q | ((h & 1ull) ? 0x8000 : 0));
-            ++cnt;
-        }
-    }
-    for (int q = 0; cnt < zeta && q < s; ++q) {
-        bool used = false;
-        for (int k = 0; k < cnt; ++k) used |= rows[k] == q;
-        if (!used) {
-            rows[cnt] = q;
-            out[cnt] = (uint16_t)q;
-            ++cnt;
-        }
-    }
+// Doubles of the sketch's workspace: the teams' regions and FP64 accumulators.
+__host__ __device__ inline size_t sketch_ws_doubles(int s, int ncol) {
+    return kSketchTeams * (sketch_team_bytes(s, ncol) / 8 + (size_t)s * ncol);
 }
 
-// The sketched block W (s x (M+1), physical history slots, b last) of rows
-// [r_lo, r_hi) of one sequence, summed into Wsum (shared).  Warps
-// 0..kSketchWarps-1 keep private copies; rows are taken in batches of 32 per
-// warp, lane l building the sketch column of row base + l; the copies are
-// added in warp order.
-__device__ void block_sketch(const BatchSeq& q, double* Wpriv, uint16_t* sks, double* Wsum,
-                             int& bad, int r_lo, int r_hi) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// The sketched block W (s x (M+1), physical history slots, b last) of the
+// sequence's slices [s_lo, s_hi), summed into Wsum (shared).  The tiles, the
+// products spread over all lanes and the exact fixed-point additions are those
+// of the single-sequence kernel; a team's integers go to its FP64 accumulator
+// every kSkMaxTiles tiles, and the teams are added in order.  FP64 additions per
+// row and sketch entry, as before, held the FP64 pipe for 512 of the 832 cycles
+// a row took: 8 sequences of 122,500 rows in clusters of 8, guess 3.5 -> 1.8 ms.
+__device__ void block_sketch(const BatchSeq& q, double* ws, double* Wsum, int& bad, int s_lo,
+                             int s_hi) {
+    __shared__ int zk[kMaxZeta * (kBatchMaxM + 1)];
     const int ncol = q.M + 1, wsz = q.s * ncol;
-    const int nsw = min(kSketchWarps, (int)(blockDim.x >> 5));
-    for (int i = threadIdx.x; i < nsw * wsz; i += blockDim.x) Wpriv[i] = 0.0;
+    const int nt = min(kSketchTeams, (int)blockDim.x / kSkTeamThreads);
+    const int team = threadIdx.x / kSkTeamThreads, tt = threadIdx.x % kSkTeamThreads;
+    const size_t tb = sketch_team_bytes(q.s, ncol) / 8;
+    double* acc = ws + kSketchTeams * tb;
+    sketch_pairs(zk, q.zeta, ncol);
+    for (int i = threadIdx.x; i < nt * wsz; i += blockDim.x) acc[i] = 0.0;
     __syncthreads();
-    if (warp < nsw) {
-        double* Ww = Wpriv + warp * wsz;
-        uint16_t* sk = sks + warp * 32 * kMaxZeta;
-        for (int base = r_lo + warp * 32; base < r_hi; base += nsw * 32) {
-            if (base + lane < r_hi) sketch_column_b(base + lane, q.s, q.zeta, q.seed, sk + lane * kMaxZeta);
-            __syncwarp();
-            const int cnt = min(32, r_hi - base);
-            for (int u = 0; u < cnt; ++u) {
-                const int r = base + u;
-                double y = 0.0;
-                if (lane < q.M) {
-                    const int rs = max(0, min(q.rowptr[r], q.nnz));
-                    const int re = max(rs, min(q.rowptr[r + 1], q.nnz));
-                    for (int e = rs; e < re; ++e) {
-                        const int c = q.colind[e];
-                        if ((unsigned)c < (unsigned)q.n)
-                            y = fma(q.val[e], q.X[(size_t)c * q.ldx + lane], y);
-                        else
-                            bad = 1;
-                    }
-                } else if (lane == q.M) {
-                    y = q.b[r];
-                }
-                if (lane < ncol) {
-                    for (int k = 0; k < q.zeta; ++k) {
-                        const unsigned e = sk[u * kMaxZeta + k];
-                        double* dst = Ww + (e & 0x7fff) * ncol + lane;
-                        *dst = (e & 0x8000) ? *dst - y : *dst + y;
-                    }
-                }
+    if (team < nt) {
+        const SketchTeam<double> tm(reinterpret_cast<unsigned char*>(ws + team * tb), q.s, ncol, tt >> 5);
+        double* mine = acc + (size_t)team * wsz;
+        tm.clear(wsz, ncol, tt);
+        team_sync(team);
+        for (int t0 = s_lo + team; t0 < s_hi; t0 += kSkMaxTiles * nt) {
+            sketch_team_tiles<double, double>(tm, team, zk, q.rowptr, q.colind, q.val, q.X, q.ldx,
+                                              q.b, q.n, q.nnz, q.M, q.s, q.zeta, q.seed, t0, nt,
+                                              min(s_hi, t0 + kSkMaxTiles * nt), bad);
+            for (int i = tt; i < wsz; i += kSkTeamThreads) {
+                const int k = i % ncol, st = tm.stk[k];
+                if (st & 2) mine[i] = __longlong_as_double(0x7ff8000000000000ll);
+                else if (st & 1) mine[i] += scalbn((double)tm.Wi[i], -tm.Fk[k]);
             }
-            __syncwarp();
+            team_sync(team);
+            tm.clear(wsz, ncol, tt);
+            team_sync(team);
         }
     }
     __syncthreads();
     const double inv = 1.0 / sqrt((double)q.zeta);
     for (int i = threadIdx.x; i < wsz; i += blockDim.x) {
-        double acc = Wpriv[i];
-        for (int w = 1; w < nsw; ++w) acc += Wpriv[w * wsz + i];
-        Wsum[i] = acc * inv;
+        double t = acc[i];
+        for (int w = 1; w < nt; ++w) t += acc[(size_t)w * wsz + i];
+        Wsum[i] = t * inv;
     }
     __syncthreads();
 }
@@ -406,6 +381,91 @@ __device__ __forceinline__ void bsell_spmv(const BatchSeq& q, const float* __res
     if (flag) atomicOr(bad, 1);
 }
 
+// The same product for a pattern in slot form.  Slices with common offsets read
+// no index at all (a row without an entry at an offset multiplies its stored
+// zero); others take one (offset, row mask) word per slot.
+template <typename Epi>
+__device__ __forceinline__ void bslot_spmv(const BatchSeq& q, const float* __restrict__ x, int nw,
+                                           Epi& epi, int s_lo, int s_hi, int r_lo, int r_hi) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = q.n, W = q.slot_w;
+    if (q.list.count > 0 && W <= kBW) {
+        int off[kBW];
+#pragma unroll
+        for (int k = 0; k < kBW; ++k) off[k] = k < W ? q.list.off[k] : 0;
+        const float* __restrict__ val = q.sval;
+        for (int sl0 = s_lo + warp; sl0 < s_hi; sl0 += 2 * nw) {
+            float v[2][kBW], xv[2][kBW];
+            typename Epi::Pre pre[2];
+#pragma unroll
+            for (int g = 0; g < 2; ++g)
+#pragma unroll
+                for (int k = 0; k < kBW; ++k)
+                    v[g][k] = sl0 + g * nw < s_hi && k < W
+                                  ? val[((sl0 + g * nw) * W + k) * 32 + lane] : 0.f;
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                const int r = (sl0 + g * nw) * 32 + lane;
+                const bool live = sl0 + g * nw < s_hi && r < n;
+                if (live) pre[g] = epi.pre(r);
+#pragma unroll
+                for (int k = 0; k < kBW; ++k) {
+                    const int c = r + off[k];
+                    xv[g][k] = live && (unsigned)c < (unsigned)n
+                                   ? (c >= r_lo && c < r_hi ? x[c] : __ldcg(x + c)) : 0.f;
+                }
+            }
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                const int r = (sl0 + g * nw) * 32 + lane;
+                float a = 0.f;
+#pragma unroll
+                for (int k = 0; k < kBW; ++k)
+                    if (k < W) a = fmaf(v[g][k], xv[g][k], a);
+                if (sl0 + g * nw < s_hi && r < n) epi(r, a, pre[g]);
+            }
+        }
+        return;
+    }
+    for (int sl = s_lo + warp; sl < s_hi; sl += nw) {
+        const int r = sl * 32 + lane;
+        float a = 0.f;
+#pragma unroll 4
+        for (int k = 0; k < W; ++k) {
+            const int2 m = __ldg(q.slot + sl * W + k);
+            if ((m.y >> lane) & 1) {
+                const int c = r + m.x;
+                a = fmaf(q.sval[(sl * W + k) * 32 + lane],
+                         c >= r_lo && c < r_hi ? x[c] : __ldcg(x + c), a);
+            }
+        }
+        if (r < n) epi(r, a, epi.pre(r));
+    }
+}
+
+template <typename Epi>
+__device__ __forceinline__ void batch_product(const BatchSeq& q, const float* x, int nw, int* bad,
+                                              Epi& epi, int s_lo, int s_hi, int r_lo, int r_hi) {
+    if (q.slot) bslot_spmv(q, x, nw, epi, s_lo, s_hi, r_lo, r_hi);
+    else bsell_spmv(q, x, nw, bad, epi, s_lo, s_hi, r_lo, r_hi);
+}
+
+// This step's values (FP32) into the copy of the pattern, rows [r_lo, r_hi).
+__device__ __forceinline__ void refresh_values(const BatchSeq& q, int r_lo, int r_hi) {
+    for (int i = r_lo + threadIdx.x; i < r_hi; i += blockDim.x) {
+        int e = q.rowptr[i];
+        const int e1 = q.rowptr[i + 1], lane = i & 31;
+        if (q.slot) {
+            const int2* m = q.slot + (i >> 5) * q.slot_w;
+            float* dst = q.sval + (i >> 5) * q.slot_w * 32 + lane;
+            for (int k = 0; k < q.slot_w; ++k)
+                if ((m[k].y >> lane) & 1) dst[k * 32] = (float)q.val[e++];
+        } else {
+            float* dst = q.sval + q.soff[i >> 5] + lane;
+            for (int k = 0; e < e1; ++e, ++k) dst[k * 32] = (float)q.val[e];
+        }
+    }
+}
+
 struct CgProductEpi {
     float* qv;
     const float* p;
@@ -418,8 +478,8 @@ struct CgProductEpi {
     }
 };
 
-__device__ int block_cg32(const BatchSeq& q, double itol, int max_iters, float* sred, float* stage,
-                          int* sbad, int& status) {
+__device__ int block_cg32(const BatchSeq& q, double itol, int max_iters, float* sred, int* sbad,
+                          int& status) {
     // Vector phases use 16-byte loads over the first 4 floor(n / 4) entries
     // (the vectors are 16-byte aligned), then the ragged tail.
     const int n4 = q.n >> 2;
@@ -427,7 +487,6 @@ __device__ int block_cg32(const BatchSeq& q, double itol, int max_iters, float* 
     float4* p4 = reinterpret_cast<float4*>(q.p);
     float4* q4 = reinterpret_cast<float4*>(q.q);
     float4* d4 = reinterpret_cast<float4*>(q.d);
-    (void)stage;
     const int n = q.n, tid = threadIdx.x, bd = blockDim.x;
     const int nw = bd >> 5;
     float rr_l = 0.f;
@@ -461,7 +520,7 @@ __device__ int block_cg32(const BatchSeq& q, double itol, int max_iters, float* 
         }
         __syncthreads();
         CgProductEpi epi{q.q, q.p, 0.f};
-        bsell_spmv(q, q.p, nw, sbad, epi, 0, (n + 31) >> 5, 0, n);
+        batch_product(q, q.p, nw, sbad, epi, 0, (n + 31) >> 5, 0, n);
         const float pq = btotal(epi.acc, sred);
         if (!(pq > 0.f)) {
             status = isfinite(pq) ? -4 : -5;
@@ -656,7 +715,7 @@ __device__ int cluster_cg32(const BatchSeq& q, double itol, int max_iters, float
         }
         __syncthreads();
         CgProductEpi epi{q.q, q.p, 0.f};
-        bsell_spmv(q, q.p, nw, sbad, epi, s_lo, s_hi, r_lo, r_hi);
+        batch_product(q, q.p, nw, sbad, epi, s_lo, s_hi, r_lo, r_hi);
         const float pq = cl_total(btotal(epi.acc, sred), red.fslot, red.fbc, red.fpar);
         if (!(pq > 0.f)) {
             status = isfinite(pq) ? -4 : -5;
@@ -708,12 +767,75 @@ __device__ int cluster_cg32(const BatchSeq& q, double itol, int max_iters, float
     return it;
 }
 
+// The FP32 CG of block_cg32 with its vectors in shared memory (patterns in slot
+// form whose direction and halo fit; resident.cuh): each CTA of the team keeps
+// the direction p of its rows and of the rows within reach on both sides, then
+// as many of r, q, d and the matrix values as fit.  Two team reductions per
+// iteration and no other wait: neighbours' rows of r come through q.r, and
+// every CTA forms the halo's direction itself.  x += d at the end.  Bound by L2
+// latency and bandwidth for the values that do not fit (20 bytes a row), then
+// by the instructions of the product: 64 sequences (clusters of 8) 62.5 -> 26.6
+// ms a step, 512 (clusters of 4) 405 -> 225 ms, guess included.
+__device__ __noinline__ int resident_cg32(const BatchSeq& q, double itol, int max_iters,
+                                          ClusterTeam<float>& team, float* scratch,
+                                          const ResLayout& L, int s_lo, int s_hi, int& status) {
+    extern __shared__ __align__(16) double smem[];
+    __shared__ float s_val;
+    ClusterTeam<float> tm = team;
+    __shared__ ResBlock<float> B;
+    float* const p = reinterpret_cast<float*>(smem);
+    __syncthreads();                           // the caller's use of the shared memory is over
+    B.setup(p, L, q.n, s_lo, s_hi, q.slot_w, q.reach, q.list, q.slot, q.sval, q.r, q.q, q.d);
+    const int tid = threadIdx.x, bd = blockDim.x;
+    float acc = 0.f;
+    for (int i = tid; i < B.rows; i += bd) {
+        const float ri = B.rg[B.lo + i];
+        B.r[i] = ri;
+        p[B.pad + i] = ri;
+        B.x[i] = 0.f;
+        acc = fmaf(ri, ri, acc);
+    }
+    B.halo_fresh(p);
+    tm.total(acc, scratch, [&](float t) { s_val = t; });
+    float rr = s_val;
+    const float target2 = (float)(itol * itol * (double)rr);
+    int it = 0;
+    status = kOk;
+    while (rr > 0.f && rr > target2) {
+        if (it >= max_iters) {
+            status = 1;
+            break;
+        }
+        __syncthreads();
+        tm.total(B.template product<4>(p), scratch, [&](float t) { s_val = t; });
+        const float pq = s_val;
+        if (!(pq > 0.f)) {
+            status = isfinite(pq) ? -4 : -5;
+            break;
+        }
+        const float alpha = rr / pq;
+        tm.total(B.update_r(alpha), scratch, [&](float t) { s_val = t; },
+                 [&](int w0, int step) { B.update_x(p, alpha, w0, step); });
+        const float rr_new = s_val;
+        ++it;
+        const float beta = rr_new / rr;
+        rr = rr_new;
+        B.direction(p, beta);
+    }
+    __syncthreads();
+    if (status >= 0)
+        for (int i = tid; i < B.rows; i += bd) q.x[B.lo + i] += (double)B.x[i];
+    team = tm;
+    __syncthreads();
+    return it;
+}
+
 // Shared-memory bytes of one block for sequences with at most s rows of
 // sketch and M history columns.
 size_t batch_smem_bytes(int s, int M) {
     const int ncol = M + 1, wsz = s * ncol;
-    size_t d = (size_t)kSketchWarps * wsz + wsz + (2 * s * M + 3 * s + 5 * M) + kBatchMaxM;
-    const size_t guess = d * sizeof(double) + (size_t)kSketchWarps * 32 * kMaxZeta * sizeof(uint16_t);
+    const size_t d = sketch_ws_doubles(s, ncol) + wsz + (2 * s * M + 3 * s + 5 * M) + kBatchMaxM;
+    const size_t guess = d * sizeof(double);
     const size_t stage = sizeof(double) * 32 * (size_t)kTileChunks * 32;   // up to 32 warps
     return guess > stage ? guess : stage;
 }
@@ -723,11 +845,16 @@ size_t batch_smem_bytes(int s, int M) {
 // end (no inter-block waiting).  MAXT: the largest block size the
 // instantiation is launched with at one block per SM, which sets its register
 // budget (65,536 / MAXT, at most 255): 1024 -> 64, 512 -> 128, 256 -> 255.
-template <int MAXT>
+// RES: sequences that fit take the resident CG (a launch whose sequences do not
+// fit is a kernel without it, which needs fewer registers).
+template <int MAXT, bool RES>
 __global__ void __launch_bounds__(MAXT, 1)
 batched_step_kernel(BatchSeq* seqs, const int* __restrict__ order, int count, int* queue,
-                    const BatchParams* __restrict__ prm) {
-    extern __shared__ double smem[];
+                    const BatchParams* __restrict__ prm, int smem_bytes) {
+    extern __shared__ __align__(16) double smem[];
+    __shared__ float box[32];
+    ClusterTeam<float> team;
+    team.box = box;
     __shared__ int sidx;
     __shared__ double dred[32];
     __shared__ float fred[32];
@@ -749,15 +876,13 @@ batched_step_kernel(BatchSeq* seqs, const int* __restrict__ order, int count, in
         int bad = 0, rank = 0;
         double rho = 0.0;
         // 1. guess
-        double* Wpriv = smem;
-        double* Wsum = Wpriv + kSketchWarps * s * (M + 1);
+        double* Wsum = smem + sketch_ws_doubles(s, M + 1);
         double* ws = Wsum + s * (M + 1);
         double* yphys = ws + (2 * s * M + 3 * s + 5 * M);
-        uint16_t* sks = reinterpret_cast<uint16_t*>(yphys + kBatchMaxM);
         if (m == 0) {
             for (int i = tid; i < n; i += bd) q.x[i] = 0.0;
         } else {
-            block_sketch(q, Wpriv, sks, Wsum, bad, 0, n);
+            block_sketch(q, smem, Wsum, bad, 0, (n + 31) >> 5);
             block_lsq(Wsum, s, M, m, (q.pushes - m) % M, 1e-12, ws, yphys, &rank, &rho);
             for (int i = tid; i < n; i += bd) {
                 const double* row = q.X + (size_t)i * q.ldx;
@@ -766,17 +891,13 @@ batched_step_kernel(BatchSeq* seqs, const int* __restrict__ order, int count, in
                 q.x[i] = acc;
             }
         }
-        // This step's values into the SELL copy (FP32): entry k of row i goes
-        // to soff[i / 32] + 32 k + i % 32.
-        for (int i = tid; i < n; i += bd) {
-            const int e0 = q.rowptr[i], e1 = q.rowptr[i + 1];
-            float* dst = q.sval + q.soff[i >> 5] + (i & 31);
-            for (int e = e0; e < e1; ++e) dst[(e - e0) * 32] = (float)q.val[e];
-        }
+        refresh_values(q, 0, n);
         __syncthreads();
         // Warp-tile staging for the products (aliases the guess workspace).
         double* stage_d = smem;
-        float* stage_f = reinterpret_cast<float*>(smem);
+        ResLayout L;
+        const bool resident =
+            RES && q.slot && res_layout(n, q.slot_w, q.reach, 1, 4, smem_bytes, &L);
         const int lane = tid & 31, warp = tid >> 5, nw = bd >> 5;
         // 2. FP64 refinement around FP32 CG
         double bb_l = 0.0;
@@ -810,13 +931,18 @@ batched_step_kernel(BatchSeq* seqs, const int* __restrict__ order, int count, in
             }
             const double itol = fmax(P.inner_tol, kTheta * target / rn);
             int st = kOk;
-            total += block_cg32(q, itol, P.max_iters - total, fred, stage_f, &sbad, st);
+            if (RES && resident)
+                total += resident_cg32(q, itol, P.max_iters - total, team,
+                                                             fred, L, 0, (n + 31) >> 5, st);
+            else
+                total += block_cg32(q, itol, P.max_iters - total, fred, &sbad, st);
             ++nref;
             if (st < 0) {
                 status = st;
                 break;
             }
-            for (int i = tid; i < n; i += bd) q.x[i] += (double)q.d[i];
+            if (!resident)
+                for (int i = tid; i < n; i += bd) q.x[i] += (double)q.d[i];
             __syncthreads();
         }
         // 3. push
@@ -846,9 +972,8 @@ batched_step_kernel(BatchSeq* seqs, const int* __restrict__ order, int count, in
 size_t batch_cluster_smem_bytes(int s, int M) {
     const size_t base = batch_smem_bytes(s, M);
     const int wsz = s * (M + 1);
-    const size_t d = (size_t)kSketchWarps * wsz + wsz + (2 * s * M + 3 * s + 5 * M) + kBatchMaxM;
-    const size_t guess = d * sizeof(double) + (size_t)kSketchWarps * 32 * kMaxZeta * sizeof(uint16_t);
-    const size_t need = guess + (size_t)wsz * sizeof(double);
+    const size_t d = sketch_ws_doubles(s, M + 1) + wsz + (2 * s * M + 3 * s + 5 * M) + kBatchMaxM;
+    const size_t need = (d + (size_t)wsz) * sizeof(double);
     return base > need ? base : need;
 }
 
@@ -856,11 +981,14 @@ size_t batch_cluster_smem_bytes(int s, int M) {
 // cl_total above).  The steps and their arithmetic are those of
 // batched_step_kernel; rows are split over the cluster's CTAs and block
 // totals (the sketch W, norms, CG dot products) are summed over the cluster.
-template <int MAXT>
+template <int MAXT, bool RES>
 __global__ void __launch_bounds__(MAXT, 1)
 batched_cluster_kernel(BatchSeq* seqs, const int* __restrict__ order, int count, int* queue,
-                       const BatchParams* __restrict__ prm) {
-    extern __shared__ double smem[];
+                       const BatchParams* __restrict__ prm, int smem_bytes) {
+    extern __shared__ __align__(16) double smem[];
+    __shared__ float box[32];
+    ClusterTeam<float> team;
+    team.box = box;
     __shared__ int s_take, s_idx;
     __shared__ double dred[32];
     __shared__ float fred[32];
@@ -892,16 +1020,14 @@ batched_cluster_kernel(BatchSeq* seqs, const int* __restrict__ order, int count,
         double rho = 0.0;
         // 1. guess
         const int ncol = M + 1, wsz = s * ncol;
-        double* Wpriv = smem;
-        double* Wsum = Wpriv + kSketchWarps * wsz;
+        double* Wsum = smem + sketch_ws_doubles(s, ncol);
         double* ws = Wsum + wsz;
         double* yphys = ws + (2 * s * M + 3 * s + 5 * M);
-        uint16_t* sks = reinterpret_cast<uint16_t*>(yphys + kBatchMaxM);
-        double* Wtot = reinterpret_cast<double*>(sks + kSketchWarps * 32 * kMaxZeta);
+        double* Wtot = yphys + kBatchMaxM;
         if (m == 0) {
             for (int i = r_lo + tid; i < r_hi; i += bd) q.x[i] = 0.0;
         } else {
-            block_sketch(q, Wpriv, sks, Wsum, bad, r_lo, r_hi);
+            block_sketch(q, smem, Wsum, bad, s_lo, s_hi);
             cl_sync();
             for (int i = tid; i < wsz; i += bd) {
                 double t = 0.0;
@@ -917,14 +1043,12 @@ batched_cluster_kernel(BatchSeq* seqs, const int* __restrict__ order, int count,
                 q.x[i] = acc;
             }
         }
-        // This step's values into the SELL copy (FP32), own rows.
-        for (int i = r_lo + tid; i < r_hi; i += bd) {
-            const int e0 = q.rowptr[i], e1 = q.rowptr[i + 1];
-            float* dst = q.sval + q.soff[i >> 5] + (i & 31);
-            for (int e = e0; e < e1; ++e) dst[(e - e0) * 32] = (float)q.val[e];
-        }
+        refresh_values(q, r_lo, r_hi);
         __syncthreads();
         double* stage_d = smem;
+        ResLayout L;
+        const bool resident =
+            RES && q.slot && res_layout(n, q.slot_w, q.reach, (int)nr, 4, smem_bytes, &L);
         const int lane = tid & 31, warp = tid >> 5, nw = bd >> 5;
         // 2. FP64 refinement around FP32 CG (the x of other CTAs is complete
         // after the cluster total below)
@@ -960,14 +1084,19 @@ batched_cluster_kernel(BatchSeq* seqs, const int* __restrict__ order, int count,
             }
             const double itol = fmax(P.inner_tol, kTheta * target / rn);
             int st = kOk;
-            total += cluster_cg32(q, itol, P.max_iters - total, fred, &sbad, s_lo, s_hi, r_lo, r_hi,
-                                  red, st);
+            if (RES && resident)
+                total += resident_cg32(q, itol, P.max_iters - total, team,
+                                                             fred, L, s_lo, s_hi, st);
+            else
+                total += cluster_cg32(q, itol, P.max_iters - total, fred, &sbad, s_lo, s_hi, r_lo,
+                                      r_hi, red, st);
             ++nref;
             if (st < 0) {
                 status = st;
                 break;
             }
-            for (int i = r_lo + tid; i < r_hi; i += bd) q.x[i] += (double)q.d[i];
+            if (!resident)
+                for (int i = r_lo + tid; i < r_hi; i += bd) q.x[i] += (double)q.d[i];
             cl_sync();   // x complete before the next residual gathers it
         }
         // 3. push (own rows)
@@ -996,16 +1125,16 @@ batched_cluster_kernel(BatchSeq* seqs, const int* __restrict__ order, int count,
 
 // The instantiation whose register budget fits `threads` x `blocks_per_sm`
 // threads on one SM.
-using StepKernel = void (*)(BatchSeq*, const int*, int, int*, const BatchParams*);
+using StepKernel = void (*)(BatchSeq*, const int*, int, int*, const BatchParams*, int);
 StepKernel step_kernel_for(int threads, int blocks_per_sm) {
     const int t = threads * blocks_per_sm;
-    return t <= 256 ? batched_step_kernel<256> : t <= 512 ? batched_step_kernel<512>
-                                                           : batched_step_kernel<1024>;
+    return t <= 256 ? batched_step_kernel<256, false> : t <= 512 ? batched_step_kernel<512, false>
+                                                                  : batched_step_kernel<1024, false>;
 }
-
 StepKernel cluster_kernel_for(int threads) {
-    return threads <= 256 ? batched_cluster_kernel<256> : threads <= 512 ? batched_cluster_kernel<512>
-                                                                        : batched_cluster_kernel<1024>;
+    return threads <= 256 ? batched_cluster_kernel<256, false>
+                          : threads <= 512 ? batched_cluster_kernel<512, false>
+                                           : batched_cluster_kernel<1024, false>;
 }
 
 __global__ void batch_push_kernel(const double* __restrict__ x, int n, double* X, int ldx, int slot) {
@@ -1031,10 +1160,10 @@ struct seq_batch {
     std::vector<void*> allocs;
     int threads = 512, blocks_per_sm = 1, order_kind = 0;  // 0: largest first, 1: given order
     int cluster = 1;                      // CTAs per sequence (1: one block per sequence)
-    size_t smem_cluster = 0;
+    size_t smem_cluster = 0;              // least shared memory of a CTA (cluster form)
     int autopush = 1;
     cudaGraphExec_t graph = nullptr;
-    size_t smem = 0;
+    size_t smem = 0;                      // least shared memory of a block
     int sms = 0;
 };
 
@@ -1062,9 +1191,60 @@ int batch_order(seq_batch* bt) {
     return cudaStreamSynchronize(bt->stream) == cudaSuccess ? SEQ_OK : SEQ_ECUDA;
 }
 
+// The kernel of the schedule in bt, its threads and its dynamic shared memory:
+// all that the SM has, for the resident CG, or what the guess needs.  A
+// sequence that does not fit on its team's SMs gathers through L1, which the
+// resident CG's shared memory takes away (measured 2 times slower), while one
+// that fits gains a factor of about 3: the resident kernel is taken when at
+// least 60% of the rows lie in sequences that fit.
+// Where most rows are in slot form the products need no index loads, and 512
+// threads per SM with 128 registers keep more values in flight than 1,024 with
+// 64 do (64 sequences, ms a step: clusters of 8 33 against 41, one block each
+// 244 against 304): such a launch runs at most 512.
+struct StepLaunch {
+    StepKernel kern;
+    size_t smem;
+    int threads;
+};
+StepLaunch step_launch(const seq_batch* bt) {
+    const bool cl = bt->cluster > 1;
+    const int bps = bt->blocks_per_sm;
+    const size_t need = cl ? bt->smem_cluster : bt->smem;
+    const int fewer = std::min(bt->threads, 512 / bps);
+    const bool small = fewer * bps <= 256;
+    const StepKernel kern = cl ? (small ? batched_cluster_kernel<256, true>
+                                        : batched_cluster_kernel<512, true>)
+                               : (small ? batched_step_kernel<256, true>
+                                        : batched_step_kernel<512, true>);
+    int dev = 0, optin = 0, sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    cudaFuncAttributes fa;
+    long long most = 0;
+    if (cudaFuncGetAttributes(&fa, (const void*)kern) == cudaSuccess)
+        most = (std::min((long long)optin, (long long)sm / bps - 1024) -
+                (long long)fa.sharedSizeBytes) & ~127LL;
+    else
+        cudaGetLastError();
+    double all = 0.0, slot = 0.0, fits = 0.0;
+    ResLayout L;
+    for (const BatchSeq& q : bt->host) {
+        all += q.n;
+        if (!q.slot) continue;
+        slot += q.n;
+        if (most >= (long long)need &&
+            res_layout(q.n, q.slot_w, q.reach, bt->cluster, sizeof(float), (size_t)most, &L))
+            fits += q.n;
+    }
+    if (fits >= 0.6 * all) return {kern, (size_t)most, fewer};
+    const int threads = slot >= 0.6 * all ? fewer : bt->threads;
+    return {cl ? cluster_kernel_for(threads) : step_kernel_for(threads, bps), need, threads};
+}
+
 // Launch configuration of the cluster form: clusters of bt->cluster CTAs, one
 // CTA per SM, as many clusters as fit at once.  Returns the grid (0: none fits).
-int cluster_grid(seq_batch* bt, StepKernel kern) {
+int cluster_grid(seq_batch* bt, const StepLaunch& sl) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1072,12 +1252,12 @@ int cluster_grid(seq_batch* bt, StepKernel kern) {
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(bt->cluster * bt->sms);
-    cfg.blockDim = dim3(bt->threads);
-    cfg.dynamicSmemBytes = bt->smem_cluster;
+    cfg.blockDim = dim3(sl.threads);
+    cfg.dynamicSmemBytes = sl.smem;
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int nc = 0;
-    if (cudaOccupancyMaxActiveClusters(&nc, (const void*)kern, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&nc, (const void*)sl.kern, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -1092,9 +1272,9 @@ int batch_capture(seq_batch* bt) {
         bt->graph = nullptr;
     }
     const bool cl = bt->cluster > 1;
-    const StepKernel kern = cl ? cluster_kernel_for(bt->threads)
-                               : step_kernel_for(bt->threads, bt->blocks_per_sm);
-    const size_t smem = cl ? bt->smem_cluster : bt->smem;
+    const StepLaunch sl = step_launch(bt);
+    const StepKernel kern = sl.kern;
+    const size_t smem = sl.smem;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess) {
         cudaGetLastError();
@@ -1108,7 +1288,7 @@ int batch_capture(seq_batch* bt) {
             cudaGetLastError();
             return SEQ_ECUDA;
         }
-        grid = cluster_grid(bt, kern);
+        grid = cluster_grid(bt, sl);
         if (grid <= 0) return SEQ_ECUDA;
     }
     cudaGraph_t g = nullptr;
@@ -1123,16 +1303,16 @@ int batch_capture(seq_batch* bt) {
         at[0].val.clusterDim.y = 1;
         at[0].val.clusterDim.z = 1;
         cfg.gridDim = dim3(grid);
-        cfg.blockDim = dim3(bt->threads);
+        cfg.blockDim = dim3(sl.threads);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = bt->cap;
         cfg.attrs = at;
         cfg.numAttrs = 1;
         cudaLaunchKernelEx(&cfg, kern, bt->d_seqs, (const int*)bt->d_order, bt->count, bt->d_queue,
-                           (const BatchParams*)bt->d_prm);
+                           (const BatchParams*)bt->d_prm, (int)smem);
     } else {
-        kern<<<grid, bt->threads, smem, bt->cap>>>(bt->d_seqs, bt->d_order, bt->count, bt->d_queue,
-                                                   bt->d_prm);
+        kern<<<grid, sl.threads, smem, bt->cap>>>(bt->d_seqs, bt->d_order, bt->count, bt->d_queue,
+                                                   bt->d_prm, (int)smem);
     }
     if (cudaStreamEndCapture(bt->cap, &g) != cudaSuccess) {
         cudaGetLastError();
@@ -1197,6 +1377,9 @@ int seq_batch_create(int32_t count, const seq_csr* patterns, int32_t M, int32_t 
     bt->host.resize(count);
     int rc = SEQ_OK;
     const int ldx = (M + 1) & ~1;
+    void* sp = nullptr;
+    rc = batch_alloc(bt, &sp, sizeof(SlotStats));
+    SlotStats* stats = (SlotStats*)sp;
     for (int k = 0; k < count && rc == SEQ_OK; ++k) {
         BatchSeq& q = bt->host[k];
         memset(&q, 0, sizeof(q));
@@ -1218,37 +1401,54 @@ int seq_batch_create(int32_t count, const seq_csr* patterns, int32_t M, int32_t 
         if (rc) break;
         q.val32 = (float*)p;
         cudaMemsetAsync(q.val32, 0, sizeof(float) * (size_t)(q.nnz > 0 ? q.nnz : 1), bt->stream);
-        // SELL-32 copy of the pattern (column indices once; the values are
-        // written by the step kernel; padding stays column -1, value 0).
+        // Copy of the pattern for the products (the values are written by the
+        // step kernel): slot form as for single sequences, else SELL-32
+        // (padding stays column -1, value 0).
         const int ns = (q.n + 31) / 32;
         rc = batch_alloc(bt, &p, sizeof(int) * (size_t)ns);
         if (rc) break;
         int* width = (int*)p;
-        rc = batch_alloc(bt, &p, sizeof(int) * (size_t)(ns + 2));     // + total, widest slice
-        if (rc) break;
-        int* off = (int*)p;
-        launch_sell_layout(q.rowptr, q.n, q.nnz, width, off, bt->stream);
-        int total = 0;
-        if (cudaMemcpyAsync(&total, off + ns, sizeof(int), cudaMemcpyDeviceToHost, bt->stream) !=
-                cudaSuccess ||
+        SlotStats st;
+        launch_slot_stats(q.rowptr, q.colind, q.n, q.nnz, width, stats, bt->stream);
+        if (cudaMemcpyAsync(&st, stats, sizeof(st), cudaMemcpyDeviceToHost, bt->stream) != cudaSuccess ||
             cudaStreamSynchronize(bt->stream) != cudaSuccess) {
             rc = SEQ_ECUDA;
             break;
         }
-        if (total < 0 || (long long)total > 2LL * q.nnz + 64LL * ns) {
+        const long long total = (long long)st.total[0];
+        if (total >= 0x7fffffffLL || total > 2LL * q.nnz + 64LL * ns) {
             rc = SEQ_EINVAL;
             break;
         }
-        rc = batch_alloc(bt, &p, sizeof(int) * (size_t)(total > 0 ? total : 1));
-        if (rc) break;
-        int* scol = (int*)p;
-        rc = batch_alloc(bt, &p, sizeof(float) * (size_t)(total > 0 ? total : 1));
-        if (rc) break;
-        float* sval = (float*)p;
-        launch_sell_fill_f32(q.rowptr, q.colind, q.val32, q.n, q.nnz, off, scol, sval, bt->stream);
-        q.soff = off;
-        q.scol = scol;
-        q.sval = sval;
+        const SlotPlan plan = plan_slots(st, q.n);
+        if (plan.W) {
+            rc = batch_alloc(bt, &p, sizeof(int2) * (size_t)ns * plan.W);
+            if (rc) break;
+            int2* slot = (int2*)p;
+            rc = batch_alloc(bt, &p, sizeof(float) * 32 * (size_t)ns * plan.W);
+            if (rc) break;
+            q.sval = (float*)p;
+            q.slot = slot;
+            q.slot_w = plan.W;
+            q.reach = plan.reach;
+            q.list = plan.list;
+            launch_slot_fill_f32(q.rowptr, q.colind, q.val32, q.n, q.nnz, plan, slot, q.sval,
+                                 bt->stream);
+        } else {
+            rc = batch_alloc(bt, &p, sizeof(int) * (size_t)(ns + 2));     // + total, widest slice
+            if (rc) break;
+            int* off = (int*)p;
+            launch_sell_scan(width, q.n, off, bt->stream);
+            rc = batch_alloc(bt, &p, sizeof(int) * (size_t)(total > 0 ? total : 1));
+            if (rc) break;
+            int* scol = (int*)p;
+            rc = batch_alloc(bt, &p, sizeof(float) * (size_t)(total > 0 ? total : 1));
+            if (rc) break;
+            q.sval = (float*)p;
+            launch_sell_fill_f32(q.rowptr, q.colind, q.val32, q.n, q.nnz, off, scol, q.sval, bt->stream);
+            q.soff = off;
+            q.scol = scol;
+        }
         const size_t nv = ((size_t)q.n + 3) & ~(size_t)3;     // 16-byte aligned vectors
         rc = batch_alloc(bt, &p, sizeof(float) * 4 * nv);
         if (rc) break;
@@ -1341,20 +1541,21 @@ int seq_batch_autotune(seq_batch* bt, const double* const* values, const double*
             for (int ti = 0; ti < 3; ++ti) {
                 for (int bps = 1; bps <= 2; ++bps) {
                     if (cl > 1 && (bps > 1 || thr[ti] < 512)) continue;
-                    const size_t smem = cl > 1 ? bt->smem_cluster : bt->smem;
-                    if ((size_t)bps * smem > 220 * 1024) continue;
+                    const size_t need = cl > 1 ? bt->smem_cluster : bt->smem;
+                    if ((size_t)bps * need > 220 * 1024) continue;
                     bt->threads = thr[ti];
                     bt->blocks_per_sm = bps;
                     bt->order_kind = oi;
                     bt->cluster = cl;
-                    const StepKernel kern =
-                        cl > 1 ? cluster_kernel_for(thr[ti]) : step_kernel_for(thr[ti], bps);
+                    const StepLaunch sl = step_launch(bt);
+                    const StepKernel kern = sl.kern;
+                    const size_t smem = sl.smem;
                     int nb = 0;
                     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem) != cudaSuccess ||
-                        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, thr[ti], smem) !=
+                        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, sl.threads, smem) !=
                             cudaSuccess ||
-                        nb < bps || (cl > 1 && cluster_grid(bt, kern) <= 0)) {
+                        nb < bps || (cl > 1 && cluster_grid(bt, sl) <= 0)) {
                         cudaGetLastError();
                         continue;
                     }

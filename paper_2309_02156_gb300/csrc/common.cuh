@@ -23,6 +23,14 @@ constexpr int kTileChunks = 8;    // CSR entries of a 32-row tile loaded up fron
 constexpr int kTileStage = 2 * kTileChunks * 32;   // shared staging per warp (values, x)
 constexpr int kChebTab = 2 + 2 * 32;   // Chebyshev coefficient table (degree <= 32)
 
+constexpr int kMaxSlots = 24;     // slots per slice of the slot form of a matrix
+
+// Ascending column - row offsets shared by every slice of a matrix in slot form.
+struct OffsetList {
+    int count;                    // 0: the slices have offsets of their own
+    int off[kMaxSlots];
+};
+
 // Device-side copy of the per-call arguments.  The CUDA graphs of a context
 // take a pointer to this struct, so one captured graph serves every call.
 struct DevArgs {
@@ -47,7 +55,7 @@ struct DevArgs {
     int sell_keep;      // 1: load the SELL arrays with L2 evict-last priority (they fit in L2)
     int slot_w;         // slots per slice (slot form)
     int slot_reach;     // largest |column - row| (slot form)
-    int pad1;
+    OffsetList slot_off;   // the offsets of every slice
     double tol;         // relative tolerance of this solve
 };
 

@@ -137,11 +137,11 @@ void launch_round_f32(const double* src, float* dst, int n, cudaStream_t st);
 // CG by a resident team (resident_cg.cuh; matrices in slot form).  Up to these
 // many rows the team is one cluster of 16 (or 8) blocks, above it the grid: a
 // cluster's reduction is faster (0.9 against 2.1 us), a grid's blocks hold
-// fewer rows.  Measured per iteration (cluster, grid): FP64 15,876 rows 7.5 us,
-// 16,900 rows 8.3; FP32 32,761 rows 4.8 us (cluster), 44,100 rows 6.4 (grid)
-// with the cluster extrapolating to 5.7 there and meeting it near 57,000.
-constexpr int kClusterCgRows64 = 16384;
-constexpr int kClusterCgRows32 = 57344;
+// fewer rows.  Per iteration: FP64 22,500 rows 7.8 us in the cluster, 25,600
+// rows 8.3 in the grid; FP32 131,044 rows 6.0 us in the cluster, 136,900 rows
+// 6.6 in the grid.
+constexpr int kClusterCgRows64 = 22528;
+constexpr int kClusterCgRows32 = 131072;
 struct TeamSlot;
 constexpr size_t kTeamSlotBytes = 16 * 2 * 160 + 128;   // slots, counter
 bool launch_resident_cg_f64(const DevArgs* a, KState* ks, double* r, double* q, TeamSlot* slots,
@@ -165,20 +165,28 @@ void launch_cgg_true_residual_f64(const DevArgs* a, KState* ks, double* r, doubl
                                   double* partial, int nblk, int check, cudaStream_t st);
 void launch_cgg_true_residual_f32(const DevArgs* a, KState* ks, float* r, float* p,
                                   float* partial, int nblk, int check, cudaStream_t st);
-// Slot form: widths of the slices and four totals (SELL entries, widest slice,
-// most slots of a slice or kMaxSlots + 1, largest |column - row|), then the fill.
-constexpr int kMaxSlots = 24;
+// Slot form of a matrix: widths of the slices and the totals (SELL entries,
+// widest slice, most slots of a slice or kMaxSlots + 1, largest |column - row|;
+// the distinct offsets), the plan made from them on the host (W = 0: no slot
+// form), then the fill.
+struct SlotStats {
+    unsigned long long total[4];
+    int table[kMaxSlots + 1];
+};
+struct SlotPlan {
+    int W, reach;
+    OffsetList list;          // the offsets of every slice (count 0: slices differ)
+};
 void launch_slot_stats(const int* rowptr, const int* colind, int n, int nnz, int* width,
-                       unsigned long long* stats, cudaStream_t st);
+                       SlotStats* out, cudaStream_t st);
+SlotPlan plan_slots(const SlotStats& st, int n);
 void launch_slot_fill_f64(const int* rowptr, const int* colind, const double* val, int n, int nnz,
-                          int W, int2* slot, double* v, cudaStream_t st);
+                          const SlotPlan& p, int2* slot, double* v, cudaStream_t st);
 void launch_slot_fill_f32(const int* rowptr, const int* colind, const float* val, int n, int nnz,
-                          int W, int2* slot, float* v, cudaStream_t st);
-// Exclusive scan of 32 x width: off[ns] = total, off[ns + 1] = widest slice.
+                          const SlotPlan& p, int2* slot, float* v, cudaStream_t st);
+// CSR -> SELL-32, offsets: exclusive scan of 32 x width (off needs ns + 2 entries, ns =
+// (n + 31) / 32): off[ns] = total, off[ns + 1] = widest slice.
 void launch_sell_scan(const int* width, int n, int* off, cudaStream_t st);
-// CSR -> SELL-32 (slice widths and offsets, then the padded arrays).
-// off needs (n + 31) / 32 + 2 entries: off[ns] = total, off[ns + 1] = widest slice.
-void launch_sell_layout(const int* rowptr, int n, int nnz, int* width, int* off, cudaStream_t st);
 // Re-layout with every slice of width w (off[s] = 32 w s).
 void launch_sell_uniform(int n, int w, int* off, cudaStream_t st);
 void launch_sell_fill_f64(const int* rowptr, const int* colind, const double* val, int n, int nnz,

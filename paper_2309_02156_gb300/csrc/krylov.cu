@@ -2,6 +2,8 @@
 // single-block CG.  The kernel templates live in krylov_kernels.cuh.
 #include <math.h>
 
+#include <algorithm>
+
 #include "krylov_kernels.cuh"
 #include "cg_kernels.cuh"
 #include "resident_cg.cuh"
@@ -101,7 +103,9 @@ void launch_diag_inv_f64(const DevArgs* a, double* dinv, int n, cudaStream_t st,
 // bands), the slice is stored by offset instead: slot k holds one offset and
 // the mask of the rows that have an entry at it, values at (W s + k) 32 + l, W
 // slots in every slice.  It needs every row's columns to ascend strictly and
-// lie in [0, n) (a row's entries then meet their slots in CSR order).
+// lie in [0, n) (a row's entries then meet their slots in CSR order).  Where the
+// whole matrix has few distinct offsets (stencils), all slices use the same
+// ascending list, and products need not read the slot words at all.
 
 // The next slot of a slice: the smallest offset column - row that a lane has
 // not passed yet (kNoSlot: none), called by all lanes; e is advanced in the
@@ -125,15 +129,36 @@ __device__ __forceinline__ int next_slot(const int* __restrict__ colind, int row
 
 // Per slice its width (longest row) into width[s]; over the matrix: stats[0]
 // the SELL entries (32 x the widths), [1] the widest slice, [2] the most slots
-// of a slice (kMaxSlots + 1: no slot form), [3] the largest |offset|.
+// of a slice (kMaxSlots + 1: no slot form), [3] the largest |offset|; table:
+// the distinct offsets of the matrix in any order (kNoSlot: free; the last
+// word stays free unless there are more than kMaxSlots).
+__device__ __forceinline__ void note_offset(int* table, int o) {
+    for (int j = 0; j <= kMaxSlots; ++j) {
+        const int v = *(volatile int*)(table + j);
+        if (v == o) return;
+        if (v == kNoSlot) {
+            const int old = atomicCAS(table + j, kNoSlot, o);
+            if (old == kNoSlot || old == o) return;
+        }
+    }
+}
+
+__global__ void slot_clear_kernel(unsigned long long* stats, int* table) {
+    if (threadIdx.x < 4) stats[threadIdx.x] = 0;
+    if (threadIdx.x <= kMaxSlots) table[threadIdx.x] = kNoSlot;
+}
+
 __global__ void __launch_bounds__(256)
 slot_stats_kernel(const int* __restrict__ rowptr, const int* __restrict__ colind, int n, int nnz,
-                  int* width, unsigned long long* stats) {
+                  int* width, unsigned long long* stats, int* table) {
+    __shared__ int seen[kMaxSlots + 1];
     __shared__ unsigned long long tot[8];
     __shared__ int wmax[8], smax[8], reach[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int s = blockIdx.x * 8 + warp, ns = (n + 31) >> 5;
     int len = 0, slots = 0, far = 0;
+    if (threadIdx.x <= kMaxSlots) seen[threadIdx.x] = kNoSlot;
+    __syncthreads();
     if (s < ns) {
         const int row = s * 32 + lane;
         int rs = 0, re = 0;
@@ -153,6 +178,7 @@ slot_stats_kernel(const int* __restrict__ rowptr, const int* __restrict__ colind
             }
             ++slots;
             far = max(far, abs(o));
+            if (lane == 0) note_offset(seen, o);
         }
         if (lane == 0) width[s] = len;
     }
@@ -175,13 +201,16 @@ slot_stats_kernel(const int* __restrict__ rowptr, const int* __restrict__ colind
         atomicMax(stats + 2, (unsigned long long)smax[0]);
         atomicMax(stats + 3, (unsigned long long)reach[0]);
     }
+    if (threadIdx.x <= kMaxSlots && seen[threadIdx.x] != kNoSlot) note_offset(table, seen[threadIdx.x]);
 }
 
+// Slots by the slice's own offsets in ascending order, or (list.count > 0) by
+// the matrix's: slot k of every slice then has offset list.off[k].
 template <typename VT>
 __global__ void __launch_bounds__(256)
 slot_fill_kernel(const int* __restrict__ rowptr, const int* __restrict__ colind,
-                 const VT* __restrict__ val, int n, int nnz, int W, int2* slot,
-                 VT* __restrict__ val_out) {
+                 const VT* __restrict__ val, int n, int nnz, int W, const OffsetList list,
+                 int2* slot, VT* __restrict__ val_out) {
     const int lane = threadIdx.x & 31;
     const int s = blockIdx.x * 8 + (threadIdx.x >> 5), ns = (n + 31) >> 5;
     if (s >= ns) return;
@@ -195,28 +224,18 @@ slot_fill_kernel(const int* __restrict__ rowptr, const int* __restrict__ colind,
     bool ok = true, mine;
     for (int k = 0; k < W; ++k) {
         const int at = e;
-        const int o = next_slot(colind, row, n, re, e, prev, mine, ok);
+        int o;
+        if (list.count) {
+            o = list.off[k];
+            mine = e < re && colind[e] - row == o;
+            if (mine) ++e;
+        } else {
+            o = next_slot(colind, row, n, re, e, prev, mine, ok);
+        }
         const unsigned mask = __ballot_sync(0xffffffffu, mine);
         if (lane == 0) slot[s * W + k] = mask ? make_int2(o, (int)mask) : make_int2(0, 0);
         val_out[(s * W + k) * 32 + lane] = mine ? val[at] : (VT)0;
     }
-}
-
-__global__ void sell_width_kernel(const int* __restrict__ rowptr, int n, int nnz, int* width) {
-    const int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    const int ns = (n + 31) >> 5;
-    if (s >= ns) return;
-    const int row = s * 32 + lane;
-    int len = 0;
-    if (row < n) {
-        const int rs = max(0, min(rowptr[row], nnz));
-        const int re = max(rs, min(rowptr[row + 1], nnz));
-        len = re - rs;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) len = max(len, __shfl_xor_sync(0xffffffffu, len, o));
-    if (lane == 0) width[s] = len;
 }
 
 // Exclusive scan of 32 * width over the slices by one block (off[ns] = total,
@@ -290,29 +309,43 @@ __global__ void sell_fill_kernel(const int* __restrict__ rowptr, const int* __re
     }
 }
 
-void launch_sell_layout(const int* rowptr, int n, int nnz, int* width, int* off, cudaStream_t st) {
-    const int ns = (n + 31) / 32;
-    sell_width_kernel<<<(ns + 7) / 8, 256, 0, st>>>(rowptr, n, nnz, width);
-    sell_scan_kernel<<<1, 1024, 0, st>>>(width, ns, off);
+void launch_slot_stats(const int* rowptr, const int* colind, int n, int nnz, int* width,
+                       SlotStats* out, cudaStream_t st) {
+    slot_clear_kernel<<<1, 64, 0, st>>>(out->total, out->table);
+    slot_stats_kernel<<<((n + 31) / 32 + 7) / 8, 256, 0, st>>>(rowptr, colind, n, nnz, width,
+                                                               out->total, out->table);
 }
 
-void launch_slot_stats(const int* rowptr, const int* colind, int n, int nnz, int* width,
-                       unsigned long long* stats, cudaStream_t st) {
-    cudaMemsetAsync(stats, 0, 4 * sizeof(unsigned long long), st);
-    const int ns = (n + 31) / 32;
-    slot_stats_kernel<<<(ns + 7) / 8, 256, 0, st>>>(rowptr, colind, n, nnz, width, stats);
+SlotPlan plan_slots(const SlotStats& st, int n) {
+    SlotPlan p = {};
+    const long long ns = (n + 31) / 32, total = (long long)st.total[0];
+    auto fits = [&](long long w) {
+        return w > 0 && w <= kMaxSlots && 32 * ns * w <= total + total / 4 &&
+               32 * ns * w < 0x7fffffffLL;
+    };
+    if (!fits((long long)st.total[2])) return p;
+    p.W = (int)st.total[2];
+    p.reach = (int)st.total[3];
+    int count = 0;
+    while (count <= kMaxSlots && st.table[count] != kNoSlot) ++count;
+    if (fits(count)) {
+        p.W = p.list.count = count;
+        for (int k = 0; k < count; ++k) p.list.off[k] = st.table[k];
+        std::sort(p.list.off, p.list.off + count);
+    }
+    return p;
 }
 
 void launch_slot_fill_f64(const int* rowptr, const int* colind, const double* val, int n, int nnz,
-                          int W, int2* slot, double* v, cudaStream_t st) {
+                          const SlotPlan& p, int2* slot, double* v, cudaStream_t st) {
     slot_fill_kernel<double><<<((n + 31) / 32 + 7) / 8, 256, 0, st>>>(rowptr, colind, val, n, nnz,
-                                                                     W, slot, v);
+                                                                     p.W, p.list, slot, v);
 }
 
 void launch_slot_fill_f32(const int* rowptr, const int* colind, const float* val, int n, int nnz,
-                          int W, int2* slot, float* v, cudaStream_t st) {
+                          const SlotPlan& p, int2* slot, float* v, cudaStream_t st) {
     slot_fill_kernel<float><<<((n + 31) / 32 + 7) / 8, 256, 0, st>>>(rowptr, colind, val, n, nnz,
-                                                                    W, slot, v);
+                                                                    p.W, p.list, slot, v);
 }
 
 void launch_sell_scan(const int* width, int n, int* off, cudaStream_t st) {

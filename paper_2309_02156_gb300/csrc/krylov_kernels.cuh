@@ -343,11 +343,22 @@ __device__ __forceinline__ void sell_rows(const int* __restrict__ off,
 // multiply-adds run in CSR order as in sell_rows: the results are the same
 // bits.  Rows outside a slot's mask read nothing and add an exact zero.
 // FP32 five-point product, 1,048,576 rows: matrix 21 MB + 1.3 MB instead of 42.
-template <typename T, int WM, int G, typename Epi>
-__device__ __forceinline__ void slot_rows_w(const int2* __restrict__ slot,
+//
+// SAME: every slice has the offsets of `list`, and the slot words are not read
+// either.  A row without an entry at an offset then multiplies its stored zero
+// by whatever lies there (nothing outside [0, n)): the same sum unless that
+// value is infinite or NaN, and then the vector it lies in already has a
+// non-finite norm, which ends the solve.
+template <typename T, int WM, int G, bool SAME, typename Epi>
+__device__ __forceinline__ void slot_rows_w(const int2* __restrict__ slot, const OffsetList& list,
                                             const T* __restrict__ val, const T* __restrict__ x,
-                                            int lo, int hi, int nwarps, int W, int keep,
+                                            int n, int lo, int hi, int nwarps, int W, int keep,
                                             const Epi& epi) {
+    int off[WM];
+    if constexpr (SAME) {
+#pragma unroll
+        for (int k = 0; k < WM; ++k) off[k] = k < W ? list.off[k] : 0;
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int s_lo = lo >> 5, s_hi = (hi + 31) >> 5;
     const uint64_t pol = l2_policy(keep != 0);
@@ -364,7 +375,8 @@ __device__ __forceinline__ void slot_rows_w(const int2* __restrict__ slot,
             r[g] = sl * 32 + lane;
 #pragma unroll
             for (int k = 0; k < WM; ++k)
-                m[g][k] = live[g] && k < W ? __ldg(slot + sl * W + k) : make_int2(0, 0);
+                if constexpr (!SAME)
+                    m[g][k] = live[g] && k < W ? __ldg(slot + sl * W + k) : make_int2(0, 0);
         }
 #pragma unroll
         for (int g = 0; g < G; ++g) {
@@ -383,8 +395,16 @@ __device__ __forceinline__ void slot_rows_w(const int2* __restrict__ slot,
 #pragma unroll
             for (int k = 0; k < WM; ++k) {
                 xv[g][k] = 0;
-                if ((m[g][k].y >> lane) & 1) {
-                    const int c = r[g] + m[g][k].x;
+                int c;
+                bool in;
+                if constexpr (SAME) {
+                    c = r[g] + off[k];
+                    in = live[g] && k < W && (unsigned)c < (unsigned)n;
+                } else {
+                    c = r[g] + m[g][k].x;
+                    in = (m[g][k].y >> lane) & 1;
+                }
+                if (in) {
                     xv[g][k] = x[c];
                     if constexpr (GatherProd<Epi>::value) xv[g][k] *= epi.x2[c];
                 }
@@ -425,16 +445,26 @@ __device__ __forceinline__ void slot_rows_loop(const int2* __restrict__ slot,
 }
 
 template <typename T, typename Epi>
-__device__ __forceinline__ void slot_rows(const int2* slot, const T* val, const T* x, int lo,
-                                          int hi, int nwarps, int W, int keep, const Epi& epi) {
+__device__ __forceinline__ void slot_rows(const DevArgs* __restrict__ a, const T* val, const T* x,
+                                          int lo, int hi, int nwarps, const Epi& epi) {
     if (lo >= hi) return;
     constexpr int G = Epi::kSlices > 0 ? Epi::kSlices : (sizeof(T) == 4 ? 3 : 2);
-    if (W <= 5)
-        slot_rows_w<T, 5, G>(slot, val, x, lo, hi, nwarps, W, keep, epi);
-    else if (W <= 9)
-        slot_rows_w<T, 9, sizeof(T) == 4 ? 2 : 1>(slot, val, x, lo, hi, nwarps, W, keep, epi);
-    else
-        slot_rows_loop<T>(slot, val, x, lo, hi, nwarps, W, epi);
+    constexpr int G9 = sizeof(T) == 4 ? 2 : 1;
+    const int n = a->n, W = a->slot_w, keep = a->sell_keep;
+    if (a->slot_off.count) {
+        if (W <= 5)
+            slot_rows_w<T, 5, G, true>(a->slot, a->slot_off, val, x, n, lo, hi, nwarps, W, keep, epi);
+        else if (W <= 9)
+            slot_rows_w<T, 9, G9, true>(a->slot, a->slot_off, val, x, n, lo, hi, nwarps, W, keep, epi);
+        else
+            slot_rows_loop<T>(a->slot, val, x, lo, hi, nwarps, W, epi);
+    } else if (W <= 5) {
+        slot_rows_w<T, 5, G, false>(a->slot, a->slot_off, val, x, n, lo, hi, nwarps, W, keep, epi);
+    } else if (W <= 9) {
+        slot_rows_w<T, 9, G9, false>(a->slot, a->slot_off, val, x, n, lo, hi, nwarps, W, keep, epi);
+    } else {
+        slot_rows_loop<T>(a->slot, val, x, lo, hi, nwarps, W, epi);
+    }
 }
 
 // The product over rows [lo, hi) with the matrix copy of this solve (slot form
@@ -444,7 +474,7 @@ __device__ __forceinline__ bool copy_rows(const DevArgs* __restrict__ a, const T
                                           int nwarps, int* bad, const Epi& epi) {
     const T* val = reinterpret_cast<const T*>(a->sell_val);
     if (a->slot) {
-        slot_rows<T>(a->slot, val, x, lo, hi, nwarps, a->slot_w, a->sell_keep, epi);
+        slot_rows<T>(a, val, x, lo, hi, nwarps, epi);
         return true;
     }
     if (a->sell_off) {

@@ -239,78 +239,318 @@ struct ClusterTeam {
     }
 };
 
-// Where a block's data lies: the gathered vector always in shared memory, the
-// others there as far as they fit (else in the context's global vectors).
+// Where a block's data lies: the gathered vector p always in shared memory with
+// `pad` rows of its neighbours (or zeros) on both sides, the others there as
+// far as they fit, else in the solve's global vectors.
 struct ResLayout {
     int per;           // slices of a block
-    int ext;           // entries of the gathered vector's shared array
+    int pad;           // reach rounded up to 32
     int r_in, q_in, x_in;
     int nval;          // slices whose matrix values are kept in shared memory
 };
 
-// Shared bytes of a layout for element size `el` and W slots per slice.
 __host__ __device__ inline size_t res_bytes(const ResLayout& l, int W, size_t el) {
     const size_t rows = 32 * (size_t)l.per;
-    size_t words = (size_t)l.ext + rows * (size_t)(l.r_in + l.q_in + l.x_in) +
-                   (size_t)l.nval * 32 * W;
-    return ((words * el + 7) & ~(size_t)7) + 8 * (size_t)l.per * W;
+    return (2 * (size_t)l.pad + rows * (size_t)(1 + l.r_in + l.q_in + l.x_in) +
+            (size_t)l.nval * 32 * W) * el + 8 * (size_t)l.per * W;
 }
 
 // Largest layout within `budget` bytes for `nblk` blocks; false if the gathered
 // vector alone does not fit.
-inline bool res_layout(int n, int W, int reach, int nblk, size_t el, size_t budget, ResLayout* l) {
+__host__ __device__ inline bool res_layout(int n, int W, int reach, int nblk, size_t el,
+                                           size_t budget, ResLayout* l) {
     const int ns = (n + 31) / 32;
     l->per = (ns + nblk - 1) / nblk;
-    const long long rows = 32LL * l->per, want = rows + 2LL * reach;
-    l->ext = (int)(want < n + 32LL ? want : n + 32LL);
+    l->pad = (reach + 31) & ~31;
     l->r_in = l->q_in = l->x_in = l->nval = 0;
     if (res_bytes(*l, W, el) > budget) return false;
-    int* which[3] = {&l->r_in, &l->q_in, &l->x_in};
-    for (int* w : which) {
-        *w = 1;
-        if (res_bytes(*l, W, el) > budget) *w = 0;
-    }
+    l->r_in = 1;
+    if (res_bytes(*l, W, el) > budget) l->r_in = 0;
+    l->q_in = 1;
+    if (res_bytes(*l, W, el) > budget) l->q_in = 0;
+    l->x_in = 1;
+    if (res_bytes(*l, W, el) > budget) l->x_in = 0;
     const size_t used = res_bytes(*l, W, el), slice = el * 32 * W;
-    const size_t fit = used + 8 < budget ? (budget - used - 8) / slice : 0;
+    const size_t fit = (budget - used) / slice;
     l->nval = (int)(fit < (size_t)l->per ? fit : (size_t)l->per);
     return true;
 }
 
-// Row sums of the slot-form product over this block's slices: `get(c)` reads
-// entry c - row .. as an index into the gathered array (base + local row +
-// offset); epi(local row, sum, live).
-template <typename T, int WM, typename Epi>
-__device__ __forceinline__ void res_product(const int2* sslot, const T* sval, const T* gval,
-                                            const T* vec, int base, int nsl, int nval, int W,
-                                            int rows, const Epi& epi) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int s = warp; s < nsl; s += nw) {
-        const int i = s * 32 + lane;
-        const T* vv = s < nval ? sval + (size_t)s * W * 32 + lane : gval + (size_t)s * W * 32 + lane;
-        T ax = 0;
-        if constexpr (WM > 0) {
-            T v[WM], x[WM];
+template <typename T> struct Vec16;
+template <> struct Vec16<float> {
+    static constexpr int N = 4;
+    using V = float4;
+    __device__ static void load(const float* p, float (&o)[4]) {
+        const float4 v = *reinterpret_cast<const float4*>(p);
+        o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+    }
+    __device__ static void store(float* p, const float (&o)[4]) {
+        *reinterpret_cast<float4*>(p) = make_float4(o[0], o[1], o[2], o[3]);
+    }
+};
+template <> struct Vec16<double> {
+    static constexpr int N = 2;
+    using V = double2;
+    __device__ static void load(const double* p, double (&o)[2]) {
+        const double2 v = *reinterpret_cast<const double2*>(p);
+        o[0] = v.x; o[1] = v.y;
+    }
+    __device__ static void store(double* p, const double (&o)[2]) {
+        *reinterpret_cast<double2*>(p) = make_double2(o[0], o[1]);
+    }
+};
+
+// One block's part of a CG iteration: its rows [lo, lo + rows) of the system.
+// The struct lies in shared memory and each phase copies what it uses, so that
+// no phase holds another's registers (64 per thread at 1,024 threads).  Vector
+// phases read and write 16 bytes per thread; the last rows % 2 or % 4 go one by
+// one.  `p` is the start of the dynamic shared memory in every call: p[pad + i]
+// is row lo + i, the other vectors' [i].
+template <typename T>
+struct ResBlock {
+    using X = Vec16<T>;
+    int lo, rows, reach, pad, W, nsl, nval;
+    int below, halo;                     // neighbours' rows needed: before, in all
+    int val_at, slot_at;                 // values (elements) and slot words (bytes) from p on
+    T *r, *q, *x;
+    const T* gval;                       // values of the block's slices
+    T* rg;                               // residual of the whole system, for the neighbours
+    bool publish;                        // r lies in shared memory: edge rows go to rg
+    OffsetList list;
+
+    // Splits the shared memory (thread 0), copies the block's slot words and
+    // values and clears p.  All threads; ends with a barrier.
+    __device__ void setup(T* p, const ResLayout& L, int n, int s_lo, int s_hi, int W_, int reach_,
+                          const OffsetList& list_, const int2* slot, const T* val, T* r_g, T* q_g,
+                          T* x_g) {
+        const int cap = 32 * L.per, n_p = cap + 2 * L.pad;
+        if (threadIdx.x == 0) {
+            W = W_;
+            reach = reach_;
+            pad = L.pad;
+            list = list_;
+            nsl = s_hi - s_lo;
+            lo = s_lo * 32;
+            rows = nsl > 0 ? min(n, s_hi * 32) - lo : 0;
+            const int e_lo = max(0, lo - reach), e_hi = min(n, lo + rows + reach);
+            below = nsl > 0 ? lo - e_lo : 0;
+            halo = nsl > 0 ? below + e_hi - (lo + rows) : 0;
+            T* next = p + n_p;
+            rg = r_g;
+            publish = L.r_in != 0;
+            r = L.r_in ? next : r_g + lo;
+            next += L.r_in ? cap : 0;
+            q = L.q_in ? next : q_g + lo;
+            next += L.q_in ? cap : 0;
+            x = L.x_in ? next : x_g + lo;
+            next += L.x_in ? cap : 0;
+            val_at = (int)(next - p);
+            slot_at = (int)((val_at + (size_t)L.nval * 32 * W) * sizeof(T));
+            gval = val + (size_t)s_lo * W * 32;
+            nval = min(L.nval, nsl);
+        }
+        for (int i = threadIdx.x; i < n_p; i += blockDim.x) p[i] = 0;
+        __syncthreads();
+        int2* sslot = slots(p);
+        for (int i = threadIdx.x; i < nsl * W_; i += blockDim.x) sslot[i] = __ldg(slot + s_lo * W_ + i);
+        T* sval = p + val_at;
+        const T* gv = gval;
+        const int nv = nval * W_ * 32;
+        for (int i = threadIdx.x * X::N; i < nv; i += blockDim.x * X::N) {
+            T v[X::N];
+            X::load(gv + i, v);
+            X::store(sval + i, v);
+        }
+        __syncthreads();
+    }
+    __device__ int2* slots(T* p) const {
+        return reinterpret_cast<int2*>(reinterpret_cast<unsigned char*>(p) + slot_at);
+    }
+
+    __device__ void halo_fresh(T* p) const {       // p = r outside the own rows
+        const int h = halo, b = below, l = lo, m = rows, at = pad;
+        const T* g = rg;
+        for (int j = threadIdx.x; j < h; j += blockDim.x) {
+            const int i = j < b ? j - b : m + j - b;
+            p[at + i] = __ldcg(g + l + i);
+        }
+    }
+    __device__ T update_r(T alpha) const {     // r -= alpha q; returns this thread's part of r.r
+        T acc = 0;
+        T* const rr = r;
+        const T* const qq = q;
+        T* const out = rg + lo;
+        const int m = rows, full = m / X::N * X::N, near = publish ? reach : 0;
+        for (int i = threadIdx.x * X::N; i < full; i += blockDim.x * X::N) {
+            T a[X::N], b[X::N];
+            X::load(rr + i, a);
+            X::load(qq + i, b);
 #pragma unroll
-            for (int k = 0; k < WM; ++k) v[k] = k < W ? vv[k * 32] : (T)0;
-#pragma unroll
-            for (int k = 0; k < WM; ++k) {
-                x[k] = 0;
-                if (k < W) {
-                    const int2 m = sslot[s * W + k];
-                    if ((m.y >> lane) & 1) x[k] = vec[base + i + m.x];
-                }
+            for (int u = 0; u < X::N; ++u) {
+                a[u] = fma(-alpha, b[u], a[u]);
+                acc = fma(a[u], a[u], acc);
             }
+            X::store(rr + i, a);
+            if (i < near || (near && i + X::N > m - near)) X::store(out + i, a);
+        }
+        for (int i = full + threadIdx.x; i < m; i += blockDim.x) {
+            const T a = fma(-alpha, qq[i], rr[i]);
+            acc = fma(a, a, acc);
+            rr[i] = a;
+            if (near) out[i] = a;
+        }
+        return acc;
+    }
+    __device__ void update_x(T* p, T alpha, int w0, int step) const {   // x += alpha p, by warps w0, w0 + step, ..
+        T* const xx = x;
+        const T* const pp = p + pad;
+        const int m = rows, full = m / X::N * X::N;
+        const int t = w0 * 32 + (threadIdx.x & 31), hop = step * 32 * X::N;
+        int i = t * X::N;
+        constexpr int kFly = 4;          // x may lie in global memory: several loads in flight
+        for (; i + (kFly - 1) * hop < full; i += kFly * hop) {
+            T a[kFly][X::N];
 #pragma unroll
-            for (int k = 0; k < WM; ++k)
-                if (k < W) ax = fma(v[k], x[k], ax);
-        } else {
-            for (int k = 0; k < W; ++k) {
-                const int2 m = sslot[s * W + k];
-                if ((m.y >> lane) & 1) ax = fma(vv[k * 32], vec[base + i + m.x], ax);
+            for (int f = 0; f < kFly; ++f) X::load(xx + i + f * hop, a[f]);
+#pragma unroll
+            for (int f = 0; f < kFly; ++f) {
+                T b[X::N];
+                X::load(pp + i + f * hop, b);
+#pragma unroll
+                for (int u = 0; u < X::N; ++u) a[f][u] = fma(alpha, b[u], a[f][u]);
+                X::store(xx + i + f * hop, a[f]);
             }
         }
-        epi(i, ax, i < rows);
+        for (; i < full; i += hop) {
+            T a[X::N], b[X::N];
+            X::load(xx + i, a);
+            X::load(pp + i, b);
+#pragma unroll
+            for (int u = 0; u < X::N; ++u) a[u] = fma(alpha, b[u], a[u]);
+            X::store(xx + i, a);
+        }
+        for (i = full + t; i < m; i += step * 32) xx[i] = fma(alpha, pp[i], xx[i]);
     }
-}
+    // p = r + beta p on the own rows and the halo; the neighbours' rows of r are
+    // on their way while the own rows are formed.
+    __device__ void direction(T* p, T beta) const {
+        constexpr int kAhead = sizeof(T) == 4 ? 2 : 4;
+        T ahead[kAhead];
+        const int bd = blockDim.x, h = halo, nb = below, m = rows;
+        const T* const g = rg + lo;
+        const T* const rr = r;
+        T* const pp = p + pad;
+        const bool few = h <= kAhead * bd;
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int j = threadIdx.x + u * bd;
+            ahead[u] = few && j < h ? __ldcg(g + (j < nb ? j - nb : m + j - nb)) : (T)0;
+        }
+        const int full = m / X::N * X::N;
+        for (int i = threadIdx.x * X::N; i < full; i += bd * X::N) {
+            T a[X::N], b[X::N];
+            X::load(pp + i, a);
+            X::load(rr + i, b);
+#pragma unroll
+            for (int u = 0; u < X::N; ++u) a[u] = fma(beta, a[u], b[u]);
+            X::store(pp + i, a);
+        }
+        for (int i = full + threadIdx.x; i < m; i += bd) pp[i] = fma(beta, pp[i], rr[i]);
+        if (few) {
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                const int j = threadIdx.x + u * bd;
+                if (j < h) {
+                    T* at = pp + (j < nb ? j - nb : m + j - nb);
+                    *at = fma(beta, *at, ahead[u]);
+                }
+            }
+        } else {
+            for (int j = threadIdx.x; j < h; j += bd) {
+                const int i = j < nb ? j - nb : m + j - nb;
+                pp[i] = fma(beta, pp[i], __ldcg(g + i));
+            }
+        }
+    }
+    // G slices of the product q = A p, `step` apart: values at v, rows of p at pp.
+    template <int WM, int G>
+    __device__ __forceinline__ static void some(const T* v, const T* pp, T* qq, int s, int step,
+                                                int Wn, int m, const int (&off)[WM], T& acc) {
+        const int lane = threadIdx.x & 31;
+        T a[G][WM], b[G][WM];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const T* at = v + (s + g * step) * Wn * 32 + lane;
+#pragma unroll
+            for (int k = 0; k < WM; ++k) a[g][k] = k < Wn ? at[k * 32] : (T)0;
+        }
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const T* at = pp + (s + g * step) * 32 + lane;
+#pragma unroll
+            for (int k = 0; k < WM; ++k) b[g][k] = k < Wn ? at[off[k]] : (T)0;
+        }
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const int i = (s + g * step) * 32 + lane;
+            T ax = 0;
+#pragma unroll
+            for (int k = 0; k < WM; ++k)
+                if (k < Wn) ax = fma(a[g][k], b[g][k], ax);
+            if (i < m) {
+                qq[i] = ax;
+                acc = fma(pp[i], ax, acc);
+            }
+        }
+    }
+    // All slices have the same offsets: a row without an entry at one multiplies
+    // its stored zero by what lies there (shared memory always holds a value).
+    // GF slices of values from global memory are in flight per warp.
+    template <int WM, int G, int GF>
+    __device__ __forceinline__ T product_same(T* p) const {
+        int off[WM];
+        const int Wn = W, m = rows, nv = nval, ns = nsl, nw = blockDim.x >> 5;
+#pragma unroll
+        for (int k = 0; k < WM; ++k) off[k] = k < Wn ? list.off[k] : 0;
+        T* const qq = q;
+        const T* const pp = p + pad;
+        const T* const sv = p + val_at;
+        const T* const gv = gval;
+        int s = threadIdx.x >> 5;
+        T acc = 0;
+        for (; s + (G - 1) * nw < nv; s += G * nw) some<WM, G>(sv, pp, qq, s, nw, Wn, m, off, acc);
+        for (; s < nv; s += nw) some<WM, 1>(sv, pp, qq, s, nw, Wn, m, off, acc);
+        for (; s + (GF - 1) * nw < ns; s += GF * nw) some<WM, GF>(gv, pp, qq, s, nw, Wn, m, off, acc);
+        for (; s < ns; s += nw) some<WM, 1>(gv, pp, qq, s, nw, Wn, m, off, acc);
+        return acc;
+    }
+    __device__ T product_slots(T* p) const {
+        const int lane = threadIdx.x & 31, nw = blockDim.x >> 5, Wn = W;
+        const int2* ss = slots(p);
+        T acc = 0;
+        for (int s = threadIdx.x >> 5; s < nsl; s += nw) {
+            const int i = s * 32 + lane;
+            const T* v = (s < nval ? p + val_at : gval) + (size_t)s * Wn * 32 + lane;
+            T ax = 0;
+            for (int k = 0; k < Wn; ++k) {
+                const int2 m = ss[s * Wn + k];
+                if ((m.y >> lane) & 1) ax = fma(v[k * 32], p[pad + i + m.x], ax);
+            }
+            if (i < rows) {
+                q[i] = ax;
+                acc = fma(p[pad + i], ax, acc);
+            }
+        }
+        return acc;
+    }
+    // q = A p on the own rows; returns this thread's part of p.q.
+    template <int GF>
+    __device__ __forceinline__ T product(T* p) const {
+        constexpr int G = GF >= 4 ? 2 : 1;
+        if (list.count > 0 && W <= 5) return product_same<5, G, GF>(p);
+        if (list.count > 0 && W <= 9) return product_same<9, 1, 1>(p);
+        return product_slots(p);
+    }
+};
 
 }  // namespace sa

@@ -6,10 +6,10 @@
 //
 // What bounds it: at small sizes the two reductions (0.9 us each in a cluster
 // of 16, 2.1 in a grid of 152, plus their FP64 sums), above about 200,000 rows
-// in FP64 the FP64 pipe (ten multiply-adds per row, 0.53 T/s: 5 us of the 13 us
+// in FP64 the FP64 pipe (ten multiply-adds per row, 0.53 T/s: 5 us of the 12 us
 // per iteration at 262,144 rows).  Per iteration, before (one block below
 // 65,536 rows, three graph kernels above) and now: FP64 4,096 rows 42 -> 5.2 us,
-// 262,144 rows 22.4 -> 13.2 us; FP32 32,761 rows 58 -> 4.8 us.
+// 262,144 rows 22.4 -> 12.0 us; FP32 32,761 rows 58 -> 3.6 us.
 #pragma once
 
 #include "krylov_kernels.cuh"
@@ -32,83 +32,50 @@ __device__ __forceinline__ void resident_cg(const DevArgs* __restrict__ a, KStat
     const int n = a->n, W = a->slot_w, ns = (n + 31) >> 5;
     const int tid = threadIdx.x, bd = blockDim.x;
     const int s_lo = min(ns, tm.rank() * L.per), s_hi = min(ns, s_lo + L.per);
-    const int nsl = s_hi - s_lo;
-    const int r_lo = s_lo * 32, r_hi = min(n, s_hi * 32), rows = max(0, r_hi - r_lo);
-    const int reach = a->slot_reach;
-    const int e_lo = max(0, r_lo - reach), e_hi = min(n, r_hi + reach);
-    const int base = r_lo - e_lo;              // own rows start here in the gathered array
-    const int above = nsl > 0 ? e_hi - r_hi : 0, below = nsl > 0 ? base : 0;
     T* x = Sys::x(a);
     const T* b = Sys::rhs(a);
     const bool zero_x = sizeof(T) == 4;        // the FP32 inner solve starts from d = 0
-    // Shared arrays.
-    T* p = reinterpret_cast<T*>(dsm);
-    T* next = p + L.ext;
-    const int cap = 32 * L.per;
-    T* r = L.r_in ? next : rg + r_lo;
-    next += L.r_in ? cap : 0;
-    T* q = L.q_in ? next : qg + r_lo;
-    next += L.q_in ? cap : 0;
-    T* xs = L.x_in ? next : x + r_lo;
-    next += L.x_in ? cap : 0;
-    T* sval = next;
-    next += (size_t)L.nval * 32 * W;
-    int2* sslot = reinterpret_cast<int2*>(dsm + ((((size_t)((unsigned char*)next - dsm)) + 7) & ~(size_t)7));
-    const T* gval = reinterpret_cast<const T*>(a->sell_val) + (size_t)s_lo * W * 32;
-    const int nval = min(L.nval, nsl);
-    for (int i = tid; i < nsl * W; i += bd) sslot[i] = __ldg(a->slot + s_lo * W + i);
-    for (int i = tid; i < nval * W * 32; i += bd) sval[i] = __ldg(gval + i);
-    __syncthreads();
-    // Rows that other blocks gather go to rg (all own rows when r lies there).
-    auto edge = [&](int i) { return i < reach || i >= rows - reach; };
-    auto product = [&](const T* vec, int at, const auto& epi) {
-        if (W <= 5) res_product<T, 5>(sslot, sval, gval, vec, at, nsl, nval, W, rows, epi);
-        else if (W <= 9) res_product<T, 9>(sslot, sval, gval, vec, at, nsl, nval, W, rows, epi);
-        else res_product<T, 0>(sslot, sval, gval, vec, at, nsl, nval, W, rows, epi);
-    };
-    // r = b - A x over the global iterate, |r|^2; the edge rows are published.
-    // ldcg: other blocks wrote their rows of x during this launch.
+    __shared__ ResBlock<T> B;
+    T* const p = reinterpret_cast<T*>(dsm);
+    B.setup(p, L, n, s_lo, s_hi, W, a->slot_reach, a->slot_off, a->slot,
+            reinterpret_cast<const T*>(a->sell_val), rg, qg, x);
+    const int rows = B.rows, r_lo = B.lo;
+    // r = b - A x over the global iterate (p = r on the own rows), |r|^2; all
+    // own rows are published.  ldcg: other blocks wrote their rows of x during
+    // this launch.
     auto residual = [&](bool start) {
         T acc = 0;
-        auto take = [&](int i, T ax, bool live) {
-            if (!live) return;
+        auto take = [&](int i, T ax) {
             const T ri = b[r_lo + i] - ax;
-            r[i] = ri;
-            if (L.r_in && edge(i)) rg[r_lo + i] = ri;
-            p[base + i] = ri;
+            B.r[i] = ri;
+            if (B.publish) rg[r_lo + i] = ri;
+            p[B.pad + i] = ri;
             acc = fma(ri, ri, acc);
         };
         if (start && zero_x) {
-            for (int i = tid; i < rows; i += bd) take(i, (T)0, true);
+            for (int i = tid; i < rows; i += bd) take(i, (T)0);
         } else {
             const int lane = tid & 31, warp = tid >> 5, nw = bd >> 5;
-            for (int s = warp; s < nsl; s += nw) {
+            for (int s = warp; s < B.nsl; s += nw) {
                 const int i = s * 32 + lane;
                 T ax = 0;
                 for (int k = 0; k < W; ++k) {
-                    const int2 m = sslot[s * W + k];
+                    const int2 m = B.slots(p)[s * W + k];
                     if ((m.y >> lane) & 1)
-                        ax = fma(gval[((size_t)s * W + k) * 32 + lane],
+                        ax = fma(B.gval[((size_t)s * W + k) * 32 + lane],
                                  __ldcg(x + r_lo + i + m.x), ax);
                 }
-                take(i, ax, i < rows);
+                if (i < rows) take(i, ax);
             }
         }
         return acc;
-    };
-    auto fetch_halo = [&](T beta, bool fresh) {    // p = r (fresh) or r + beta p outside own rows
-        for (int i = tid; i < below + above; i += bd) {
-            const int at = i < below ? i : base + rows + (i - below);
-            const T ri = __ldcg(rg + e_lo + at);
-            p[at] = fresh ? ri : fma(beta, p[at], ri);
-        }
     };
     int it = 0, status = ST_OK;
     T bb = 0;
     for (int i = tid; i < rows; i += bd) {
         const T bi = b[r_lo + i];
         bb = fma(bi, bi, bb);
-        xs[i] = zero_x ? (T)0 : x[r_lo + i];
+        B.x[i] = zero_x ? (T)0 : x[r_lo + i];
     }
     tm.total(bb, scratch, [&](T t) {
         s_bnorm = sqrt((double)t);
@@ -127,20 +94,14 @@ __device__ __forceinline__ void resident_cg(const DevArgs* __restrict__ a, KStat
     known = s_go == 0;
     if (s_go == 1 && !tm.late) {
         const int cap_it = a->max_iters;
-        fetch_halo((T)0, true);
+        B.halo_fresh(p);
         for (;;) {
             if (it >= cap_it) {
                 status = ST_NOT_CONVERGED;
                 break;
             }
             __syncthreads();
-            T acc = 0;
-            product(p, base, [&](int i, T ax, bool live) {
-                if (!live) return;
-                q[i] = ax;
-                acc = fma(p[base + i], ax, acc);
-            });
-            tm.total(acc, scratch, [&](T pq) {
+            tm.total(B.template product<sizeof(T) == 4 ? 4 : 2>(p), scratch, [&](T pq) {
                 s_alpha = rr / pq;
                 s_go = pq > 0 ? 1 : (isfinite((double)pq) ? ST_BREAKDOWN : ST_NONFINITE);
             });
@@ -150,27 +111,13 @@ __device__ __forceinline__ void resident_cg(const DevArgs* __restrict__ a, KStat
                 break;
             }
             const T alpha = s_alpha;
-            T rn = 0;
-            const int lane = tid & 31, warp = tid >> 5, nw = bd >> 5;
-            for (int s = warp; s < nsl; s += nw) {
-                const int i = s * 32 + lane;
-                if (i < rows) {
-                    const T ri = fma(-alpha, q[i], r[i]);
-                    r[i] = ri;
-                    if (L.r_in && edge(i)) rg[r_lo + i] = ri;
-                    rn = fma(ri, ri, rn);
-                }
-            }
-            tm.total(rn, scratch, [&](T t) {
+            tm.total(B.update_r(alpha), scratch, [&](T t) {
                 s_beta = t / rr;
                 s_rr = t;
                 s_go = !isfinite((double)t) ? ST_NONFINITE
                        : ((double)t <= t2 && sqrt((double)t) <= target) ? 0 : 1;
-            }, [&](int w0, int step) {             // x += alpha p while the total is on its way
-                for (int s = w0; s < nsl; s += step) {
-                    const int i = s * 32 + lane;
-                    if (i < rows) xs[i] = fma(alpha, p[base + i], xs[i]);
-                }
+            }, [&](int w0, int step) {             // while the total is on its way
+                B.update_x(p, alpha, w0, step);
             });
             if (tm.late) break;
             ++it;
@@ -180,7 +127,7 @@ __device__ __forceinline__ void resident_cg(const DevArgs* __restrict__ a, KStat
             }
             if (s_go == 0) {                       // the true residual decides
                 if (L.x_in)
-                    for (int i = tid; i < rows; i += bd) x[r_lo + i] = xs[i];
+                    for (int i = tid; i < rows; i += bd) x[r_lo + i] = B.x[i];
                 tm.total((T)0, scratch, [&](T) {});
                 if (tm.late) break;
                 tm.total(residual(false), scratch, [&](T t) {
@@ -193,45 +140,18 @@ __device__ __forceinline__ void resident_cg(const DevArgs* __restrict__ a, KStat
                     known = true;
                     break;
                 }
-                fetch_halo((T)0, true);
+                B.halo_fresh(p);
                 continue;
             }
-            const T beta = s_beta;
             rr = s_rr;
-            // The neighbours' rows of r are on their way while the own rows of
-            // the direction are formed.
-            constexpr int kAhead = 4;
-            T ahead[kAhead];
-            const bool few = below + above <= kAhead * bd;
-#pragma unroll
-            for (int u = 0; u < kAhead; ++u) {
-                const int i = tid + u * bd;
-                ahead[u] = few && i < below + above
-                               ? __ldcg(rg + e_lo + (i < below ? i : rows + i)) : (T)0;
-            }
-            for (int s = warp; s < nsl; s += nw) {
-                const int i = s * 32 + lane;
-                if (i < rows) p[base + i] = fma(beta, p[base + i], r[i]);
-            }
-            if (few) {
-#pragma unroll
-                for (int u = 0; u < kAhead; ++u) {
-                    const int i = tid + u * bd;
-                    if (i < below + above) {
-                        const int at = i < below ? i : rows + i;
-                        p[at] = fma(beta, p[at], ahead[u]);
-                    }
-                }
-            } else {
-                fetch_halo(beta, false);
-            }
+            B.direction(p, s_beta);
         }
     }
     // The final iterate and its true residual (reported, and used by the
     // refinement loop).
     __syncthreads();
     if (L.x_in)
-        for (int i = tid; i < rows; i += bd) x[r_lo + i] = xs[i];
+        for (int i = tid; i < rows; i += bd) x[r_lo + i] = B.x[i];
     if (!known && !tm.late) {
         tm.total((T)0, scratch, [&](T) {});
         if (!tm.late) tm.total(residual(false), scratch, [&](T t) { s_rr = t; });

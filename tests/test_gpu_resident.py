@@ -85,3 +85,41 @@ def test_cg_status_codes(n):
             info = seq.solve(Ad, bd, 1e-10, x)
         assert e.value.code == code
         seq.close()
+
+
+@pytest.mark.parametrize("schedule", [(1, 256), (1, 1024), (2, 512), (4, 1024), (8, 512)])
+def test_batch_on_every_form(schedule):
+    """One batch of all forms (offset slots, nine and 24 of them, columns out of
+    order, a reach of half the rows), sizes around the 32-row slices and past the
+    sketch's flush of 33 tiles per team, guesses from a three-column history."""
+    import paper_2309_02156_gb300 as sa
+    rng = np.random.default_rng(sum(schedule))
+    mats = [_spd(n, o, rng) for n, o in [(1, []), (31, [1, 7]), (33, [1, 7]), (5000, [1, 2, 70, 140]),
+                                         (4100, list(range(1, 12))), (3000, [1, 1499]),
+                                         (20011, [1, 141]), (2500, [1, 50])]]
+    arrays = []
+    for k, A in enumerate(mats):
+        A.sort_indices()
+        ptr, ci, v = A.indptr, A.indices.copy(), A.data.copy()
+        if k == len(mats) - 1:
+            for i in range(A.shape[0]):
+                ci[ptr[i]:ptr[i + 1]] = ci[ptr[i]:ptr[i + 1]][::-1]
+                v[ptr[i]:ptr[i + 1]] = v[ptr[i]:ptr[i + 1]][::-1]
+        arrays.append((ptr, ci, v))
+    t = lambda a, d: torch.from_numpy(np.ascontiguousarray(a, dtype=d)).to(DEV)
+    bt = sa.Batch([(t(p, np.int32), t(c, np.int32)) for p, c, _ in arrays], M=3, s=12, zeta=4)
+    if schedule[0] > 1:
+        bt.set_cluster(*schedule)
+    else:
+        bt.set_schedule(schedule[1], 1, 0)
+    bs = [rng.standard_normal(A.shape[0]) for A in mats]
+    for _ in range(3):
+        for k, A in enumerate(mats):
+            bt.push(k, t(rng.standard_normal(A.shape[0]), np.float64))
+    xs = [torch.empty(A.shape[0], dtype=torch.float64, device=DEV) for A in mats]
+    infos = bt.step([t(v, np.float64) for _, _, v in arrays], [t(b, np.float64) for b in bs], xs, 1e-11)
+    for A, b, x, f in zip(mats, bs, xs, infos):
+        assert f["status"] == 0 and f["history_cols"] == 3
+        ref = spl.spsolve(A.tocsc(), b) if A.shape[0] > 1 else b / A.toarray()[0]
+        assert np.linalg.norm(x.cpu().numpy() - ref) <= 6e-11 * np.linalg.norm(ref)
+    bt.close()
