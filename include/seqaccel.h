@@ -181,7 +181,9 @@ int seq_guess(seq_ctx* ctx, const seq_csr* A, const double* b_dev,
  * thread-block cluster for small n, a cooperative grid above.  Other matrices
  * take one thread block for n < 65,536 and the whole GPU above (three kernels
  * per iteration, captured as a CUDA graph of 16 iterations); the algorithm and
- * its stopping test are the same.  With b = 0 the
+ * its stopping test are the same.  GMRES on such matrices up to about 90,000
+ * rows (FP32 inner solves: 70,000 to 200,000) is one launch too, with its basis
+ * on the chip.  With b = 0 the
  * test is ||b - A x|| <= 0 and x = 0 passes it.  Does not push x.
  * Synchronises.
  * Errors: SEQ_EINVAL, SEQ_EBREAKDOWN (CG p^T A p <= 0, singular Hessenberg),

@@ -8,6 +8,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -128,6 +129,10 @@ int fail(seq_ctx* c, int code, const std::string& msg) {
         if (e_ != cudaSuccess)                                                           \
             return fail(ctx, SEQ_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
+
+// Per-block partial sums: 80 per block of the streaming kernels, or two buffers
+// of 32 for each block of a resident grid (which has more blocks at small n).
+size_t partial_doubles(int nblk) { return std::max((size_t)nblk * 80, (size_t)2 * 32 * kTeamBlocks); }
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
@@ -409,6 +414,32 @@ void account_cycle(seq_ctx* ctx, bool f32, int jd, bool updated, int nnz) {
 // the FP32 inner kernels.  Returns a seq_status; h_ks holds the final tail.
 int run_gmres(seq_ctx* ctx, bool f32) {
     KState* ks = f32 ? ctx->ks_in : ctx->ks;
+    if (ctx->sell_ok && ctx->plan.W && !ctx->profiling) {
+        const seq_config& c = ctx->cfg;
+        const ChebConfig cheb{c.precond_kind == 1, ctx->pc_tab};
+        cudaError_t e = cudaSuccess;
+        const bool taken =
+            f32 ? launch_resident_gmres_f32(ctx->d_args_in, ks, (float*)ctx->V, ctx->ldv, c.restart,
+                                            (float*)ctx->kpartial, ctx->team, c.precond_sweeps,
+                                            c.precond_omega, (const float*)ctx->dinv,
+                                            (float*)ctx->za, (float*)ctx->zb, (float*)ctx->tprec,
+                                            &cheb, c.n, ctx->plan, ctx->stream, &e)
+                : launch_resident_gmres_f64(ctx->d_args, ks, (double*)ctx->V, ctx->ldv, c.restart,
+                                            ctx->kpartial, ctx->team, c.precond_sweeps,
+                                            c.precond_omega, (const double*)ctx->dinv,
+                                            (double*)ctx->za, (double*)ctx->zb, (double*)ctx->tprec,
+                                            &cheb, c.n, ctx->plan, ctx->stream, &e);
+        if (taken) {
+            ctx->launches += 1;
+            CK(e);
+            CK(cudaGetLastError());
+            const int rc = read_tail(ctx, ks);
+            if (rc) return rc;
+            if (ctx->h_ks->status == SEQ_ETIMEOUT)
+                return fail(ctx, SEQ_ETIMEOUT, "GMRES: a wait between blocks ran out");
+            return SEQ_OK;
+        }
+    }
     if (!f32)
         launch_gmres_start_f64(ctx->d_args, ks, (double*)ctx->V, ctx->ldv, ctx->kpartial,
                                ctx->nblk, 1, ctx->stream);
@@ -601,7 +632,8 @@ int seq_create(const seq_config* cfg, void* cuda_stream, seq_ctx** out) {
     ok = ok && cudaMalloc(&ctx->lsq, sizeof(LsqOut)) == cudaSuccess;
     ok = ok && cudaMallocHost(&ctx->lsq_host, sizeof(LsqOut)) == cudaSuccess;
     ctx->nblk = stream_grid(n);
-    ok = ok && cudaMalloc(&ctx->kpartial, sizeof(double) * (size_t)ctx->nblk * 80) == cudaSuccess;
+    ok = ok && cudaMalloc(&ctx->kpartial, sizeof(double) * partial_doubles(ctx->nblk)) == cudaSuccess;
+    ok = ok && cudaMalloc((void**)&ctx->team, kTeamSlotBytes) == cudaSuccess;
     ctx->ldv = (size_t)round_up(n, 64);
     if (c.krylov == SEQ_GMRES) {
         ok = ok && cudaMalloc(&ctx->V, el * ctx->ldv * (c.restart + 1)) == cudaSuccess;
@@ -610,7 +642,6 @@ int seq_create(const seq_config* cfg, void* cuda_stream, seq_ctx** out) {
         ok = ok && cudaMalloc(&ctx->r, el * (size_t)n) == cudaSuccess;
         ok = ok && cudaMalloc(&ctx->p, el * (size_t)n) == cudaSuccess;
         ok = ok && cudaMalloc(&ctx->q, el * (size_t)n) == cudaSuccess;
-        ok = ok && cudaMalloc((void**)&ctx->team, kTeamSlotBytes) == cudaSuccess;
     }
     if (ctx->mixed) {
         ok = ok && cudaMalloc(&ctx->rhs32, sizeof(float) * (size_t)n) == cudaSuccess;

@@ -134,6 +134,25 @@ void launch_cg_block_f64(const DevArgs* a, KState* ks, double* r, double* p, dou
 void launch_cg_block_f32(const DevArgs* a, KState* ks, float* r, float* p, float* q,
                          cudaStream_t st);
 void launch_round_f32(const double* src, float* dst, int n, cudaStream_t st);
+// Slot form of a matrix: widths of the slices and the totals (SELL entries,
+// widest slice, most slots of a slice or kMaxSlots + 1, largest |column - row|;
+// the distinct offsets), the plan made from them on the host (W = 0: no slot
+// form), then the fill.
+struct SlotStats {
+    unsigned long long total[4];
+    int table[kMaxSlots + 1];
+};
+struct SlotPlan {
+    int W, reach;
+    OffsetList list;          // the offsets of every slice (count 0: slices differ)
+};
+void launch_slot_stats(const int* rowptr, const int* colind, int n, int nnz, int* width,
+                       SlotStats* out, cudaStream_t st);
+SlotPlan plan_slots(const SlotStats& st, int n);
+void launch_slot_fill_f64(const int* rowptr, const int* colind, const double* val, int n, int nnz,
+                          const SlotPlan& p, int2* slot, double* v, cudaStream_t st);
+void launch_slot_fill_f32(const int* rowptr, const int* colind, const float* val, int n, int nnz,
+                          const SlotPlan& p, int2* slot, float* v, cudaStream_t st);
 // CG by a resident team (resident_cg.cuh; matrices in slot form).  Up to these
 // many rows the team is one cluster of 16 (or 8) blocks, above it the grid: a
 // cluster's reduction is faster (0.9 against 2.1 us), a grid's blocks hold
@@ -143,7 +162,28 @@ void launch_round_f32(const double* src, float* dst, int n, cudaStream_t st);
 constexpr int kClusterCgRows64 = 22528;
 constexpr int kClusterCgRows32 = 131072;
 struct TeamSlot;
-constexpr size_t kTeamSlotBytes = 16 * 2 * 160 + 128;   // slots, counter
+constexpr int kTeamBlocks = 160;                                // most blocks of a grid team
+constexpr size_t kTeamSlotBytes = 16 * 2 * kTeamBlocks + 128;   // slots, counter
+// A whole GMRES solve by a resident grid (resident_gmres.cuh), up to these many
+// rows: above them the streaming kernels of the cycle graph use the chip as well
+// and their launches weigh less.  Per Arnoldi step (cycle graph, resident), us:
+// FP64 10,000 rows 39.7, 27.3; 40,000 45.4, 35.2; 90,000 47.1, 42.2; 131,044
+// 53.2, 54.2.  FP32 22,500 rows 25.6, 21.1; 131,044 30.3, 25.2; 160,000 31,
+// 26.8 (near 200,000 rows the basis fills the shared memory).  FP32 with eight
+// Chebyshev sweeps 40,000 rows 50.2, 44.0; 90,000 50.6, 52.0.
+constexpr int kResGmresRows64 = 92160;
+constexpr int kResGmresRows32 = 196608;
+constexpr int kResGmresRows32Pre = 73728;
+bool launch_resident_gmres_f64(const DevArgs* a, KState* ks, double* V, size_t ldv, int R,
+                               double* kpart, TeamSlot* team, int sweeps, double omega,
+                               const double* dinv, double* za, double* zb, double* t,
+                               const ChebConfig* cheb, int n, const SlotPlan& plan,
+                               cudaStream_t st, cudaError_t* launched);
+bool launch_resident_gmres_f32(const DevArgs* a, KState* ks, float* V, size_t ldv, int R,
+                               float* kpart, TeamSlot* team, int sweeps, double omega,
+                               const float* dinv, float* za, float* zb, float* t,
+                               const ChebConfig* cheb, int n, const SlotPlan& plan,
+                               cudaStream_t st, cudaError_t* launched);
 bool launch_resident_cg_f64(const DevArgs* a, KState* ks, double* r, double* q, TeamSlot* slots,
                             int n, int W, int reach, cudaStream_t st, cudaError_t* launched);
 bool launch_resident_cg_f32(const DevArgs* a, KState* ks, float* r, float* q, TeamSlot* slots,
@@ -165,25 +205,6 @@ void launch_cgg_true_residual_f64(const DevArgs* a, KState* ks, double* r, doubl
                                   double* partial, int nblk, int check, cudaStream_t st);
 void launch_cgg_true_residual_f32(const DevArgs* a, KState* ks, float* r, float* p,
                                   float* partial, int nblk, int check, cudaStream_t st);
-// Slot form of a matrix: widths of the slices and the totals (SELL entries,
-// widest slice, most slots of a slice or kMaxSlots + 1, largest |column - row|;
-// the distinct offsets), the plan made from them on the host (W = 0: no slot
-// form), then the fill.
-struct SlotStats {
-    unsigned long long total[4];
-    int table[kMaxSlots + 1];
-};
-struct SlotPlan {
-    int W, reach;
-    OffsetList list;          // the offsets of every slice (count 0: slices differ)
-};
-void launch_slot_stats(const int* rowptr, const int* colind, int n, int nnz, int* width,
-                       SlotStats* out, cudaStream_t st);
-SlotPlan plan_slots(const SlotStats& st, int n);
-void launch_slot_fill_f64(const int* rowptr, const int* colind, const double* val, int n, int nnz,
-                          const SlotPlan& p, int2* slot, double* v, cudaStream_t st);
-void launch_slot_fill_f32(const int* rowptr, const int* colind, const float* val, int n, int nnz,
-                          const SlotPlan& p, int2* slot, float* v, cudaStream_t st);
 // CSR -> SELL-32, offsets: exclusive scan of 32 x width (off needs ns + 2 entries, ns =
 // (n + 31) / 32): off[ns] = total, off[ns + 1] = widest slice.
 void launch_sell_scan(const int* width, int n, int* off, cudaStream_t st);

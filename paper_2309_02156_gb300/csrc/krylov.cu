@@ -7,6 +7,7 @@
 #include "krylov_kernels.cuh"
 #include "cg_kernels.cuh"
 #include "resident_cg.cuh"
+#include "resident_gmres.cuh"
 
 namespace sa {
 
@@ -607,6 +608,16 @@ bool launch_resident_cg_f64(const DevArgs* a, KState* ks, double* r, double* q, 
 bool launch_resident_cg_f32(const DevArgs* a, KState* ks, float* r, float* q, TeamSlot* slots,
                             int n, int W, int reach, cudaStream_t st, cudaError_t* launched) {
     return launch_resident_cg<SysF32>(a, ks, r, q, slots, n, W, reach, st, launched);
+}
+
+bool launch_resident_gmres_f64(const DevArgs* a, KState* ks, double* V, size_t ldv, int R,
+                               double* kpart, TeamSlot* team, int sweeps, double omega,
+                               const double* dinv, double* za, double* zb, double* t,
+                               const ChebConfig* cheb, int n, const SlotPlan& plan,
+                               cudaStream_t st, cudaError_t* launched) {
+    const GmresArgs<double> A = {V, ldv, R, kpart, team, sweeps, cheb && cheb->on, omega, dinv, za, zb, t,
+                                cheb ? cheb->tab : nullptr};
+    return launch_resident_gmres<SysF64>(a, ks, A, n, plan, st, launched);
 }
 
 void launch_cgg_start_f64(const DevArgs* a, KState* ks, double* r, double* p, double* partial,

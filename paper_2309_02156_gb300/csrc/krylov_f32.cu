@@ -1,6 +1,7 @@
 // FP32 instantiation of the restarted GMRES kernels (inner solves of the
 // mixed-precision form).  The kernel templates live in krylov_kernels.cuh.
 #include "krylov_kernels.cuh"
+#include "resident_gmres.cuh"
 
 namespace sa {
 
@@ -31,6 +32,16 @@ void launch_diag_inv_f32(const DevArgs* a, float* dinv, int n, cudaStream_t st,
     int b = (n + 255) / 256;
     if (b > 152 * 8) b = 152 * 8;
     diag_inv_kernel<SysF32><<<b > 0 ? b : 1, 256, 0, st>>>(a, dinv, bound);
+}
+
+bool launch_resident_gmres_f32(const DevArgs* a, KState* ks, float* V, size_t ldv, int R,
+                               float* kpart, TeamSlot* team, int sweeps, double omega,
+                               const float* dinv, float* za, float* zb, float* t,
+                               const ChebConfig* cheb, int n, const SlotPlan& plan,
+                               cudaStream_t st, cudaError_t* launched) {
+    const GmresArgs<float> A = {V, ldv, R, kpart, team, sweeps, cheb && cheb->on, omega, dinv, za, zb, t,
+                                cheb ? cheb->tab : nullptr};
+    return launch_resident_gmres<SysF32>(a, ks, A, n, plan, st, launched);
 }
 
 }  // namespace sa

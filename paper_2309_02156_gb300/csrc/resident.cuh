@@ -11,10 +11,11 @@
 #pragma once
 
 #include "common.cuh"
+#include "internal.h"
 
 namespace sa {
 
-constexpr int kTeamMax = 160;              // blocks of a grid team
+constexpr int kTeamMax = kTeamBlocks;      // blocks of a grid team
 constexpr int kTeamPolls = 1 << 21;        // bound of a wait (each poll is an L2 round trip)
 
 // One posted partial: the value's bits and the reduction's number.
@@ -154,7 +155,7 @@ struct GridTeam {
                 asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(count) : "memory");
                 const unsigned want = epoch * (unsigned)nb;
                 unsigned seen = 0;
-                for (int left = kTeamPolls; left > 0; --left) {
+                for (int left = *bad ? 0 : kTeamPolls; left > 0; --left) {
                     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
                     if (seen >= want) break;
                 }

@@ -123,3 +123,43 @@ def test_batch_on_every_form(schedule):
         ref = spl.spsolve(A.tocsc(), b) if A.shape[0] > 1 else b / A.toarray()[0]
         assert np.linalg.norm(x.cpu().numpy() - ref) <= 6e-11 * np.linalg.norm(ref)
     bt.close()
+
+
+# rows per block from one slice up, restarts around the pass widths (8, 16, 24,
+# 32 columns) and past the longest resident one (33), each preconditioner
+@pytest.mark.parametrize("opts", [
+    dict(restart=1), dict(restart=9), dict(restart=17), dict(restart=25), dict(restart=32),
+    dict(restart=33), dict(precond_sweeps=1), dict(precond_sweeps=2),
+    dict(precond_sweeps=3, precond_kind="chebyshev"), dict(precond_sweeps=4, precond_kind="chebyshev")])
+@pytest.mark.parametrize("precision", ["f64", "mixed_krylov"])
+@pytest.mark.parametrize("n,offsets", [(1, []), (33, [1, 7]), (1000, [1, 31]), (1000, [1, 2, 31, 62]),
+                                       (20011, [1, 141]), (6000, [1, 2900]), (92161, [1, 303])])
+def test_gmres_matches_direct_solve(n, offsets, precision, opts):
+    rng = np.random.default_rng(n + len(offsets))
+    A = _spd(n, offsets, rng)
+    b = rng.standard_normal(n)
+    info, x = _solve(A, b, 1e-12, krylov="gmres", precision=precision, **opts)
+    assert info["status"] == 0 and info["final_relres"] <= 1e-12
+    assert np.linalg.norm(b - A @ x) <= 1.01e-12 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("n", [500, 30000])
+@pytest.mark.parametrize("precision", ["f64", "mixed_krylov"])
+def test_gmres_status_codes(n, precision):
+    """Iteration cap, a zero and a NaN right-hand side, a start at the solution."""
+    import paper_2309_02156_gb300 as sa
+    rng = np.random.default_rng(n)
+    A = _spd(n, [1, 50], rng)
+    b = rng.standard_normal(n)
+    info, _ = _solve(A, b, 1e-12, max_iters=4, krylov="gmres", precision=precision)
+    assert info["status"] == 1 and info["iters"] == 4
+    info, x = _solve(A, 0 * b, 1e-12, krylov="gmres", precision=precision)
+    assert info["status"] == 0 and info["iters"] == 0 and not x.any()
+    seq = sa.Sequence(n, 2, 8, zeta=2, guess="zero", krylov="gmres", precision=precision)
+    bad = b.copy()
+    bad[n // 2] = np.nan
+    Ad, bd = _dev(A, bad)
+    with pytest.raises(sa.SeqError) as e:
+        seq.solve(Ad, bd, 1e-10, torch.zeros(n, dtype=torch.float64, device=DEV))
+    assert e.value.code == -5
+    seq.close()
