@@ -18,6 +18,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "../../include/seqaccel.h"
@@ -41,20 +42,57 @@ __device__ __forceinline__ float bf(uint16_t v) {
     return __bfloat162float(__ushort_as_bfloat16(v));
 }
 
+// The GEMMs are tiny (at most 64 x 256 x 256 in use), so a kernel's time is the
+// latency of its loads: each block loads kChunk of the summed index at once
+// (16 before, one load latency and two barriers per 16 terms: 137 us per batch
+// of 32, now 56 with the launches below).  Every output stays one chain of fused multiply-adds in the
+// order of the summed index, zeros up to a multiple of 16 included, so results
+// are the same bits as with the smaller tiles.
+constexpr int kChunk = 128;
+constexpr int kStride = kChunk + 1;
+
+struct Tiles {
+    float a[TB * kStride], b[TB * kStride];
+};
+
+// Rows of a batch: sample idx[r] of S (idx NULL: r).
+__device__ __forceinline__ const float* sample_row(const float* S, int stride, const int* idx, int r) {
+    return S + (size_t)(idx ? idx[r] : r) * stride;
+}
+
 // Y = X W^T + b (X: B x K fp32, W: N x K bf16); optional H = GELU(Y).
-__global__ void linear_fwd(const float* __restrict__ X, int ldx, const uint16_t* __restrict__ W,
-                           const float* __restrict__ bias, int B, int N, int K, float* A, float* H) {
-    __shared__ float xs[TB][TB + 1], ws[TB][TB + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
+// FIRST: X is the normalised features of the samples, also written to z.
+template <bool FIRST>
+__global__ void __launch_bounds__(TB * TB)
+linear_fwd(const float* __restrict__ X, int ldx, const uint16_t* __restrict__ W,
+           const float* __restrict__ bias, int B, int N, int K, float* A, float* H,
+           const int* __restrict__ idx, const float* __restrict__ mu, const float* __restrict__ sd,
+           float* z) {
+    __shared__ Tiles t;
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TB + tx;
     const int row = blockIdx.y * TB + ty, col = blockIdx.x * TB + tx;
     float acc = 0.f;
-    for (int k0 = 0; k0 < K; k0 += TB) {
-        xs[ty][tx] = (row < B && k0 + tx < K) ? X[(size_t)row * ldx + k0 + tx] : 0.f;
-        const int wn = blockIdx.x * TB + ty;
-        ws[ty][tx] = (wn < N && k0 + tx < K) ? bf(W[(size_t)wn * K + k0 + tx]) : 0.f;
-        __syncthreads();
+    for (int k0 = 0; k0 < K; k0 += kChunk) {
 #pragma unroll
-        for (int k = 0; k < TB; ++k) acc = fmaf(xs[ty][k], ws[tx][k], acc);
+        for (int q = 0; q < kChunk / TB; ++q) {
+            const int i = tid + q * TB * TB, r = i / kChunk, k = i % kChunk;
+            const int br = blockIdx.y * TB + r, wn = blockIdx.x * TB + r;
+            float xv = 0.f;
+            if (br < B && k0 + k < K) {
+                if constexpr (FIRST) {
+                    xv = (sample_row(X, ldx, idx, br)[k0 + k] - mu[k0 + k]) / sd[k0 + k];
+                    if (blockIdx.x == 0) z[(size_t)br * K + k0 + k] = xv;
+                } else {
+                    xv = X[(size_t)br * ldx + k0 + k];
+                }
+            }
+            t.a[r * kStride + k] = xv;
+            t.b[r * kStride + k] = (wn < N && k0 + k < K) ? bf(W[(size_t)wn * K + k0 + k]) : 0.f;
+        }
+        __syncthreads();
+        const int m = min(kChunk, (K - k0 + TB - 1) / TB * TB);
+#pragma unroll 16
+        for (int k = 0; k < m; ++k) acc = fmaf(t.a[ty * kStride + k], t.b[tx * kStride + k], acc);
         __syncthreads();
     }
     if (row < B && col < N) {
@@ -64,20 +102,26 @@ __global__ void linear_fwd(const float* __restrict__ X, int ldx, const uint16_t*
     }
 }
 
-// dX = (dY W) * GELU'(Apre)   (dY: B x N, W: N x K bf16, dX: B x K)
-__global__ void linear_bwd_input(const float* __restrict__ dY, const uint16_t* __restrict__ W,
-                                 const float* __restrict__ Apre, int B, int N, int K, float* dX) {
-    __shared__ float ds[TB][TB + 1], ws[TB][TB + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int row = blockIdx.y * TB + ty, col = blockIdx.x * TB + tx;
+// dX = (dY W) * GELU'(Apre)   (dY: B x N, W: N x K bf16, dX: B x K), block (bx, by).
+__device__ void bwd_input_block(Tiles& t, int bx, int by, const float* __restrict__ dY,
+                                const uint16_t* __restrict__ W, const float* __restrict__ Apre, int B,
+                                int N, int K, float* dX) {
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TB + tx;
+    const int row = by * TB + ty, col = bx * TB + tx;
     float acc = 0.f;
-    for (int n0 = 0; n0 < N; n0 += TB) {
-        ds[ty][tx] = (row < B && n0 + tx < N) ? dY[(size_t)row * N + n0 + tx] : 0.f;
-        const int wk = blockIdx.x * TB + tx;
-        ws[ty][tx] = (n0 + ty < N && wk < K) ? bf(W[(size_t)(n0 + ty) * K + wk]) : 0.f;
-        __syncthreads();
+    for (int n0 = 0; n0 < N; n0 += kChunk) {
 #pragma unroll
-        for (int n = 0; n < TB; ++n) acc = fmaf(ds[ty][n], ws[n][tx], acc);
+        for (int q = 0; q < kChunk / TB; ++q) {
+            const int i = tid + q * TB * TB;
+            const int r = i / kChunk, n = i % kChunk;            // dY: by rows
+            t.a[r * kStride + n] = (by * TB + r < B && n0 + n < N) ? dY[(size_t)(by * TB + r) * N + n0 + n] : 0.f;
+            const int wn = i / TB, wk = bx * TB + i % TB;        // W: TB columns of each row
+            t.b[(i % TB) * kStride + wn] = (n0 + wn < N && wk < K) ? bf(W[(size_t)(n0 + wn) * K + wk]) : 0.f;
+        }
+        __syncthreads();
+        const int m = min(kChunk, (N - n0 + TB - 1) / TB * TB);
+#pragma unroll 16
+        for (int n = 0; n < m; ++n) acc = fmaf(t.a[ty * kStride + n], t.b[tx * kStride + n], acc);
         __syncthreads();
     }
     if (row < B && col < K) {
@@ -86,79 +130,112 @@ __global__ void linear_bwd_input(const float* __restrict__ dY, const uint16_t* _
     }
 }
 
-// dW = dY^T X (N x K), db = sum_b dY (b in order)
-__global__ void linear_bwd_weight(const float* __restrict__ dY, const float* __restrict__ X, int ldx,
-                                  int B, int N, int K, float* dW, float* db) {
-    __shared__ float ds[TB][TB + 1], xs[TB][TB + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int n = blockIdx.y * TB + ty, k = blockIdx.x * TB + tx;
+// dW = dY^T X (N x K), db = sum_b dY (b in order), block (bx, by).
+__device__ void bwd_weight_block(Tiles& t, int bx, int by, const float* __restrict__ dY,
+                                 const float* __restrict__ X, int ldx, int B, int N, int K, float* dW,
+                                 float* db) {
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TB + tx;
+    const int n = by * TB + ty, k = bx * TB + tx;
     float acc = 0.f, bacc = 0.f;
-    for (int b0 = 0; b0 < B; b0 += TB) {
-        ds[ty][tx] = (b0 + tx < B && blockIdx.y * TB + ty < N) ? dY[(size_t)(b0 + tx) * N + blockIdx.y * TB + ty] : 0.f;
-        xs[ty][tx] = (b0 + ty < B && k < K) ? X[(size_t)(b0 + ty) * ldx + k] : 0.f;
-        __syncthreads();
+    for (int b0 = 0; b0 < B; b0 += kChunk) {
 #pragma unroll
-        for (int b = 0; b < TB; ++b) acc = fmaf(ds[ty][b], xs[b][tx], acc);
-        if (blockIdx.x == 0 && tx == 0) {
-            for (int b = 0; b < TB; ++b) bacc += ds[ty][b];
+        for (int q = 0; q < kChunk / TB; ++q) {
+            const int i = tid + q * TB * TB, b = i / TB, c = i % TB;   // TB columns of each sample
+            t.a[c * kStride + b] = (b0 + b < B && by * TB + c < N) ? dY[(size_t)(b0 + b) * N + by * TB + c] : 0.f;
+            t.b[c * kStride + b] = (b0 + b < B && bx * TB + c < K) ? X[(size_t)(b0 + b) * ldx + bx * TB + c] : 0.f;
         }
+        __syncthreads();
+        const int m = min(kChunk, (B - b0 + TB - 1) / TB * TB);
+#pragma unroll 16
+        for (int b = 0; b < m; ++b) acc = fmaf(t.a[ty * kStride + b], t.b[tx * kStride + b], acc);
+        if (bx == 0 && tx == 0)
+            for (int b = 0; b < m; ++b) bacc += t.a[ty * kStride + b];
         __syncthreads();
     }
     if (n < N && k < K) dW[(size_t)n * K + k] = acc;
-    if (blockIdx.x == 0 && tx == 0 && n < N) db[n] = bacc;
+    if (bx == 0 && tx == 0 && n < N) db[n] = bacc;
 }
 
-__global__ void normalize_kernel(const float* __restrict__ S, int stride, int B, int in,
-                                 const float* __restrict__ mu, const float* __restrict__ sd, float* z) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= B * in) return;
-    const int b = i / in, f = i - b * in;
-    z[i] = (S[(size_t)b * stride + f] - mu[f]) / sd[f];
+// Both gradients of one layer in one launch (they share only dY): blocks
+// [0, wx wy) form dW and db, the others dX (none when dX is NULL).  sum_out: block
+// 0 also writes the mean of loss[0..B) (added in order).
+__global__ void __launch_bounds__(TB * TB)
+linear_bwd(const float* __restrict__ dY, const float* __restrict__ X, int ldx,
+           const uint16_t* __restrict__ W, const float* __restrict__ Apre, int B, int N, int K,
+           float* dW, float* db, float* dX, const float* __restrict__ loss, float* sum_out) {
+    __shared__ Tiles t;
+    const int wx = (K + TB - 1) / TB, wy = (N + TB - 1) / TB;
+    const int blk = blockIdx.x;
+    if (blk < wx * wy)
+        bwd_weight_block(t, blk % wx, blk / wx, dY, X, ldx, B, N, K, dW, db);
+    else
+        bwd_input_block(t, (blk - wx * wy) % wx, (blk - wx * wy) / wx, dY, W, Apre, B, N, K, dX);
+    if (sum_out && blk == 0 && threadIdx.x == 0 && threadIdx.y == 0) {
+        float s = 0.f;
+        for (int i = 0; i < B; ++i) s += loss[i];
+        *sum_out = s / (float)B;
+    }
 }
 
-// y = base + sigma * d; for training also the loss gradient and per-sample loss.
-__global__ void head_kernel(const float* __restrict__ S, int stride, int B, int out,
-                            const float* __restrict__ d, const float* __restrict__ sig, int in,
-                            float* y, float* dd, float* loss) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+// y = base + sigma * d; for training also the loss gradient and per-sample
+// loss.  A warp per sample (one output per lane; out <= 31).
+__global__ void __launch_bounds__(128)
+head_kernel(const float* __restrict__ S, int stride, int B, int out, const float* __restrict__ d,
+            const float* __restrict__ sig, int in, float* y, float* dd, float* loss,
+            const int* __restrict__ idx) {
+    __shared__ float es[4][32], gs[4][32];
+    const int w = threadIdx.x >> 5, j = threadIdx.x & 31, b = blockIdx.x * 4 + w;
     if (b >= B) return;
-    const float* s = S + (size_t)b * stride;
-    float yy[kMaxM];
-    for (int j = 0; j < out; ++j) {
-        yy[j] = s[j] + sig[j] * d[(size_t)b * out + j];
-        y[(size_t)b * out + j] = yy[j];
+    const float* s = sample_row(S, stride, idx, b);
+    float yy = 0.f, e = 0.f;
+    const float* T = s + in;
+    if (j < out) {
+        yy = s[j] + sig[j] * d[(size_t)b * out + j];
+        if (y) y[(size_t)b * out + j] = yy;
+        if (dd) e = yy - T[j];
     }
     if (!dd) return;
-    const float* T = s + in;
+    es[w][j] = e;
+    __syncwarp();
     const float* G = T + out;
     const float nb = s[in + out + out * out];
     const float inv = 1.f / (nb * nb);
-    float l = 0.f;
-    for (int j = 0; j < out; ++j) {
-        float ge = 0.f;
-        for (int k = 0; k < out; ++k) ge = fmaf(G[j * out + k], yy[k] - T[k], ge);
-        l = fmaf(yy[j] - T[j], ge, l);
+    float ge = 0.f;
+    if (j < out) {
+        for (int k = 0; k < out; ++k) ge = fmaf(G[j * out + k], es[w][k], ge);
         dd[(size_t)b * out + j] = (2.f / (float)B) * ge * inv * sig[j];
     }
-    loss[b] = l * inv;
+    gs[w][j] = ge;
+    __syncwarp();
+    if (j == 0) {
+        float l = 0.f;
+        for (int k = 0; k < out; ++k) l = fmaf(es[w][k], gs[w][k], l);
+        loss[b] = l * inv;
+    }
 }
 
-__global__ void sum_kernel(const float* __restrict__ v, int n, float* out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    float s = 0.f;
-    for (int i = 0; i < n; ++i) s += v[i];
-    *out = s / (float)n;
-}
+// Where the bf16 copy of parameter i lies: three weight blocks, biases have none.
+struct Bf16Map {
+    size_t at[3], end[3], to[3];
+    uint16_t* W;
+};
 
 __global__ void adam_kernel(float* P, const float* __restrict__ G, float* M, float* V, size_t n,
-                            float lr, float b1, float b2, float eps, float c1, float c2) {
+                            float lr, float b1, float b2, float eps, float c1, float c2,
+                            const Bf16Map map) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const float g = G[i];
         const float m = b1 * M[i] + (1.f - b1) * g;
         const float v = b2 * V[i] + (1.f - b2) * g * g;
         M[i] = m;
         V[i] = v;
-        P[i] -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+        float p = P[i];
+        p -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+        P[i] = p;
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (i >= map.at[q] && i < map.end[q])
+                map.W[map.to[q] + (i - map.at[q])] = __bfloat16_as_ushort(__float2bfloat16_rn(p));
     }
 }
 
@@ -177,22 +254,25 @@ __global__ void he_init_kernel(float* W, size_t n, int fan_in, uint64_t seed, ui
     }
 }
 
-__global__ void gather_kernel(const float* __restrict__ S, const int* __restrict__ idx, int B,
-                              int stride, float* out) {
-    const size_t total = (size_t)B * stride;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int b = (int)(i / stride);
-        out[i] = S[(size_t)idx[b] * stride + (i - (size_t)b * stride)];
-    }
-}
-
 // Per-feature mean/std over the samples, and per-output std of (target - base).
 __global__ void norm_stats_kernel(const float* __restrict__ S, int stride, int count, int in,
                                   int out, float* mu, float* sd, float* sig) {
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f < in) {
         double s = 0, s2 = 0;
-        for (int b = 0; b < count; ++b) {
+        int b = 0;
+        for (; b + 16 <= count; b += 16) {        // loads ahead of the ordered sums
+            float v[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) v[u] = S[(size_t)(b + u) * stride + f];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+                const double w = v[u];
+                s += w;
+                s2 += w * w;
+            }
+        }
+        for (; b < count; ++b) {
             const double v = S[(size_t)b * stride + f];
             s += v;
             s2 += v * v;
@@ -203,7 +283,18 @@ __global__ void norm_stats_kernel(const float* __restrict__ S, int stride, int c
     } else if (f < in + out) {
         const int j = f - in;
         double s2 = 0;
-        for (int b = 0; b < count; ++b) {
+        int b = 0;
+        for (; b + 16 <= count; b += 16) {
+            float v[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) v[u] = S[(size_t)(b + u) * stride + in + j] - S[(size_t)(b + u) * stride + j];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+                const double w = v[u];
+                s2 += w * w;
+            }
+        }
+        for (; b < count; ++b) {
             const double v = S[(size_t)b * stride + in + j] - S[(size_t)b * stride + j];
             s2 += v * v;
         }
@@ -317,8 +408,10 @@ struct seq_mlp {
     float *P = nullptr, *G = nullptr, *Mm = nullptr, *Vv = nullptr;
     uint16_t* Wb = nullptr;            // bf16 W1 | W2 | W3
     float *mu = nullptr, *sd = nullptr, *sig = nullptr;
-    float *z, *a1, *h1, *a2, *h2, *d, *y, *dd, *dh2, *dh1, *loss, *batch, *scalar;
-    int* idx = nullptr;
+    float *z, *a1, *h1, *a2, *h2, *d, *y, *dd, *dh2, *dh1, *loss, *scalar;
+    int* idx = nullptr;                // a training call's batches, and its losses
+    float* step_loss = nullptr;
+    size_t idx_cap = 0, loss_cap = 0;
     int t = 0;
     std::vector<void*> allocs;
 };
@@ -334,6 +427,20 @@ int mlp_alloc(seq_mlp* m, void** p, size_t bytes) {
     return SEQ_OK;
 }
 
+// A buffer that grows and is kept for the next call.
+int mlp_reserve(void** p, size_t* cap, size_t want, size_t size) {
+    if (want <= *cap) return SEQ_OK;
+    if (*p) cudaFree(*p);
+    *p = nullptr;
+    *cap = 0;
+    if (cudaMalloc(p, size * want) != cudaSuccess) {
+        cudaGetLastError();
+        return SEQ_ENOMEM;
+    }
+    *cap = want;
+    return SEQ_OK;
+}
+
 void refresh_bf16(seq_mlp* m) {
     const size_t n1 = (size_t)m->hid * m->in, n2 = (size_t)m->hid * m->hid, n3 = (size_t)m->out * m->hid;
     to_bf16_kernel<<<64, 256, 0, m->stream>>>(m->P + m->oW1, m->Wb, n1);
@@ -341,36 +448,37 @@ void refresh_bf16(seq_mlp* m) {
     to_bf16_kernel<<<16, 256, 0, m->stream>>>(m->P + m->oW3, m->Wb + n1 + n2, n3);
 }
 
-// Forward pass on B samples (rows of S with the sample stride).
-void mlp_forward(seq_mlp* m, const float* S, int stride, int B, cudaStream_t st) {
+// Forward pass on B samples (rows idx[..] of S with the sample stride).
+void mlp_forward(seq_mlp* m, const float* S, int stride, int B, cudaStream_t st,
+                 const int* idx = nullptr) {
     const size_t n1 = (size_t)m->hid * m->in, n2 = (size_t)m->hid * m->hid;
-    normalize_kernel<<<(B * m->in + 255) / 256, 256, 0, st>>>(S, stride, B, m->in, m->mu, m->sd, m->z);
-    dim3 blk(TB, TB);
-    linear_fwd<<<dim3((m->hid + TB - 1) / TB, (B + TB - 1) / TB), blk, 0, st>>>(
-        m->z, m->in, m->Wb, m->P + m->ob1, B, m->hid, m->in, m->a1, m->h1);
-    linear_fwd<<<dim3((m->hid + TB - 1) / TB, (B + TB - 1) / TB), blk, 0, st>>>(
-        m->h1, m->hid, m->Wb + n1, m->P + m->ob2, B, m->hid, m->hid, m->a2, m->h2);
-    linear_fwd<<<dim3((m->out + TB - 1) / TB, (B + TB - 1) / TB), blk, 0, st>>>(
-        m->h2, m->hid, m->Wb + n1 + n2, m->P + m->ob3, B, m->out, m->hid, m->d, nullptr);
+    const dim3 blk(TB, TB), hidden((m->hid + TB - 1) / TB, (B + TB - 1) / TB);
+    linear_fwd<true><<<hidden, blk, 0, st>>>(S, stride, m->Wb, m->P + m->ob1, B, m->hid, m->in, m->a1,
+                                             m->h1, idx, m->mu, m->sd, m->z);
+    linear_fwd<false><<<hidden, blk, 0, st>>>(m->h1, m->hid, m->Wb + n1, m->P + m->ob2, B, m->hid,
+                                              m->hid, m->a2, m->h2, nullptr, nullptr, nullptr, nullptr);
+    linear_fwd<false><<<dim3((m->out + TB - 1) / TB, (B + TB - 1) / TB), blk, 0, st>>>(
+        m->h2, m->hid, m->Wb + n1 + n2, m->P + m->ob3, B, m->out, m->hid, m->d, nullptr, nullptr,
+        nullptr, nullptr, nullptr);
 }
 
-// Loss and gradients (into m->G) on B samples.
-void mlp_backward(seq_mlp* m, const float* S, int stride, int B) {
+// Loss (mean over the samples, to *mean) and gradients (into m->G) on B samples.
+void mlp_backward(seq_mlp* m, const float* S, int stride, int B, const int* idx, float* mean) {
     const size_t n1 = (size_t)m->hid * m->in, n2 = (size_t)m->hid * m->hid;
-    head_kernel<<<(B + 127) / 128, 128, 0, m->stream>>>(S, stride, B, m->out, m->d, m->sig, m->in, m->y,
-                                                        m->dd, m->loss);
-    dim3 blk(TB, TB);
-    linear_bwd_weight<<<dim3((m->hid + TB - 1) / TB, (m->out + TB - 1) / TB), blk, 0, m->stream>>>(
-        m->dd, m->h2, m->hid, B, m->out, m->hid, m->G + m->oW3, m->G + m->ob3);
-    linear_bwd_input<<<dim3((m->hid + TB - 1) / TB, (B + TB - 1) / TB), blk, 0, m->stream>>>(
-        m->dd, m->Wb + n1 + n2, m->a2, B, m->out, m->hid, m->dh2);
-    linear_bwd_weight<<<dim3((m->hid + TB - 1) / TB, (m->hid + TB - 1) / TB), blk, 0, m->stream>>>(
-        m->dh2, m->h1, m->hid, B, m->hid, m->hid, m->G + m->oW2, m->G + m->ob2);
-    linear_bwd_input<<<dim3((m->hid + TB - 1) / TB, (B + TB - 1) / TB), blk, 0, m->stream>>>(
-        m->dh2, m->Wb + n1, m->a1, B, m->hid, m->hid, m->dh1);
-    linear_bwd_weight<<<dim3((m->in + TB - 1) / TB, (m->hid + TB - 1) / TB), blk, 0, m->stream>>>(
-        m->dh1, m->z, m->in, B, m->hid, m->in, m->G + m->oW1, m->G + m->ob1);
-    sum_kernel<<<1, 1, 0, m->stream>>>(m->loss, B, m->scalar);
+    head_kernel<<<(B + 3) / 4, 128, 0, m->stream>>>(S, stride, B, m->out, m->d, m->sig, m->in, m->y,
+                                                    m->dd, m->loss, idx);
+    const dim3 blk(TB, TB);
+    auto tiles = [](int n) { return (n + TB - 1) / TB; };
+    const int bx = tiles(B);
+    linear_bwd<<<tiles(m->hid) * (tiles(m->out) + bx), blk, 0, m->stream>>>(
+        m->dd, m->h2, m->hid, m->Wb + n1 + n2, m->a2, B, m->out, m->hid, m->G + m->oW3, m->G + m->ob3,
+        m->dh2, m->loss, mean);
+    linear_bwd<<<tiles(m->hid) * (tiles(m->hid) + bx), blk, 0, m->stream>>>(
+        m->dh2, m->h1, m->hid, m->Wb + n1, m->a1, B, m->hid, m->hid, m->G + m->oW2, m->G + m->ob2,
+        m->dh1, nullptr, nullptr);
+    linear_bwd<<<tiles(m->in) * tiles(m->hid), blk, 0, m->stream>>>(
+        m->dh1, m->z, m->in, nullptr, nullptr, B, m->hid, m->in, m->G + m->oW1, m->G + m->ob1, nullptr,
+        nullptr, nullptr);
 }
 
 }  // namespace
@@ -380,8 +488,8 @@ namespace sa {
 // concurrently with training on another stream).
 void mlp_predict_dev(seq_mlp* m, const float* features, int B, float* y, cudaStream_t st) {
     mlp_forward(m, features, m->stride, B, st);
-    head_kernel<<<(B + 127) / 128, 128, 0, st>>>(features, m->stride, B, m->out, m->d, m->sig,
-                                                 m->in, y, nullptr, nullptr);
+    head_kernel<<<(B + 3) / 4, 128, 0, st>>>(features, m->stride, B, m->out, m->d, m->sig, m->in, y,
+                                             nullptr, nullptr, nullptr);
 }
 int mlp_stride(const seq_mlp* m) { return m->stride; }
 int mlp_dims_ok(const seq_mlp* m, int M, int s) { return m && m->M == M && m->s == s; }
@@ -441,16 +549,11 @@ int seq_mlp_create(int32_t M, int32_t s, int32_t hidden, int32_t max_batch, uint
     A(&m->dh2, B * m->hid);
     A(&m->dh1, B * m->hid);
     A(&m->loss, B);
-    A(&m->batch, B * m->stride);
     A(&m->scalar, 4);
     if (rc == SEQ_OK) {
         rc = mlp_alloc(m, &p, sizeof(uint16_t) * ((size_t)m->hid * m->in + (size_t)m->hid * m->hid +
                                                    (size_t)m->out * m->hid));
         m->Wb = (uint16_t*)p;
-    }
-    if (rc == SEQ_OK) {
-        rc = mlp_alloc(m, &p, sizeof(int) * B);
-        m->idx = (int*)p;
     }
     if (rc != SEQ_OK) {
         seq_mlp_destroy(m);
@@ -481,6 +584,8 @@ int seq_mlp_destroy(seq_mlp* m) {
     if (!m) return SEQ_OK;
     cudaStreamSynchronize(m->stream);
     for (void* p : m->allocs) cudaFree(p);
+    if (m->idx) cudaFree(m->idx);
+    if (m->step_loss) cudaFree(m->step_loss);
     delete m;
     return SEQ_OK;
 }
@@ -529,7 +634,7 @@ int seq_mlp_loss_grad(seq_mlp* m, const float* samples_dev, int32_t B, float* lo
                       float* grads_host) {
     if (!m || !samples_dev || B < 1 || B > m->bmax) return SEQ_EINVAL;
     mlp_forward(m, samples_dev, m->stride, B, m->stream);
-    mlp_backward(m, samples_dev, m->stride, B);
+    mlp_backward(m, samples_dev, m->stride, B, nullptr, m->scalar);
     if (cudaStreamSynchronize(m->stream) != cudaSuccess) return SEQ_ECUDA;
     if (loss_host && cudaMemcpy(loss_host, m->scalar, sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess)
         return SEQ_ECUDA;
@@ -542,38 +647,65 @@ int seq_mlp_train(seq_mlp* m, const float* samples_dev, int32_t count, int32_t e
                   float lr, uint64_t seed, float* losses_host) {
     if (!m || !samples_dev || count < 1 || epochs < 0 || batch < 1 || batch > m->bmax || !(lr > 0))
         return SEQ_EINVAL;
-    std::vector<int> perm(count);
-    std::vector<float> ep_loss(epochs > 0 ? epochs : 1, 0.f);
+    // The sample numbers of as many epochs as kMaxRows allows go up at once and
+    // their batches' losses come back together: one synchronisation per group.
+    constexpr long long kMaxRows = 1 << 22;
+    const int nb = count / batch;
+    const long long per_epoch = (long long)nb * batch;
+    const int group = per_epoch > 0 ? (int)std::max(1LL, std::min((long long)epochs, kMaxRows / per_epoch)) : 1;
+    std::vector<int> perm(count), rows;
+    std::vector<float> losses, ep_loss(epochs > 0 ? epochs : 1, 0.f);
+    Bf16Map map;
+    const size_t at[3] = {m->oW1, m->oW2, m->oW3};
+    const size_t len[3] = {(size_t)m->hid * m->in, (size_t)m->hid * m->hid, (size_t)m->out * m->hid};
+    map.W = m->Wb;
+    for (size_t q = 0, to = 0; q < 3; to += len[q], ++q) {
+        map.at[q] = at[q];
+        map.end[q] = at[q] + len[q];
+        map.to[q] = to;
+    }
     uint64_t ctr = 0;
-    for (int e = 0; e < epochs; ++e) {
-        for (int i = 0; i < count; ++i) perm[i] = i;
-        for (int i = count - 1; i > 0; --i) {          // Fisher-Yates with SplitMix64 draws
-            uint64_t z = seed + (++ctr) * 0x9E3779B97F4A7C15ull;
-            z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-            z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-            z ^= z >> 31;
-            const int j = (int)(((z >> 32) * (uint64_t)(i + 1)) >> 32);
-            std::swap(perm[i], perm[j]);
+    for (int e0 = 0; e0 < epochs && nb > 0; e0 += group) {
+        const int ne = std::min(group, epochs - e0);
+        const size_t steps = (size_t)ne * nb;
+        rows.clear();
+        for (int e = 0; e < ne; ++e) {
+            for (int i = 0; i < count; ++i) perm[i] = i;
+            for (int i = count - 1; i > 0; --i) {      // Fisher-Yates with SplitMix64 draws
+                uint64_t z = seed + (++ctr) * 0x9E3779B97F4A7C15ull;
+                z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+                z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+                z ^= z >> 31;
+                const int j = (int)(((z >> 32) * (uint64_t)(i + 1)) >> 32);
+                std::swap(perm[i], perm[j]);
+            }
+            rows.insert(rows.end(), perm.begin(), perm.begin() + per_epoch);
         }
-        double acc = 0;
-        int nb = 0;
-        for (int b0 = 0; b0 + batch <= count; b0 += batch) {
-            cudaMemcpyAsync(m->idx, perm.data() + b0, sizeof(int) * batch, cudaMemcpyHostToDevice, m->stream);
-            gather_kernel<<<128, 256, 0, m->stream>>>(samples_dev, m->idx, batch, m->stride, m->batch);
-            mlp_forward(m, m->batch, m->stride, batch, m->stream);
-            mlp_backward(m, m->batch, m->stride, batch);
+        losses.resize(steps);
+        int rc = mlp_reserve((void**)&m->idx, &m->idx_cap, rows.size(), sizeof(int));
+        if (!rc) rc = mlp_reserve((void**)&m->step_loss, &m->loss_cap, steps, sizeof(float));
+        if (rc) return rc;
+        if (cudaMemcpyAsync(m->idx, rows.data(), sizeof(int) * rows.size(), cudaMemcpyHostToDevice,
+                            m->stream) != cudaSuccess)
+            return SEQ_ECUDA;
+        for (size_t i = 0; i < steps; ++i) {
+            const int* idx = m->idx + i * batch;
+            mlp_forward(m, samples_dev, m->stride, batch, m->stream, idx);
+            mlp_backward(m, samples_dev, m->stride, batch, idx, m->step_loss + i);
             m->t += 1;
             const float c1 = 1.f - powf(0.9f, (float)m->t), c2 = 1.f - powf(0.999f, (float)m->t);
             adam_kernel<<<256, 256, 0, m->stream>>>(m->P, m->G, m->Mm, m->Vv, m->np, lr, 0.9f, 0.999f,
-                                                    1e-8f, c1, c2);
-            refresh_bf16(m);
-            float l = 0.f;
-            cudaMemcpyAsync(&l, m->scalar, sizeof(float), cudaMemcpyDeviceToHost, m->stream);
-            if (cudaStreamSynchronize(m->stream) != cudaSuccess) return SEQ_ECUDA;
-            acc += l;
-            ++nb;
+                                                    1e-8f, c1, c2, map);
         }
-        ep_loss[e] = nb ? (float)(acc / nb) : 0.f;
+        if (cudaMemcpyAsync(losses.data(), m->step_loss, sizeof(float) * steps, cudaMemcpyDeviceToHost,
+                            m->stream) != cudaSuccess ||
+            cudaStreamSynchronize(m->stream) != cudaSuccess)
+            return SEQ_ECUDA;
+        for (int e = 0; e < ne; ++e) {
+            double acc = 0;
+            for (int i = 0; i < nb; ++i) acc += losses[(size_t)e * nb + i];
+            ep_loss[e0 + e] = (float)(acc / nb);
+        }
     }
     if (losses_host && epochs > 0) memcpy(losses_host, ep_loss.data(), sizeof(float) * epochs);
     return cudaGetLastError() == cudaSuccess ? SEQ_OK : SEQ_ECUDA;
