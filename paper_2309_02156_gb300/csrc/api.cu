@@ -35,7 +35,7 @@ struct seq_ctx {
     LsqOut* lsq = nullptr;
     LsqOut* lsq_host = nullptr;      // pinned
     int nblk = 0;
-    double* kpartial = nullptr;      // nblk * 80 doubles (per-block partial sums)
+    double* kpartial = nullptr;      // partial_doubles(nblk) (per-block partial sums)
     size_t ldv = 0;
     void* V = nullptr;               // (restart+1) x ldv basis (GMRES)
     void* w = nullptr;
@@ -130,9 +130,12 @@ int fail(seq_ctx* c, int code, const std::string& msg) {
             return fail(ctx, SEQ_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
-// Per-block partial sums: 80 per block of the streaming kernels, or two buffers
-// of 32 for each block of a resident grid (which has more blocks at small n).
-size_t partial_doubles(int nblk) { return std::max((size_t)nblk * 80, (size_t)2 * 32 * kTeamBlocks); }
+// Per-block partial sums: a norm's and two CGS passes' per block of the
+// streaming kernels, or two buffers of 32 for each block of a resident grid
+// (which has more blocks at small n).
+size_t partial_doubles(int nblk) {
+    return std::max((size_t)nblk * (2 + 2 * kMaxBasis), (size_t)2 * 32 * kTeamBlocks);
+}
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 

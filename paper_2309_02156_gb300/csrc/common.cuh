@@ -64,8 +64,6 @@ struct KState {
     double sigma[kMaxBasis];        // stored basis column k = v_k / sigma_k
     double h1[kMaxBasis];           // first CGS pass coefficients
     double h2[kMaxBasis];           // second CGS pass coefficients
-    double c1[kMaxBasis];           // sigma_k * h1_k (applied to stored columns)
-    double c2[kMaxBasis];           // sigma_k * h2_k
     double H[kMaxBasis * kMaxRestart];  // rotated Hessenberg, column-major (ld kMaxBasis)
     double cs[kMaxRestart];
     double sn[kMaxRestart];

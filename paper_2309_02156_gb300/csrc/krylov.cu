@@ -15,6 +15,7 @@ int stream_grid(int n) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (sms > kTeamBlocks) sms = kTeamBlocks;      // what pass_coefficients adds up
     const int need = (n + kStreamBlock - 1) / kStreamBlock;
     return need < sms ? (need > 0 ? need : 1) : sms;
 }

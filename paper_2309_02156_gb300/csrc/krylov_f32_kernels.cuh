@@ -169,17 +169,7 @@ f32_spmv_dot_kernel(const DevArgs* __restrict__ a, KState* ks, const float* __re
 #pragma unroll
     for (int k = 0; k < NK; ++k) part[k] = 0.f;
     f32_rows<NK, 0>(V, ldv, w, nullptr, nullptr, lo, hi, part);
-    block_columns<float, NK>(part, NK, wsum, partial + (size_t)blockIdx.x * kMaxBasis);
-    if (last_block_arrive(&ks->counter[CNT_DOT])) {
-        __shared__ double tot[NK];
-        reduce_blocks(partial, gridDim.x, kMaxBasis, NK, tot);
-        for (int k = threadIdx.x; k < NK; k += blockDim.x) {
-            const double hk = ks->sigma[k] * tot[k];
-            ks->h1[k] = hk;
-            ks->c1[k] = ks->sigma[k] * hk;
-        }
-        if (threadIdx.x == 0) ks->counter[CNT_DOT] = 0;
-    }
+    block_columns<float, NK>(part, NK, wsum, pass_sums(partial, gridDim.x, 0) + blockIdx.x, gridDim.x);
 }
 
 template <int NK>
@@ -188,29 +178,15 @@ f32_pass2_kernel(const DevArgs* __restrict__ a, KState* ks, const float* __restr
                  float* __restrict__ w, float* partial, int j) {
     __shared__ float cf[NK];
     __shared__ float wsum[kWarps * NK];
-    // The end-of-cycle flag and the coefficients are loaded together (one
-    // latency); every thread sees the same flag, so the return is uniform.
-    const int over = ks->cycle_over;
-    for (int k = threadIdx.x; k < NK; k += blockDim.x) cf[k] = (float)ks->c1[k];
-    if (over) return;
-    __syncthreads();
+    if (ks->cycle_over) return;
+    pass_coefficients<float>(pass_sums(partial, gridDim.x, 0), NK, ks, ks->h1, cf);
     int lo, hi;
     block_rows(a->n, gridDim.x, blockIdx.x, lo, hi);
     float part[NK];
 #pragma unroll
     for (int k = 0; k < NK; ++k) part[k] = 0.f;
     f32_rows<NK, 1>(V, ldv, w, nullptr, cf, lo, hi, part);
-    block_columns<float, NK>(part, NK, wsum, partial + (size_t)blockIdx.x * kMaxBasis);
-    if (last_block_arrive(&ks->counter[CNT_PASS2])) {
-        __shared__ double tot[NK];
-        reduce_blocks(partial, gridDim.x, kMaxBasis, NK, tot);
-        for (int k = threadIdx.x; k < NK; k += blockDim.x) {
-            const double hk = ks->sigma[k] * tot[k];
-            ks->h2[k] = hk;
-            ks->c2[k] = ks->sigma[k] * hk;
-        }
-        if (threadIdx.x == 0) ks->counter[CNT_PASS2] = 0;
-    }
+    block_columns<float, NK>(part, NK, wsum, pass_sums(partial, gridDim.x, 1) + blockIdx.x, gridDim.x);
 }
 
 template <int NK>
@@ -220,10 +196,8 @@ f32_pass3_kernel(const DevArgs* __restrict__ a, KState* ks, float* __restrict__ 
     __shared__ float cf[NK];
     __shared__ float scratch[kWarps];
     __shared__ float red[1];
-    const int over = ks->cycle_over;
-    for (int k = threadIdx.x; k < NK; k += blockDim.x) cf[k] = (float)ks->c2[k];
-    if (over) return;
-    __syncthreads();
+    if (ks->cycle_over) return;
+    pass_coefficients<float>(pass_sums(partial, gridDim.x, 1), NK, ks, ks->h2, cf);
     int lo, hi;
     block_rows(a->n, gridDim.x, blockIdx.x, lo, hi);
     float part[NK];

@@ -11,7 +11,7 @@
 //   K7b w -= V_j h2, v_{j+1} = w (unnormalised), ||w||^2; the last block then
 //       forms the Hessenberg column h1 + h2, applies the Givens rotations,
 //       updates the residual estimate and decides whether the cycle ends.
-// Reductions end in a deterministic last-block pass.  On this GPU a
+// Reductions are deterministic (blocks in order; see pass_coefficients).  On this GPU a
 // warp-wide FP64 instruction occupies a sub-partition's FP64 unit for many
 // cycles, so the CGS kernels are specialised on the exact number of basis
 // columns and issue exactly the algorithmic count of FP64 operations.
@@ -29,6 +29,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "resident.cuh"
 
 namespace sa {
 
@@ -133,7 +134,7 @@ gmres_start_kernel(const DevArgs* __restrict__ a, KState* ks, typename Sys::T* V
 // the upper one padded with zeros past column K - 1.
 template <typename T, int K>
 __device__ __forceinline__ void block_columns(T (&part)[K], int nk, T* wsum /* kWarps * K */,
-                                              T* out /* global, K */) {
+                                              T* out /* global */, int stride) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if constexpr (K <= 32 && (K & (K - 1)) == 0) {
         const T c = warp_reduce_scatter<T, K>(part);
@@ -162,8 +163,47 @@ __device__ __forceinline__ void block_columns(T (&part)[K], int nk, T* wsum /* k
     for (int k = threadIdx.x; k < nk; k += blockDim.x) {
         T s = wsum[k];
         for (int w = 1; w < kWarps; ++w) s += wsum[w * K + k];
-        out[k] = s;
+        out[(size_t)k * stride] = s;
     }
+}
+
+// The CGS passes leave their block sums in global memory (column k of block b at
+// sums[k * nblk + b]; first and second pass in turn), and the kernel that needs the
+// coefficients adds them up itself, every block all of them while its own loads
+// of the basis start: the counter, fence and last-block pass that did it at the
+// end of the producing kernel kept the whole grid waiting (about 3 us of every
+// kernel, against 1 us here).  h_k = sigma_k (V_stored^T w)_k, cf_k = sigma_k h_k.
+template <typename T>
+__device__ __forceinline__ T* pass_sums(T* partial, int nblk, int pass) {
+    return partial + (size_t)(1 + pass * kMaxBasis) * nblk;
+}
+template <typename T>
+__device__ __forceinline__ void pass_coefficients(const T* sums, int nk, const KState* ks,
+                                                  double* h_out, T* cf) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int nblk = gridDim.x;
+    constexpr int kMany = 2;
+    for (int k0 = warp; k0 < nk; k0 += kMany * nw) {
+        T u[kMany][kTeamMax / 32];
+#pragma unroll
+        for (int f = 0; f < kMany; ++f)
+#pragma unroll
+            for (int q = 0; q < kTeamMax / 32; ++q)
+                u[f][q] = k0 + f * nw < nk && lane + 32 * q < nblk
+                              ? __ldcg(sums + (size_t)(k0 + f * nw) * nblk + lane + 32 * q) : (T)0;
+#pragma unroll
+        for (int f = 0; f < kMany; ++f) {
+            const int k = k0 + f * nw;
+            if (k >= nk) break;
+            const double t = (double)warp_total(u[f]);
+            if (lane == 0) {
+                const double sg = ks->sigma[k], hk = sg * t;
+                cf[k] = (T)(sg * hk);
+                if (blockIdx.x == 0) h_out[k] = hk;
+            }
+        }
+    }
+    __syncthreads();
 }
 
 // ---------------------------------------------------------------------------
@@ -543,8 +583,7 @@ template <class Sys>
 __global__ void __launch_bounds__(kDotBlock, 1)
 arnoldi_dot_kernel(const DevArgs* __restrict__ a, KState* ks,
                    const typename Sys::T* __restrict__ V, size_t ldv,
-                   const typename Sys::T* __restrict__ w, typename Sys::T* partial, int j,
-                   int stride) {
+                   const typename Sys::T* __restrict__ w, typename Sys::T* partial, int j) {
     using T = typename Sys::T;
     if (ks->cycle_over) return;
     __shared__ T segsum[kMaxBasis * kDotWarps];
@@ -579,17 +618,8 @@ arnoldi_dot_kernel(const DevArgs* __restrict__ a, KState* ks,
         colsum[k] = t;
     }
     __syncthreads();
-    for (int k = threadIdx.x; k < nk; k += blockDim.x) partial[(size_t)blockIdx.x * stride + k] = colsum[k];
-    if (last_block_arrive(&ks->counter[CNT_DOT])) {
-        __shared__ double tot[kMaxBasis];
-        reduce_blocks(partial, gridDim.x, stride, nk, tot);
-        for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-            const double hk = ks->sigma[k] * tot[k];
-            ks->h1[k] = hk;
-            ks->c1[k] = ks->sigma[k] * hk;
-        }
-        if (threadIdx.x == 0) ks->counter[CNT_DOT] = 0;
-    }
+    T* const sums = pass_sums(partial, gridDim.x, 0) + blockIdx.x;
+    for (int k = threadIdx.x; k < nk; k += blockDim.x) sums[(size_t)k * gridDim.x] = colsum[k];
 }
 
 // K7a: w -= V_stored c1; h2 = sigma_k (V_stored^T w)_k.  NK (the number of
@@ -610,8 +640,7 @@ arnoldi_pass2_kernel(const DevArgs* __restrict__ a, KState* ks,
     __shared__ T wsum[kWarps * NK];
     const int n = a->n;
     const int nk = NK;
-    for (int k = threadIdx.x; k < NK; k += blockDim.x) cf[k] = (T)ks->c1[k];
-    __syncthreads();
+    pass_coefficients<T>(pass_sums(partial, gridDim.x, 0), NK, ks, ks->h1, cf);
     int lo, hi;
     block_rows(n, gridDim.x, blockIdx.x, lo, hi);
     T part[NK];
@@ -644,17 +673,7 @@ arnoldi_pass2_kernel(const DevArgs* __restrict__ a, KState* ks,
             }
         }
     }
-    block_columns<T, NK>(part, nk, wsum, partial + (size_t)blockIdx.x * kMaxBasis);
-    if (last_block_arrive(&ks->counter[CNT_PASS2])) {
-        __shared__ double tot[NK];
-        reduce_blocks(partial, gridDim.x, kMaxBasis, nk, tot);
-        for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-            const double hk = ks->sigma[k] * tot[k];
-            ks->h2[k] = hk;
-            ks->c2[k] = ks->sigma[k] * hk;
-        }
-        if (threadIdx.x == 0) ks->counter[CNT_PASS2] = 0;
-    }
+    block_columns<T, NK>(part, nk, wsum, pass_sums(partial, gridDim.x, 1) + blockIdx.x, gridDim.x);
 }
 
 // K5b' (nk > kDotWarps): the same h1 = sigma_k (V_stored^T w)_k, row-parallel
@@ -687,17 +706,7 @@ arnoldi_dot_rows_kernel(const DevArgs* __restrict__ a, KState* ks,
 #pragma unroll
         for (int k = 0; k < NK; ++k) part[k] = fma(vv[k], wi, part[k]);
     }
-    block_columns<T, NK>(part, NK, wsum, partial + (size_t)blockIdx.x * kMaxBasis);
-    if (last_block_arrive(&ks->counter[CNT_DOT])) {
-        __shared__ double tot[NK];
-        reduce_blocks(partial, gridDim.x, kMaxBasis, NK, tot);
-        for (int k = threadIdx.x; k < NK; k += blockDim.x) {
-            const double hk = ks->sigma[k] * tot[k];
-            ks->h1[k] = hk;
-            ks->c1[k] = ks->sigma[k] * hk;
-        }
-        if (threadIdx.x == 0) ks->counter[CNT_DOT] = 0;
-    }
+    block_columns<T, NK>(part, NK, wsum, pass_sums(partial, gridDim.x, 0) + blockIdx.x, gridDim.x);
 }
 
 // Last block of K7b, all threads: Hessenberg column j = h1 + h2 with
@@ -766,8 +775,10 @@ __device__ inline void arnoldi_finish(KState* ks, const DevArgs* a, int j, int R
     if (tid == 0) {
         const double hn = hn_s, hh = hh_s;
         hc[j + 1] = hn;
-        const double av = hc[j], bv = hn;
-        const double rr = hypot(av, bv);
+        // hypot without its scaling where the squares are in range (its FP64
+        // instructions are a microsecond of this serial part).
+        const double av = hc[j], bv = hn, sq = fma(av, av, bv * bv);
+        const double rr = sq > 1e-200 && sq < 1e200 ? sqrt(sq) : hypot(av, bv);
         double c = 1.0, sv = 0.0;
         if (rr != 0.0) {
             const double rinv = 1.0 / rr;
@@ -866,8 +877,7 @@ arnoldi_pass3_kernel(const DevArgs* __restrict__ a, KState* ks, typename Sys::T*
     __shared__ T scratch[kWarps];
     __shared__ T red[1];
     const int n = a->n;
-    for (int k = threadIdx.x; k < NK; k += blockDim.x) cf[k] = (T)ks->c2[k];
-    __syncthreads();
+    pass_coefficients<T>(pass_sums(partial, gridDim.x, 1), NK, ks, ks->h2, cf);
     T* vout = V + (size_t)(j + 1) * ldv;
     int lo, hi;
     block_rows(n, gridDim.x, blockIdx.x, lo, hi);
@@ -1025,7 +1035,7 @@ static void launch_step(const DevArgs* a, KState* ks, typename Sys::T* V, size_t
         if constexpr (NK >= kDotRowsMin)
             arnoldi_dot_rows_kernel<Sys, NK><<<nblk, kStreamBlock, 0, st>>>(a, ks, V, ldv, w, partial, j);
         else
-            arnoldi_dot_kernel<Sys><<<nblk, kDotBlock, 0, st>>>(a, ks, V, ldv, w, partial, j, kMaxBasis);
+            arnoldi_dot_kernel<Sys><<<nblk, kDotBlock, 0, st>>>(a, ks, V, ldv, w, partial, j);
         mark(ev, k, st);
         arnoldi_pass2_kernel<Sys, NK><<<nblk, kStreamBlock, 0, st>>>(a, ks, V, ldv, w, partial, j);
         mark(ev, k, st);
