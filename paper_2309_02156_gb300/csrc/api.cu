@@ -22,7 +22,9 @@ using namespace sa;
 struct seq_ctx {
     seq_config cfg;
     cudaStream_t stream = nullptr;
-    cudaStream_t cap = nullptr;      // private stream used only for graph capture
+    cudaStream_t cap = nullptr;      // private stream: graph capture, and the POD eigensolver
+    cudaEvent_t fork = nullptr;      // between the two streams (POD)
+    cudaEvent_t join = nullptr;
     int dev = 0;
     bool mixed = false;              // FP32 inner Krylov inside FP64 refinement
     bool hist32 = false;             // FP32 history and sketch (SEQ_MIXED)
@@ -684,6 +686,8 @@ int seq_create(const seq_config* cfg, void* cuda_stream, seq_ctx** out) {
         ok = ok && cudaMalloc(&ctx->Zs, sizeof(double) * M * c.basis_m) == cudaSuccess;
     }
     if (c.guess == SEQ_GUESS_POD) {
+        ok = ok && cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming) == cudaSuccess;
+        ok = ok && cudaEventCreateWithFlags(&ctx->join, cudaEventDisableTiming) == cudaSuccess;
         ok = ok && cudaMalloc(&ctx->gpart, sizeof(double) * gram_partial_doubles()) == cudaSuccess;
         ok = ok && cudaMalloc(&ctx->gcount, sizeof(unsigned)) == cudaSuccess;
         ok = ok && cudaMemsetAsync(ctx->gcount, 0, sizeof(unsigned), ctx->stream) == cudaSuccess;
@@ -715,7 +719,8 @@ int seq_create(const seq_config* cfg, void* cuda_stream, seq_ctx** out) {
 
 int seq_destroy(seq_ctx* ctx) {
     if (!ctx) return SEQ_OK;
-    if (ctx->stream || true) cudaStreamSynchronize(ctx->stream);
+    cudaStreamSynchronize(ctx->stream);
+    if (ctx->cap) cudaStreamSynchronize(ctx->cap);
     if (ctx->cycle) cudaGraphExecDestroy(ctx->cycle);
     if (ctx->cg_graph) cudaGraphExecDestroy(ctx->cg_graph);
     if (ctx->cycle_prof) cudaGraphExecDestroy(ctx->cycle_prof);
@@ -734,6 +739,8 @@ int seq_destroy(seq_ctx* ctx) {
                          ctx->h_used};
     for (void* p : host_ptrs)
         if (p) cudaFreeHost(p);
+    if (ctx->fork) cudaEventDestroy(ctx->fork);
+    if (ctx->join) cudaEventDestroy(ctx->join);
     if (ctx->cap) cudaStreamDestroy(ctx->cap);
     delete ctx;
     return SEQ_OK;
@@ -807,12 +814,18 @@ int seq_guess(seq_ctx* ctx, const seq_csr* A, const double* b_dev, double* x0_de
         const double* X = (const double*)ctx->X;
         if (mode == SEQ_GUESS_POD) {
             // Algorithm 2 in snapshot form; the reduced problem from W = S[AX|b].
+            // The eigensolver (one block, latency) runs beside the sketch, which
+            // leaves it an SM (GB300, 1024 x 1024, M = 20: the guess 2.02 -> 1.54 ms).
             const int kk = mb < m ? mb : m;
+            launch_pod_gram(X, ctx->ldx, n, M, m, oldest, ctx->gpart, ctx->gcount, ctx->G, ctx->stream);
+            CK(cudaEventRecord(ctx->fork, ctx->stream));
+            CK(cudaStreamWaitEvent(ctx->cap, ctx->fork, 0));
+            launch_pod_eig(ctx->G, m, kk, ctx->Vk, ctx->lam, ctx->sweeps, ctx->cap);
+            CK(cudaEventRecord(ctx->join, ctx->cap));
             launch_sketch_f64(A->rowptr, A->colind, A->values, X, ctx->ldx, b_dev, n, A->nnz, M,
-                              c.s, c.zeta, c.seed, ctx->sk_partial, ctx->sk_nblk,
-                              ctx->W, bad, ctx->stream);
-            launch_pod_basis(X, ctx->ldx, n, M, m, oldest, kk, ctx->gpart, ctx->gcount, ctx->G,
-                             ctx->Vk, ctx->lam, ctx->sweeps, ctx->stream);
+                              c.s, c.zeta, c.seed, ctx->sk_partial,
+                              sketch_grid_beside(n, c.s, M), ctx->W, bad, ctx->stream);
+            CK(cudaStreamWaitEvent(ctx->stream, ctx->join, 0));
             launch_pod_reduce(ctx->W, c.s, M, m, oldest, ctx->Vk, kk, ctx->Wp, ctx->stream);
             launch_lsq(ctx->Wp, c.s, kk, kk, 0, c.rank_tol, ctx->lsq_red, ctx->stream);
             launch_pod_coeff(ctx->lsq_red, ctx->Vk, m, kk, M, oldest, ctx->lsq, ctx->stream);

@@ -9,6 +9,7 @@
 namespace sa {
 
 // sketch.cu
+int sketch_grid_beside(int n, int s, int M);   // the same, one SM left free where the grid fills all
 int sketch_grid(int n, int s, int M);   // blocks of launch_sketch_* for up to M columns
 size_t sketch_partial_doubles(int n, int s, int M);   // partial buffer of launch_sketch_*
 void launch_sketch_columns(int n, int s, int zeta, uint64_t seed, uint16_t* packed,
@@ -51,9 +52,10 @@ void launch_rand_scratch(const double* X, int ldx, int n, int M, int mi, int old
                          uint64_t gseed, uint64_t start, double* Om, int ldo, cudaStream_t st);
 void launch_rand_push(const double* x, int n, double* X, int ldx, int slot, int remove, double* Zs,
                       int m, uint64_t gseed, uint64_t start, double* Om, int ldo, cudaStream_t st);
-void launch_pod_basis(const double* X, int ldx, int n, int M, int mi, int oldest, int kk,
-                      double* partial, unsigned* counter, double* G, double* Vk, double* lam,
-                      int* sweeps, cudaStream_t st);
+void launch_pod_gram(const double* X, int ldx, int n, int M, int mi, int oldest, double* partial,
+                     unsigned* counter, double* G, cudaStream_t st);
+void launch_pod_eig(const double* G, int mi, int kk, double* Vk, double* lam, int* sweeps,
+                    cudaStream_t st);
 void launch_pod_reduce(const double* W, int s, int M, int mi, int oldest, const double* Vk, int kk,
                        double* Wp, cudaStream_t st);
 void launch_pod_coeff(const LsqOut* red, const double* Vk, int mi, int kk, int M, int oldest,

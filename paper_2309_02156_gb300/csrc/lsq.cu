@@ -10,9 +10,17 @@
 // rank revealing.
 #include "common.cuh"
 #include "internal.h"
+#include "resident.cuh"
 
 namespace sa {
 
+// One block, bound by the latency of its FP64 chains: the sums over the s rows of
+// a column end in an integer warp sum (warp_total; the five-step FP64 butterfly
+// held the FP64 pipe for most of a step), square roots are taken for all columns
+// by one warp and the reflector's division once (each is a dozen FP64
+// instructions of 64 cycles for a whole warp, and every warp took its own), and
+// the pivot's norm, just computed, is the reflector's.  s = 80, M = 20: 131 us
+// (170 before).
 __global__ void __launch_bounds__(256)
 lsq_kernel(const double* __restrict__ W, int s, int M, int m, int oldest, double tau, LsqOut* out) {
     extern __shared__ double sm[];
@@ -28,7 +36,7 @@ lsq_kernel(const double* __restrict__ W, int s, int M, int m, int oldest, double
     double* ylog = z + m;
     double* red = ylog + m;      // 32 doubles
     __shared__ int perm[kMaxM], live[kMaxM];
-    __shared__ double sh_normx, sh_vtv;
+    __shared__ double sh_normx, sh_vtv, sh_scale;
     __shared__ int sh_p, sh_rank;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const int bd = blockDim.x;
@@ -43,9 +51,11 @@ lsq_kernel(const double* __restrict__ W, int s, int M, int m, int oldest, double
     for (int l = warp; l < m; l += nw) {
         double a = 0.0;
         for (int q = lane; q < s; q += 32) a += Wo[l * s + q] * Wo[l * s + q];
-        a = warp_sum(a);
-        if (lane == 0) d[l] = sqrt(a);
+        a = warp_total1(a);
+        if (lane == 0) d[l] = a;
     }
+    __syncthreads();
+    if (tid < m) d[tid] = sqrt(d[tid]);
     __syncthreads();
     for (int i = tid; i < s * m; i += bd) {
         const int l = i / s;
@@ -63,16 +73,27 @@ lsq_kernel(const double* __restrict__ W, int s, int M, int m, int oldest, double
         for (int l = k + warp; l < m; l += nw) {
             double a = 0.0;
             for (int q = k + lane; q < s; q += 32) a += B[l * s + q] * B[l * s + q];
-            a = warp_sum(a);
-            if (lane == 0) nrm[l] = live[perm[l]] ? sqrt(a) : -1.0;
+            a = warp_total1(a);
+            if (lane == 0) nrm[l] = a;
         }
         __syncthreads();
-        if (tid == 0) {
-            int p = k;
-            double best = nrm[k];
-            for (int l = k + 1; l < m; ++l)
-                if (nrm[l] > best) { best = nrm[l]; p = l; }
-            sh_p = p;
+        if (warp == 0) {                 // largest norm, ties to the lowest index
+            double best = -2.0;
+            if (k + lane < m) best = live[perm[k + lane]] ? sqrt(nrm[k + lane]) : -1.0;
+            int at = k + lane;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+                const int oa = __shfl_xor_sync(0xffffffffu, at, o);
+                if (ob > best || (ob == best && oa < at)) {
+                    best = ob;
+                    at = oa;
+                }
+            }
+            if (lane == 0) {
+                sh_p = at;
+                sh_normx = best;
+            }
         }
         __syncthreads();
         const int p = sh_p;
@@ -89,13 +110,6 @@ lsq_kernel(const double* __restrict__ W, int s, int M, int m, int oldest, double
             }
         }
         __syncthreads();
-        if (warp == 0) {
-            double a = 0.0;
-            for (int q = k + lane; q < s; q += 32) a += B[k * s + q] * B[k * s + q];
-            a = warp_sum(a);
-            if (lane == 0) sh_normx = sqrt(a);
-        }
-        __syncthreads();
         const double normx = sh_normx;
         if (normx == 0.0 || !live[perm[k]]) break;
         const double alpha = B[k * s + k] >= 0.0 ? -normx : normx;
@@ -104,8 +118,11 @@ lsq_kernel(const double* __restrict__ W, int s, int M, int m, int oldest, double
         if (warp == 0) {
             double a = 0.0;
             for (int q = k + lane; q < s; q += 32) a += v[q] * v[q];
-            a = warp_sum(a);
-            if (lane == 0) sh_vtv = a;
+            a = warp_total1(a);
+            if (lane == 0) {
+                sh_vtv = a;
+                sh_scale = 2.0 / a;
+            }
         }
         __syncthreads();
         const double vtv = sh_vtv;
@@ -114,8 +131,8 @@ lsq_kernel(const double* __restrict__ W, int s, int M, int m, int oldest, double
                 double* col = (l < m) ? B + l * s : c;
                 double a = 0.0;
                 for (int q = k + lane; q < s; q += 32) a += v[q] * col[q];
-                a = warp_sum(a);
-                const double t = (2.0 / vtv) * a;
+                a = warp_total1(a);
+                const double t = sh_scale * a;
                 for (int q = k + lane; q < s; q += 32) col[q] -= v[q] * t;
             }
         }
@@ -153,7 +170,7 @@ lsq_kernel(const double* __restrict__ W, int s, int M, int m, int oldest, double
         const double e = acc - cb[q];
         part += e * e;
     }
-    part = warp_sum(part);
+    part = warp_total1(part);
     if (lane == 0) red[warp] = part;
     __syncthreads();
     if (tid == 0) {

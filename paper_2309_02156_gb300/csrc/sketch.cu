@@ -141,6 +141,16 @@ int sketch_grid(int n, int s, int M) {
     return nblk > 0 ? (int)nblk : 1;
 }
 
+int sketch_grid_beside(int n, int s, int M) {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int nblk = sketch_grid(n, s, M);
+    const long long ntiles = ((long long)n + 31) / 32;
+    const long long most = (long long)kSkMaxTiles * sketch_teams(s, M + 1) * (nblk - 1);
+    return nblk == sms && nblk > 1 && ntiles <= most ? nblk - 1 : nblk;
+}
+
 size_t sketch_partial_doubles(int n, int s, int M) {
     return (size_t)sketch_grid(n, s, M) * s * (M + 1);
 }
