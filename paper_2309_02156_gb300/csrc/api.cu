@@ -412,7 +412,7 @@ void account_cycle(seq_ctx* ctx, bool f32, int jd, bool updated, int nnz) {
         if (updated) add_stat(ctx, SEQ_K_UPDATE, u, E * n * (jd + 2), 2.0 * n * jd);
         u += 1;
     }
-    add_stat(ctx, SEQ_K_RESTART, u, csr + 3.0 * E * n, 2.0 * nnz + 4.0 * n);
+    add_stat(ctx, SEQ_K_RESTART, u, spmv_mat + 3.0 * E * n, 2.0 * nnz + 4.0 * n);
 }
 
 // One restarted GMRES solve on the system bound to (args, ks); `f32` selects

@@ -156,6 +156,7 @@ gram_kernel(const double* __restrict__ X, int ldx, int n, int M, int mi, int old
     if (last_block_arrive(counter)) {
         for (int p = tid; p < npairs; p += kGramThreads) {
             double s = 0.0;
+#pragma unroll 16
             for (int blk = 0; blk < (int)gridDim.x; ++blk) s += partial[(size_t)blk * kMaxPairs + p];
             int a = 0, q = p;
             while (q >= mi - a) {

@@ -452,8 +452,8 @@ __device__ __forceinline__ void batch_product(const BatchSeq& q, const float* x,
 // This step's values (FP32) into the copy of the pattern, rows [r_lo, r_hi).
 __device__ __forceinline__ void refresh_values(const BatchSeq& q, int r_lo, int r_hi) {
     for (int i = r_lo + threadIdx.x; i < r_hi; i += blockDim.x) {
-        int e = q.rowptr[i];
-        const int e1 = q.rowptr[i + 1], lane = i & 31;
+        int e = max(0, min(q.rowptr[i], q.nnz));        // the clamped range the copy was made of
+        const int e1 = max(e, min(q.rowptr[i + 1], q.nnz)), lane = i & 31;
         if (q.slot) {
             const int2* m = q.slot + (i >> 5) * q.slot_w;
             float* dst = q.sval + (i >> 5) * q.slot_w * 32 + lane;

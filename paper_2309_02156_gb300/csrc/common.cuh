@@ -166,7 +166,8 @@ template <typename T>
 __device__ __forceinline__ T sum_over_blocks(const T* partial, int nblk, int stride, int k) {
     T a0 = 0, a1 = 0, a2 = 0, a3 = 0;
     int b = 0;
-    for (; b + 3 < nblk; b += 4) {
+#pragma unroll 8
+    for (; b + 3 < nblk; b += 4) {       // 32 loads in flight, same order
         a0 += __ldcg(partial + (size_t)(b + 0) * stride + k);
         a1 += __ldcg(partial + (size_t)(b + 1) * stride + k);
         a2 += __ldcg(partial + (size_t)(b + 2) * stride + k);

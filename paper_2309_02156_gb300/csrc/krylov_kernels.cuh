@@ -55,79 +55,6 @@ constexpr int kWarps = kStreamBlock / 32;
 constexpr int kTile = kTileStage;              // pipelined tiles: (value, x) staging
 constexpr int kTileP = kTileChunks * 32;       // single-stage tiles: product staging
 
-// ---------------------------------------------------------------------------
-// Cycle start: r = rhs - A x written to basis column 0, beta = ||r||.  With
-// first != 0 the solve is initialised (||rhs||, target, iteration count; the
-// FP32 inner solve also zeroes d, so r = rhs).
-template <class Sys>
-__global__ void __launch_bounds__(kStreamBlock, 1)
-gmres_start_kernel(const DevArgs* __restrict__ a, KState* ks, typename Sys::T* V,
-                   typename Sys::T* partial, int first) {
-    using T = typename Sys::T;
-    if (!first && ks->finished) return;
-    __shared__ T sprod[kWarps * kTileP];
-    __shared__ T scratch[kWarps * 2];
-    __shared__ T red[2];
-    const int n = a->n, nnz = a->nnz;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    T* x = Sys::x(a);
-    const T* rhs = Sys::rhs(a);
-    const bool zero_x = first && (sizeof(T) == 4);
-    int lo, hi;
-    block_rows(n, gridDim.x, blockIdx.x, lo, hi);
-    T acc[2] = {0, 0};
-    for (int r0 = lo + warp * 32; r0 < hi; r0 += kWarps * 32) {
-        T ax = 0;
-        if (!zero_x)
-            ax = warp_tile_spmv<T>(a->rowptr, a->colind, Sys::val(a), x, n, nnz, r0,
-                                   sprod + warp * kTileP, &ks->bad_index);
-        const int row = r0 + lane;
-        if (row < n) {
-            const T bi = rhs[row];
-            const T r = bi - ax;
-            V[row] = r;
-            if (zero_x) x[row] = 0;
-            acc[0] += r * r;
-            acc[1] += bi * bi;
-        }
-    }
-    block_sum<T, 2>(acc, 2, red, scratch);
-    if (threadIdx.x < 2) partial[blockIdx.x * 2 + threadIdx.x] = red[threadIdx.x];
-    if (last_block_arrive(&ks->counter[CNT_START])) {
-        __shared__ double tot[2];
-        reduce_blocks(partial, gridDim.x, 2, 2, tot);
-        if (threadIdx.x == 0) {
-            const double beta = sqrt(tot[0]);
-            if (first) {
-                ks->bnorm = sqrt(tot[1]);
-                ks->target = a->tol * ks->bnorm;
-                ks->iters = 0;
-                ks->status = ST_OK;
-                ks->first_relres = rel_residual(beta, ks->bnorm);
-            }
-            ks->last_jdone = first ? 0 : ks->jdone;
-            ks->beta = beta;
-            ks->g[0] = beta;
-            ks->sigma[0] = beta > 0.0 ? 1.0 / beta : 0.0;
-            ks->jdone = 0;
-            ks->cycle_over = 0;
-            ks->finished = 0;
-            if (!isfinite(beta)) {
-                ks->status = ST_NONFINITE;
-                ks->finished = 1;
-            } else if (beta <= ks->target) {
-                ks->status = ST_OK;
-                ks->finished = 1;
-            } else if (ks->iters >= a->max_iters) {
-                ks->status = ST_NOT_CONVERGED;
-                ks->finished = 1;
-            }
-            if (ks->finished) ks->cycle_over = 1;
-            ks->counter[CNT_START] = 0;
-        }
-    }
-}
-
 // Lane l of every warp holds, for K <= 32, the warp partial of column l % K
 // after warp_reduce_scatter; the block partial of column k (k < nk) is the
 // sum over warps in warp order.  32 < K <= 64 is handled as two halves of 32,
@@ -525,28 +452,16 @@ __device__ __forceinline__ bool copy_rows(const DevArgs* __restrict__ a, const T
     return false;
 }
 
-template <class Sys>
-__global__ void __launch_bounds__(kSpmvBlock, 1)
-arnoldi_spmv_kernel(const DevArgs* __restrict__ a, const KState* __restrict__ ks,
-                    const typename Sys::T* __restrict__ V, size_t ldv,
-                    typename Sys::T* __restrict__ w, int j, const typename Sys::T* src) {
-    using T = typename Sys::T;
-    if (ks->cycle_over) return;
-    extern __shared__ unsigned char dsm[];
-    T* sprod = reinterpret_cast<T*>(dsm);                   // kSpmvWarps * kTile
+// (A x)_row for the rows [lo, hi) of the CSR arrays by software-pipelined warp
+// tiles (the row range of tile k + 2, the loads of tile k + 1 and the gathers of
+// tile k in flight together); sprod: kTile entries per warp.
+template <typename T, typename F>
+__device__ __forceinline__ void csr_tile_rows(const DevArgs* __restrict__ a,
+                                              const T* __restrict__ val, const T* x, int lo, int hi,
+                                              int nwarps, T* sprod, int* bad, const F& f) {
     const int n = a->n, nnz = a->nnz;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // w = A v_j, v_j = sigma_j times the stored column, or (right
-    // preconditioning) w = A z with z = M^{-1} v_j already formed in src.
-    const T sig = src ? (T)1 : (T)ks->sigma[j];
-    const T* vj = src ? src : V + (size_t)j * ldv;
-    const T* val = Sys::val(a);
-    int lo, hi;
-    block_rows(n, gridDim.x, blockIdx.x, lo, hi);
-    if (copy_rows<T>(a, vj, lo, hi, kSpmvWarps, const_cast<int*>(&ks->bad_index),
-                     ScaleEpi<T>{w, sig}))
-        return;
-    const int step = kSpmvWarps * 32;
+    const int step = nwarps * 32;
     int r0 = lo + warp * 32;
     TileRows ta = tile_rows(a->rowptr, n, nnz, r0, hi);
     TileRows tb = tile_rows(a->rowptr, n, nnz, r0 + step, hi);
@@ -557,14 +472,129 @@ arnoldi_spmv_kernel(const DevArgs* __restrict__ a, const KState* __restrict__ ks
         const TileRows tc = tile_rows(a->rowptr, n, nnz, r0 + 2 * step, hi);
         tile_span(tb, n, r0 + step);
         if (r0 + step < hi) tile_load(a->colind, val, tb, db);
-        const T ax = tile_finish<T>(a->colind, val, vj, n, ta, da, sprod + warp * kTile,
-                                    const_cast<int*>(&ks->bad_index));
-        const int row = r0 + lane;
-        if (row < hi) w[row] = ax * sig;
+        const T ax = tile_finish<T>(a->colind, val, x, n, ta, da, sprod + warp * kTile, bad);
+        if (r0 + lane < hi) f(r0 + lane, ax);
         ta = tb;
         da = db;
         tb = tc;
     }
+}
+
+// ---------------------------------------------------------------------------
+// Cycle start: r = rhs - A x written to basis column 0 (from the copy of the
+// matrix when there is one: 17 us at 1,048,576 rows in FP32, about 75 before),
+// beta = ||r||.  With
+// first != 0 the solve is initialised (||rhs||, target, iteration count; the
+// FP32 inner solve also zeroes d, so r = rhs).
+template <typename T>
+struct StartEpi {                    // v[i] = rhs[i] - (A x)[i], its and rhs' squares
+    T* v;
+    const T* rhs;
+    T* acc;
+    static constexpr int kSlices = 0;
+    struct Pre { T b; };
+    __device__ Pre pre(int i) const { return {rhs[i]}; }
+    __device__ void operator()(int i, T ax, const Pre& o) const {
+        const T r = o.b - ax;
+        v[i] = r;
+        acc[0] = fma(r, r, acc[0]);
+        acc[1] = fma(o.b, o.b, acc[1]);
+    }
+};
+
+template <class Sys>
+__global__ void __launch_bounds__(kStreamBlock, 1)
+gmres_start_kernel(const DevArgs* __restrict__ a, KState* ks, typename Sys::T* V,
+                   typename Sys::T* partial, int first) {
+    using T = typename Sys::T;
+    if (!first && ks->finished) return;
+    __shared__ T sprod[kWarps * kTileP];
+    __shared__ T scratch[kWarps * 2];
+    __shared__ T red[2];
+    const int n = a->n, nnz = a->nnz;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T* x = Sys::x(a);
+    const T* rhs = Sys::rhs(a);
+    const bool zero_x = first && (sizeof(T) == 4);
+    int lo, hi;
+    block_rows(n, gridDim.x, blockIdx.x, lo, hi);
+    T acc[2] = {0, 0};
+    const bool copied = !zero_x && copy_rows<T>(a, x, lo, hi, kWarps, &ks->bad_index,
+                                                StartEpi<T>{V, rhs, acc});
+    for (int r0 = lo + warp * 32; !copied && r0 < hi; r0 += kWarps * 32) {
+        T ax = 0;
+        if (!zero_x)
+            ax = warp_tile_spmv<T>(a->rowptr, a->colind, Sys::val(a), x, n, nnz, r0,
+                                   sprod + warp * kTileP, &ks->bad_index);
+        const int row = r0 + lane;
+        if (row < n) {
+            const T bi = rhs[row];
+            const T r = bi - ax;
+            V[row] = r;
+            if (zero_x) x[row] = 0;
+            acc[0] += r * r;
+            acc[1] += bi * bi;
+        }
+    }
+    block_sum<T, 2>(acc, 2, red, scratch);
+    if (threadIdx.x < 2) partial[blockIdx.x * 2 + threadIdx.x] = red[threadIdx.x];
+    if (last_block_arrive(&ks->counter[CNT_START])) {
+        __shared__ double tot[2];
+        reduce_blocks(partial, gridDim.x, 2, 2, tot);
+        if (threadIdx.x == 0) {
+            const double beta = sqrt(tot[0]);
+            if (first) {
+                ks->bnorm = sqrt(tot[1]);
+                ks->target = a->tol * ks->bnorm;
+                ks->iters = 0;
+                ks->status = ST_OK;
+                ks->first_relres = rel_residual(beta, ks->bnorm);
+            }
+            ks->last_jdone = first ? 0 : ks->jdone;
+            ks->beta = beta;
+            ks->g[0] = beta;
+            ks->sigma[0] = beta > 0.0 ? 1.0 / beta : 0.0;
+            ks->jdone = 0;
+            ks->cycle_over = 0;
+            ks->finished = 0;
+            if (!isfinite(beta)) {
+                ks->status = ST_NONFINITE;
+                ks->finished = 1;
+            } else if (beta <= ks->target) {
+                ks->status = ST_OK;
+                ks->finished = 1;
+            } else if (ks->iters >= a->max_iters) {
+                ks->status = ST_NOT_CONVERGED;
+                ks->finished = 1;
+            }
+            if (ks->finished) ks->cycle_over = 1;
+            ks->counter[CNT_START] = 0;
+        }
+    }
+}
+
+template <class Sys>
+__global__ void __launch_bounds__(kSpmvBlock, 1)
+arnoldi_spmv_kernel(const DevArgs* __restrict__ a, const KState* __restrict__ ks,
+                    const typename Sys::T* __restrict__ V, size_t ldv,
+                    typename Sys::T* __restrict__ w, int j, const typename Sys::T* src) {
+    using T = typename Sys::T;
+    if (ks->cycle_over) return;
+    extern __shared__ unsigned char dsm[];
+    T* sprod = reinterpret_cast<T*>(dsm);                   // kSpmvWarps * kTile
+    const int n = a->n;
+    // w = A v_j, v_j = sigma_j times the stored column, or (right
+    // preconditioning) w = A z with z = M^{-1} v_j already formed in src.
+    const T sig = src ? (T)1 : (T)ks->sigma[j];
+    const T* vj = src ? src : V + (size_t)j * ldv;
+    const T* val = Sys::val(a);
+    int lo, hi;
+    block_rows(n, gridDim.x, blockIdx.x, lo, hi);
+    if (copy_rows<T>(a, vj, lo, hi, kSpmvWarps, const_cast<int*>(&ks->bad_index),
+                     ScaleEpi<T>{w, sig}))
+        return;
+    csr_tile_rows<T>(a, val, vj, lo, hi, kSpmvWarps, sprod, const_cast<int*>(&ks->bad_index),
+                     [&](int row, T ax) { w[row] = ax * sig; });
 }
 
 // K5b: h1 = sigma_k (V_stored^T w)_k for k <= j.  Work items (column k, row
