@@ -556,10 +556,10 @@ int run_cg(seq_ctx* ctx, bool f32) {
     if (ctx->sell_ok && ctx->plan.W) {
         cudaError_t e = cudaSuccess;
         const bool taken =
-            f32 ? launch_resident_cg_f32(args, ks, (float*)ctx->r, (float*)ctx->q, ctx->team, n,
-                                         ctx->plan.W, ctx->plan.reach, ctx->stream, &e)
-                : launch_resident_cg_f64(args, ks, (double*)ctx->r, (double*)ctx->q, ctx->team, n,
-                                         ctx->plan.W, ctx->plan.reach, ctx->stream, &e);
+            f32 ? launch_resident_cg_f32(args, ks, (float*)ctx->r, (float*)ctx->q, (float*)ctx->p,
+                                         ctx->team, n, ctx->plan.W, ctx->plan.reach, ctx->stream, &e)
+                : launch_resident_cg_f64(args, ks, (double*)ctx->r, (double*)ctx->q, (double*)ctx->p,
+                                         ctx->team, n, ctx->plan.W, ctx->plan.reach, ctx->stream, &e);
         if (taken) {
             ctx->launches += 1;
             CK(e);

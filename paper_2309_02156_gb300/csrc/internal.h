@@ -186,9 +186,9 @@ bool launch_resident_gmres_f32(const DevArgs* a, KState* ks, float* V, size_t ld
                                const float* dinv, float* za, float* zb, float* t,
                                const ChebConfig* cheb, int n, const SlotPlan& plan,
                                cudaStream_t st, cudaError_t* launched);
-bool launch_resident_cg_f64(const DevArgs* a, KState* ks, double* r, double* q, TeamSlot* slots,
+bool launch_resident_cg_f64(const DevArgs* a, KState* ks, double* r, double* q, double* x, TeamSlot* slots,
                             int n, int W, int reach, cudaStream_t st, cudaError_t* launched);
-bool launch_resident_cg_f32(const DevArgs* a, KState* ks, float* r, float* q, TeamSlot* slots,
+bool launch_resident_cg_f32(const DevArgs* a, KState* ks, float* r, float* q, float* x, TeamSlot* slots,
                             int n, int W, int reach, cudaStream_t st, cudaError_t* launched);
 // Grid-wide CG for large systems (all SMs; three kernels per iteration): the
 // start (FP32: from x = 0), `iters` iterations (the body of a CUDA graph), and

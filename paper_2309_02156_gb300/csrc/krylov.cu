@@ -577,13 +577,13 @@ void launch_cg_block_f32(const DevArgs* a, KState* ks, float* r, float* p, float
     cg_block_kernel<SysF32><<<1, 1024, 0, st>>>(a, ks, r, p, q);
 }
 
-bool launch_resident_cg_f64(const DevArgs* a, KState* ks, double* r, double* q, TeamSlot* slots,
+bool launch_resident_cg_f64(const DevArgs* a, KState* ks, double* r, double* q, double* x, TeamSlot* slots,
                             int n, int W, int reach, cudaStream_t st, cudaError_t* launched) {
-    return launch_resident_cg<SysF64>(a, ks, r, q, slots, n, W, reach, st, launched);
+    return launch_resident_cg<SysF64>(a, ks, r, q, x, slots, n, W, reach, st, launched);
 }
-bool launch_resident_cg_f32(const DevArgs* a, KState* ks, float* r, float* q, TeamSlot* slots,
+bool launch_resident_cg_f32(const DevArgs* a, KState* ks, float* r, float* q, float* x, TeamSlot* slots,
                             int n, int W, int reach, cudaStream_t st, cudaError_t* launched) {
-    return launch_resident_cg<SysF32>(a, ks, r, q, slots, n, W, reach, st, launched);
+    return launch_resident_cg<SysF32>(a, ks, r, q, x, slots, n, W, reach, st, launched);
 }
 
 bool launch_resident_gmres_f64(const DevArgs* a, KState* ks, double* V, size_t ldv, int R,

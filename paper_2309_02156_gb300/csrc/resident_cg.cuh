@@ -19,10 +19,13 @@ namespace sa {
 
 constexpr int kResThreads = 512;
 
+// r, q and x of rows that do not fit in shared memory lie in rg, qg and xg,
+// vectors of the context: the iteration reads and writes 16 bytes at a time, and
+// the caller's x is aligned to its element only.
 template <class Sys, class Team>
 __device__ __forceinline__ void resident_cg(const DevArgs* __restrict__ a, KState* ks,
-                                            typename Sys::T* rg, typename Sys::T* qg, Team& tm,
-                                            const ResLayout& L) {
+                                            typename Sys::T* rg, typename Sys::T* qg,
+                                            typename Sys::T* xg, Team& tm, const ResLayout& L) {
     using T = typename Sys::T;
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ T scratch[33];
@@ -38,7 +41,7 @@ __device__ __forceinline__ void resident_cg(const DevArgs* __restrict__ a, KStat
     __shared__ ResBlock<T> B;
     T* const p = reinterpret_cast<T*>(dsm);
     B.setup(p, L, n, s_lo, s_hi, W, a->slot_reach, a->slot_off, a->slot,
-            reinterpret_cast<const T*>(a->sell_val), rg, qg, x);
+            reinterpret_cast<const T*>(a->sell_val), rg, qg, xg);
     const int rows = B.rows, r_lo = B.lo;
     // r = b - A x over the global iterate (p = r on the own rows), |r|^2; all
     // own rows are published.  ldcg: other blocks wrote their rows of x during
@@ -126,8 +129,7 @@ __device__ __forceinline__ void resident_cg(const DevArgs* __restrict__ a, KStat
                 break;
             }
             if (s_go == 0) {                       // the true residual decides
-                if (L.x_in)
-                    for (int i = tid; i < rows; i += bd) x[r_lo + i] = B.x[i];
+                for (int i = tid; i < rows; i += bd) x[r_lo + i] = B.x[i];
                 tm.total((T)0, scratch, [&](T) {});
                 if (tm.late) break;
                 tm.total(residual(false), scratch, [&](T t) {
@@ -150,8 +152,7 @@ __device__ __forceinline__ void resident_cg(const DevArgs* __restrict__ a, KStat
     // The final iterate and its true residual (reported, and used by the
     // refinement loop).
     __syncthreads();
-    if (L.x_in)
-        for (int i = tid; i < rows; i += bd) x[r_lo + i] = B.x[i];
+    for (int i = tid; i < rows; i += bd) x[r_lo + i] = B.x[i];
     if (!known && !tm.late) {
         tm.total((T)0, scratch, [&](T) {});
         if (!tm.late) tm.total(residual(false), scratch, [&](T t) { s_rr = t; });
@@ -172,7 +173,7 @@ __device__ __forceinline__ void resident_cg(const DevArgs* __restrict__ a, KStat
 template <class Sys>
 __global__ void __launch_bounds__(kResThreads, 1)
 resident_cg_grid_kernel(const DevArgs* __restrict__ a, KState* ks, typename Sys::T* r,
-                        typename Sys::T* q, TeamSlot* slots, const ResLayout L) {
+                        typename Sys::T* q, typename Sys::T* x, TeamSlot* slots, const ResLayout L) {
     __shared__ int bad;
     if (threadIdx.x == 0) bad = 0;
     __syncthreads();
@@ -180,18 +181,18 @@ resident_cg_grid_kernel(const DevArgs* __restrict__ a, KState* ks, typename Sys:
     tm.slots = slots;
     tm.count = reinterpret_cast<unsigned*>(slots + 2 * kTeamMax);
     tm.bad = &bad;
-    resident_cg<Sys>(a, ks, r, q, tm, L);
+    resident_cg<Sys>(a, ks, r, q, x, tm, L);
 }
 
 template <class Sys>
 __global__ void __launch_bounds__(kResThreads, 1)
 resident_cg_cluster_kernel(const DevArgs* __restrict__ a, KState* ks, typename Sys::T* r,
-                           typename Sys::T* q, const ResLayout L) {
+                           typename Sys::T* q, typename Sys::T* x, const ResLayout L) {
     __shared__ typename Sys::T box[32];
     ClusterTeam<typename Sys::T> tm;
     tm.box = box;
     tm.sync();                                     // every block has started before a remote store
-    resident_cg<Sys>(a, ks, r, q, tm, L);
+    resident_cg<Sys>(a, ks, r, q, x, tm, L);
     tm.sync();                                     // no block leaves while another may store to it
 }
 
@@ -199,7 +200,7 @@ resident_cg_cluster_kernel(const DevArgs* __restrict__ a, KState* ks, typename S
 // takes the streaming kernels).  *launched: the launch's own status.
 template <class Sys>
 static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r, typename Sys::T* q,
-                               TeamSlot* slots, int n, int W, int reach, cudaStream_t st,
+                               typename Sys::T* x, TeamSlot* slots, int n, int W, int reach, cudaStream_t st,
                                cudaError_t* launched) {
     using T = typename Sys::T;
     int dev = 0, sms = 0, optin = 0;
@@ -243,7 +244,7 @@ static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r,
                 cudaGetLastError();
                 continue;
             }
-            *launched = cudaLaunchKernelEx(&cfg, k, a, ks, r, q, (const ResLayout)L);
+            *launched = cudaLaunchKernelEx(&cfg, k, a, ks, r, q, x, (const ResLayout)L);
             return true;
         }
     }
@@ -264,7 +265,7 @@ static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r,
         return false;
     }
     cudaMemsetAsync(slots, 0, kTeamSlotBytes, st);
-    void* args[] = {(void*)&a, (void*)&ks, (void*)&r, (void*)&q, (void*)&slots, (void*)&L};
+    void* args[] = {(void*)&a, (void*)&ks, (void*)&r, (void*)&q, (void*)&x, (void*)&slots, (void*)&L};
     *launched = cudaLaunchCooperativeKernel((const void*)k, dim3(nblk), dim3(threads(L.per)), args,
                                             bytes, st);
     return true;

@@ -1,0 +1,80 @@
+"""Resident solves at the edges of what the entry points take: vectors that start
+at any element.
+
+Matrices are symmetric with 1 <= a_ii <= 2 and off-diagonal row sums of at most
+a_ii / 2: eigenvalues in [1/2, 3]."""
+import numpy as np
+import pytest
+import scipy.sparse as sp
+import torch
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _spd(n, offsets, rng):
+    offs = [o for o in offsets if 0 < o < n]
+    bands = [rng.uniform(-1, 1, n - o) * 0.25 / max(len(offs), 1) for o in offs]
+    A = sp.diags([rng.uniform(1, 2, n)] + bands + bands, [0] + offs + [-o for o in offs], format="csr")
+    A.sort_indices()
+    return A
+
+
+def _dev(a, dtype):
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=dtype)).to(DEV)
+
+
+def _csr(A):
+    import paper_2309_02156_gb300 as sa
+    return sa.CSR(_dev(A.indptr, np.int32), _dev(A.indices, np.int32), _dev(A.data, np.float64))
+
+
+def _view(t, start):
+    """A copy of t that starts `start` elements into a 16-byte aligned buffer."""
+    buf = torch.zeros(t.numel() + 2, dtype=t.dtype, device=DEV)
+    assert buf.data_ptr() % 16 == 0
+    out = buf[start:start + t.numel()]
+    out.copy_(t)
+    return out
+
+
+# x in shared memory; x outside it because of its size, and because of the reach
+@pytest.mark.parametrize("krylov", ["cg", "gmres"])
+@pytest.mark.parametrize("precision", ["f64", "mixed_krylov"])
+@pytest.mark.parametrize("n,offsets", [(5001, [1, 70]), (1001 * 1001, [1, 1001]), (30000, [1, 14000])])
+def test_vectors_at_any_element(n, offsets, precision, krylov):
+    """x and b that start at an odd element give the same bits: every element is
+    computed alike, whatever the width of an access."""
+    import paper_2309_02156_gb300 as sa
+    rng = np.random.default_rng(n)
+    A = _spd(n, offsets, rng)
+    b = rng.standard_normal(n)
+    Ad, bd = _csr(A), _dev(b, np.float64)
+    seq = sa.Sequence(n, 2, 8, zeta=2, guess="zero", max_iters=500, krylov=krylov, precision=precision)
+    got = []
+    for start in (0, 1):
+        x = _view(torch.zeros_like(bd), start)
+        info = seq.solve(Ad, _view(bd, start), 1e-12, x)
+        assert info["status"] == 0
+        got.append((info, x.cpu().numpy()))
+    seq.close()
+    assert got[0][0] == got[1][0] and np.array_equal(got[0][1], got[1][1])
+    assert np.linalg.norm(b - A @ got[1][1]) <= 1.01e-12 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("start", [0, 1])
+def test_batch_vectors_at_any_element(start):
+    import paper_2309_02156_gb300 as sa
+    rng = np.random.default_rng(7)
+    mats = [_spd(n, o, rng) for n, o in [(33, [1, 7]), (5001, [1, 70]), (20011, [1, 141])]]
+    bt = sa.Batch([(_dev(A.indptr, np.int32), _dev(A.indices, np.int32)) for A in mats], M=2, s=8, zeta=2)
+    bt.set_cluster(4, 512, 0)
+    for k, A in enumerate(mats):
+        bt.push(k, _view(_dev(rng.standard_normal(A.shape[0]), np.float64), start))
+    bs = [rng.standard_normal(A.shape[0]) for A in mats]
+    xs = [_view(torch.zeros(A.shape[0], dtype=torch.float64, device=DEV), start) for A in mats]
+    bt.step([_view(_dev(A.data, np.float64), start) for A in mats],
+            [_view(_dev(b, np.float64), start) for b in bs], xs, 1e-11)
+    for A, b, x in zip(mats, bs, xs):
+        assert np.linalg.norm(b - A @ x.cpu().numpy()) <= 1.01e-11 * np.linalg.norm(b)
+    bt.close()
