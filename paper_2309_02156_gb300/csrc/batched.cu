@@ -1191,6 +1191,19 @@ int batch_order(seq_batch* bt) {
     return cudaStreamSynchronize(bt->stream) == cudaSuccess ? SEQ_OK : SEQ_ECUDA;
 }
 
+// The dynamic shared memory that a kernel may use, set to all there is: the limit
+// is the process's, and other batches launch the same kernel.
+cudaError_t lift_smem_limit(StepKernel kern) {
+    int dev = 0, optin = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaFuncAttributes fa;
+    const cudaError_t e = cudaFuncGetAttributes(&fa, (const void*)kern);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                optin - (int)fa.sharedSizeBytes);
+}
+
 // The kernel of the schedule in bt, its threads and its dynamic shared memory:
 // all that the SM has, for the resident CG, or what the guess needs.  A
 // sequence that does not fit on its team's SMs gathers through L1, which the
@@ -1275,8 +1288,7 @@ int batch_capture(seq_batch* bt) {
     const StepLaunch sl = step_launch(bt);
     const StepKernel kern = sl.kern;
     const size_t smem = sl.smem;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess) {
+    if (lift_smem_limit(kern) != cudaSuccess) {
         cudaGetLastError();
         return SEQ_ECUDA;
     }
@@ -1551,8 +1563,7 @@ int seq_batch_autotune(seq_batch* bt, const double* const* values, const double*
                     const StepKernel kern = sl.kern;
                     const size_t smem = sl.smem;
                     int nb = 0;
-                    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem) != cudaSuccess ||
+                    if (lift_smem_limit(kern) != cudaSuccess ||
                         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, sl.threads, smem) !=
                             cudaSuccess ||
                         nb < bps || (cl > 1 && cluster_grid(bt, sl) <= 0)) {

@@ -202,7 +202,7 @@ extern "C" int seq_sketch_block_noalloc(int32_t n, int32_t nnz, const int32_t* r
     const int wsz = s * (M + 1);
     const size_t smem = sizeof(double) * (size_t)kNoAllocWarps * wsz;
     if (cudaFuncSetAttribute(noalloc_sketch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess) {
+                             (int)(sizeof(double) * kNoAllocWarps * kNoAllocSlots)) != cudaSuccess) {
         cudaGetLastError();
         return SEQ_ECUDA;
     }

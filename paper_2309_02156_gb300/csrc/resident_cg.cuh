@@ -208,7 +208,10 @@ static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r,
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (sms > kTeamMax) sms = kTeamMax;
-    const size_t budget = (size_t)optin - 2048;    // the kernel's static shared memory
+    // Less the kernel's static shared memory.  A kernel's limit is the process's
+    // and other threads launch it too, so it is set to the same value each time,
+    // not to this launch's size.
+    const size_t budget = (size_t)optin - 2048;
     const int ns = (n + 31) / 32;
     // A warp per slice; in FP64 eight warps fill the FP64 pipe and more only
     // add to the reductions.
@@ -222,7 +225,7 @@ static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r,
             if (!res_layout(n, W, reach, c, sizeof(T), budget, &L)) continue;
             auto k = resident_cg_cluster_kernel<Sys>;
             const size_t bytes = res_bytes(L, W, sizeof(T));
-            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess ||
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget) != cudaSuccess ||
                 (c > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
                 cudaGetLastError();
                 continue;
@@ -258,7 +261,7 @@ static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r,
     int per_sm = 0, coop = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     if (!coop ||
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads(L.per), bytes) != cudaSuccess ||
         per_sm * sms < nblk) {
         cudaGetLastError();

@@ -573,8 +573,8 @@ static bool launch_resident_gmres(const DevArgs* a, KState* ks, const GmresArgs<
     int nblk = (ns + 3) / 4;
     if (nblk > sms) nblk = sms;
     GmresLayout L;
-    if (!gmres_layout(n, plan.W, plan.reach, nblk, A.R, A.sweeps, sizeof(T), (size_t)optin - 20480, &L))
-        return false;
+    const size_t budget = (size_t)optin - 20480;   // less the static arrays; also the kernel's limit
+    if (!gmres_layout(n, plan.W, plan.reach, nblk, A.R, A.sweeps, sizeof(T), budget, &L)) return false;
     if (n > (sizeof(T) == 8 ? kResGmresRows64 : A.sweeps > 0 ? kResGmresRows32Pre : kResGmresRows32))
         return false;
     nblk = (ns + L.per - 1) / L.per;
@@ -584,7 +584,7 @@ static bool launch_resident_gmres(const DevArgs* a, KState* ks, const GmresArgs<
     const Kern k = plan.W <= 5 ? resident_gmres_kernel<Sys, 5> : resident_gmres_kernel<Sys, 9>;
     const size_t bytes = gmres_bytes(L, plan.W, A.R, A.sweeps, sizeof(T));
     int per_sm = 0;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess ||
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, bytes) != cudaSuccess ||
         per_sm * sms < nblk) {
         cudaGetLastError();

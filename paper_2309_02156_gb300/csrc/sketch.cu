@@ -165,9 +165,10 @@ static void launch_sketch_impl(const int* rowptr, const int* colind, const T* va
     // so that no team takes more than kSkMaxTiles tiles).
     const int teams = sketch_teams(s, M + 1);
     const size_t smem = (size_t)teams * sketch_team_bytes(s, M + 1);
-    // The attribute is per device: set it on every call (cheap, host only).
+    // The attribute is per device: set it on every call (cheap, host only), to
+    // one value for all sizes (other threads launch the kernel too).
     cudaFuncSetAttribute(sketch_block_kernel<T, XT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
+                         (int)kSkSmemCap);
     sketch_block_kernel<T, XT><<<nblk, teams * kSkTeamThreads, smem, st>>>(
         rowptr, colind, val, X, ldx, b, n, nnz, M, s, zeta, seed, partial, bad);
     const double inv = 1.0 / sqrt((double)zeta);

@@ -1,8 +1,10 @@
 """Resident solves at the edges of what the entry points take: vectors that start
-at any element.
+at any element, and solves of several sizes at once.
 
 Matrices are symmetric with 1 <= a_ii <= 2 and off-diagonal row sums of at most
 a_ii / 2: eigenvalues in [1/2, 3]."""
+import threading
+
 import numpy as np
 import pytest
 import scipy.sparse as sp
@@ -78,3 +80,38 @@ def test_batch_vectors_at_any_element(start):
     for A, b, x in zip(mats, bs, xs):
         assert np.linalg.norm(b - A @ x.cpu().numpy()) <= 1.01e-11 * np.linalg.norm(b)
     bt.close()
+
+
+# sizes whose launches need different amounts of shared memory, in one kernel
+@pytest.mark.parametrize("krylov,sizes", [("cg", (90000, 28900)), ("gmres", (60025, 3600))])
+def test_two_threads_of_different_sizes(krylov, sizes):
+    """A thread per context, each with a stream of its own: every solve of either
+    succeeds and has the bits that it has alone."""
+    import paper_2309_02156_gb300 as sa
+    wrong = []
+
+    def work(n, alone, reps):
+        rng = np.random.default_rng(n)
+        A = _spd(n, [1, int(np.sqrt(n))], rng)
+        with torch.cuda.stream(torch.cuda.Stream()):
+            Ad, bd = _csr(A), _dev(rng.standard_normal(n), np.float64)
+            seq = sa.Sequence(n, 2, 8, zeta=2, guess="zero", max_iters=3, krylov=krylov)
+            for _ in range(reps):
+                x = torch.zeros_like(bd)
+                try:
+                    seq.solve(Ad, bd, 1e-12, x)
+                except sa.SeqError as e:
+                    wrong.append((n, str(e)))
+                if alone.setdefault(n, x) is not x and not torch.equal(alone[n], x):
+                    wrong.append((n, "other bits"))
+            seq.close()
+
+    alone = {}
+    for n in sizes:
+        work(n, alone, 1)
+    threads = [threading.Thread(target=work, args=(n, alone, 3000)) for n in sizes]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong, (len(wrong), wrong[:3])

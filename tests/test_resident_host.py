@@ -11,7 +11,36 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 PROGRAM = r'''
 #include <cstdio>
-#include "resident.cuh"
+#include <set>
+#include <cuda_runtime.h>
+
+// What the launch code asks the driver, answered for a GPU of 152 SMs.
+static std::set<int> limits;                 // shared-memory limits that were set
+static cudaError_t fake_device(int* d) { *d = 0; return cudaSuccess; }
+static cudaError_t fake_attribute(int* v, cudaDeviceAttr a, int) {
+    *v = a == cudaDevAttrMultiProcessorCount ? 152 : a == cudaDevAttrMaxSharedMemoryPerBlockOptin ? 232448 : 1;
+    return cudaSuccess;
+}
+template <class F> static cudaError_t fake_limit(F, cudaFuncAttribute a, int v) {
+    if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) limits.insert(v);
+    return cudaSuccess;
+}
+template <class F> static cudaError_t fake_blocks(int* b, F, int, size_t) { *b = 1; return cudaSuccess; }
+static cudaError_t fake_clusters(int* c, const void*, const cudaLaunchConfig_t*) { *c = 1; return cudaSuccess; }
+static cudaError_t fake_memset(void*, int, size_t, cudaStream_t) { return cudaSuccess; }
+static cudaError_t fake_last() { return cudaSuccess; }
+template <class... A> static cudaError_t fake_launch(A&&...) { return cudaSuccess; }
+#define cudaGetDevice fake_device
+#define cudaDeviceGetAttribute fake_attribute
+#define cudaFuncSetAttribute fake_limit
+#define cudaOccupancyMaxActiveBlocksPerMultiprocessor fake_blocks
+#define cudaOccupancyMaxActiveClusters fake_clusters
+#define cudaMemsetAsync fake_memset
+#define cudaGetLastError fake_last
+#define cudaLaunchKernelEx fake_launch
+#define cudaLaunchCooperativeKernel fake_launch
+#include "resident_cg.cuh"
+#include "resident_gmres.cuh"
 using namespace sa;
 static int bad = 0;
 #define CHECK(c) do { if (!(c)) { printf("line %d: %s\n", __LINE__, #c); bad = 1; } } while (0)
@@ -26,7 +55,44 @@ static ResLayout grid_layout(int n, int W, int reach) {
     return L;
 }
 
+static SlotPlan five(int reach) {
+    SlotPlan p = {};
+    p.W = p.list.count = 5;
+    p.reach = reach;
+    const int off[5] = {-reach, -1, 0, 1, reach};
+    for (int k = 0; k < 5; ++k) p.list.off[k] = off[k];
+    return p;
+}
+template <class Sys> static bool cg(int n, int reach) {
+    cudaError_t e = cudaSuccess;
+    return launch_resident_cg<Sys>(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, n, 5, reach,
+                                   nullptr, &e) && e == cudaSuccess;
+}
+template <class Sys> static bool gmres(int n, int reach, int sweeps) {
+    cudaError_t e = cudaSuccess;
+    GmresArgs<typename Sys::T> A = {};
+    A.R = 30;
+    A.sweeps = sweeps;
+    return launch_resident_gmres<Sys>(nullptr, nullptr, A, n, five(reach), nullptr, &e) && e == cudaSuccess;
+}
+
+// The limit of a kernel's dynamic shared memory belongs to the process: whatever
+// the size of a launch, it is set to the same value.
+static void one_limit() {
+    for (int f = 0; f < 2; ++f) {
+        limits.clear();
+        for (int n : {33, 4096, 20000, 30000, 70000, 262144})
+            CHECK(f ? cg<SysF32>(n, 100) : cg<SysF64>(n, 100));
+        CHECK(limits.size() == 1);
+        limits.clear();
+        for (int n : {33, 4096, 20000, 30000})
+            for (int sweeps : {0, 3}) CHECK(f ? gmres<SysF32>(n, 100, sweeps) : gmres<SysF64>(n, 100, sweeps));
+        CHECK(limits.size() == 1);
+    }
+}
+
 int main() {
+    one_limit();
     // The sizes of the offset-view solves: x does not fit in shared memory.
     CHECK(grid_layout(1001 * 1001, 5, 1001).x_in == 0);
     CHECK(grid_layout(30000, 5, 14000).x_in == 0);
