@@ -36,6 +36,13 @@ __device__ __forceinline__ void team_peek(const TeamSlot* s, unsigned long long&
                  : "=l"(bits), "=l"(epoch) : "l"(s) : "memory");
 }
 
+// Whether a counter that reads `seen` has reached `want`.  Both count modulo 2^32
+// (a long solve passes it) and lie less than 2^31 apart: no block is more than
+// one wait ahead of another.
+__host__ __device__ inline bool team_arrived(unsigned seen, unsigned want) {
+    return (int)(seen - want) >= 0;
+}
+
 __device__ __forceinline__ unsigned long long to_bits(double v) {
     return (unsigned long long)__double_as_longlong(v);
 }
@@ -154,12 +161,12 @@ struct GridTeam {
                 team_post(s + blockIdx.x, to_bits(b), epoch);
                 asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(count) : "memory");
                 const unsigned want = epoch * (unsigned)nb;
-                unsigned seen = 0;
+                unsigned seen = want - 1;
                 for (int left = *bad ? 0 : kTeamPolls; left > 0; --left) {
                     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
-                    if (seen >= want) break;
+                    if (team_arrived(seen, want)) break;
                 }
-                if (seen < want) *bad = 1;
+                if (!team_arrived(seen, want)) *bad = 1;
                 team_fence();
             }
             __syncwarp();

@@ -166,12 +166,12 @@ struct GmresTeam {
         if (threadIdx.x == 0) {
             asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(count) : "memory");
             const unsigned want = epoch * gridDim.x;
-            unsigned seen = 0;
+            unsigned seen = want - 1;
             for (int left = *bad ? 0 : kTeamPolls; left > 0; --left) {
                 asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
-                if (seen >= want) break;
+                if (team_arrived(seen, want)) break;
             }
-            if (seen < want) *bad = 1;
+            if (!team_arrived(seen, want)) *bad = 1;
             team_fence();
         }
         __syncthreads();

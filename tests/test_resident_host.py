@@ -91,8 +91,20 @@ static void one_limit() {
     }
 }
 
+// The grid's wait counter past 2^32: 152 blocks add one each per wait.
+static void counter_wraps() {
+    for (unsigned long long waits : {1ull, 28256362ull, 28256363ull, 28256364ull, 56512727ull, 4294967297ull}) {
+        const unsigned want = (unsigned)waits * 152u;
+        for (unsigned k = 0; k <= 304; ++k) {      // this wait's and the next one's arrivals
+            const unsigned seen = want - 152u + k;
+            CHECK(team_arrived(seen, want) == (k >= 152));
+        }
+    }
+}
+
 int main() {
     one_limit();
+    counter_wraps();
     // The sizes of the offset-view solves: x does not fit in shared memory.
     CHECK(grid_layout(1001 * 1001, 5, 1001).x_in == 0);
     CHECK(grid_layout(30000, 5, 14000).x_in == 0);
