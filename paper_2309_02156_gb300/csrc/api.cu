@@ -422,21 +422,19 @@ int run_gmres(seq_ctx* ctx, bool f32) {
     if (ctx->sell_ok && ctx->plan.W && !ctx->profiling) {
         const seq_config& c = ctx->cfg;
         const ChebConfig cheb{c.precond_kind == 1, ctx->pc_tab};
-        cudaError_t e = cudaSuccess;
         const bool taken =
             f32 ? launch_resident_gmres_f32(ctx->d_args_in, ks, (float*)ctx->V, ctx->ldv, c.restart,
                                             (float*)ctx->kpartial, ctx->team, c.precond_sweeps,
                                             c.precond_omega, (const float*)ctx->dinv,
                                             (float*)ctx->za, (float*)ctx->zb, (float*)ctx->tprec,
-                                            &cheb, c.n, ctx->plan, ctx->stream, &e)
+                                            &cheb, c.n, ctx->plan, ctx->stream)
                 : launch_resident_gmres_f64(ctx->d_args, ks, (double*)ctx->V, ctx->ldv, c.restart,
                                             ctx->kpartial, ctx->team, c.precond_sweeps,
                                             c.precond_omega, (const double*)ctx->dinv,
                                             (double*)ctx->za, (double*)ctx->zb, (double*)ctx->tprec,
-                                            &cheb, c.n, ctx->plan, ctx->stream, &e);
+                                            &cheb, c.n, ctx->plan, ctx->stream);
         if (taken) {
             ctx->launches += 1;
-            CK(e);
             CK(cudaGetLastError());
             const int rc = read_tail(ctx, ks);
             if (rc) return rc;
@@ -554,15 +552,13 @@ int run_cg(seq_ctx* ctx, bool f32) {
     const DevArgs* args = f32 ? ctx->d_args_in : ctx->d_args;
     const int n = ctx->cfg.n;
     if (ctx->sell_ok && ctx->plan.W) {
-        cudaError_t e = cudaSuccess;
         const bool taken =
             f32 ? launch_resident_cg_f32(args, ks, (float*)ctx->r, (float*)ctx->q, (float*)ctx->p,
-                                         ctx->team, n, ctx->plan.W, ctx->plan.reach, ctx->stream, &e)
+                                         ctx->team, n, ctx->plan.W, ctx->plan.reach, ctx->stream)
                 : launch_resident_cg_f64(args, ks, (double*)ctx->r, (double*)ctx->q, (double*)ctx->p,
-                                         ctx->team, n, ctx->plan.W, ctx->plan.reach, ctx->stream, &e);
+                                         ctx->team, n, ctx->plan.W, ctx->plan.reach, ctx->stream);
         if (taken) {
             ctx->launches += 1;
-            CK(e);
             CK(cudaGetLastError());
             const int rc = read_tail(ctx, ks);
             if (rc) return rc;

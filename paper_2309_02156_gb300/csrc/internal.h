@@ -180,16 +180,16 @@ bool launch_resident_gmres_f64(const DevArgs* a, KState* ks, double* V, size_t l
                                double* kpart, TeamSlot* team, int sweeps, double omega,
                                const double* dinv, double* za, double* zb, double* t,
                                const ChebConfig* cheb, int n, const SlotPlan& plan,
-                               cudaStream_t st, cudaError_t* launched);
+                               cudaStream_t st);
 bool launch_resident_gmres_f32(const DevArgs* a, KState* ks, float* V, size_t ldv, int R,
                                float* kpart, TeamSlot* team, int sweeps, double omega,
                                const float* dinv, float* za, float* zb, float* t,
                                const ChebConfig* cheb, int n, const SlotPlan& plan,
-                               cudaStream_t st, cudaError_t* launched);
+                               cudaStream_t st);
 bool launch_resident_cg_f64(const DevArgs* a, KState* ks, double* r, double* q, double* x, TeamSlot* slots,
-                            int n, int W, int reach, cudaStream_t st, cudaError_t* launched);
+                            int n, int W, int reach, cudaStream_t st);
 bool launch_resident_cg_f32(const DevArgs* a, KState* ks, float* r, float* q, float* x, TeamSlot* slots,
-                            int n, int W, int reach, cudaStream_t st, cudaError_t* launched);
+                            int n, int W, int reach, cudaStream_t st);
 // Grid-wide CG for large systems (all SMs; three kernels per iteration): the
 // start (FP32: from x = 0), `iters` iterations (the body of a CUDA graph), and
 // the true residual (check != 0: convergence check and restart).

@@ -578,22 +578,22 @@ void launch_cg_block_f32(const DevArgs* a, KState* ks, float* r, float* p, float
 }
 
 bool launch_resident_cg_f64(const DevArgs* a, KState* ks, double* r, double* q, double* x, TeamSlot* slots,
-                            int n, int W, int reach, cudaStream_t st, cudaError_t* launched) {
-    return launch_resident_cg<SysF64>(a, ks, r, q, x, slots, n, W, reach, st, launched);
+                            int n, int W, int reach, cudaStream_t st) {
+    return launch_resident_cg<SysF64>(a, ks, r, q, x, slots, n, W, reach, st);
 }
 bool launch_resident_cg_f32(const DevArgs* a, KState* ks, float* r, float* q, float* x, TeamSlot* slots,
-                            int n, int W, int reach, cudaStream_t st, cudaError_t* launched) {
-    return launch_resident_cg<SysF32>(a, ks, r, q, x, slots, n, W, reach, st, launched);
+                            int n, int W, int reach, cudaStream_t st) {
+    return launch_resident_cg<SysF32>(a, ks, r, q, x, slots, n, W, reach, st);
 }
 
 bool launch_resident_gmres_f64(const DevArgs* a, KState* ks, double* V, size_t ldv, int R,
                                double* kpart, TeamSlot* team, int sweeps, double omega,
                                const double* dinv, double* za, double* zb, double* t,
                                const ChebConfig* cheb, int n, const SlotPlan& plan,
-                               cudaStream_t st, cudaError_t* launched) {
+                               cudaStream_t st) {
     const GmresArgs<double> A = {V, ldv, R, kpart, team, sweeps, cheb && cheb->on, omega, dinv, za, zb, t,
                                 cheb ? cheb->tab : nullptr};
-    return launch_resident_gmres<SysF64>(a, ks, A, n, plan, st, launched);
+    return launch_resident_gmres<SysF64>(a, ks, A, n, plan, st);
 }
 
 void launch_cgg_start_f64(const DevArgs* a, KState* ks, double* r, double* p, double* partial,

@@ -38,10 +38,10 @@ bool launch_resident_gmres_f32(const DevArgs* a, KState* ks, float* V, size_t ld
                                float* kpart, TeamSlot* team, int sweeps, double omega,
                                const float* dinv, float* za, float* zb, float* t,
                                const ChebConfig* cheb, int n, const SlotPlan& plan,
-                               cudaStream_t st, cudaError_t* launched) {
+                               cudaStream_t st) {
     const GmresArgs<float> A = {V, ldv, R, kpart, team, sweeps, cheb && cheb->on, omega, dinv, za, zb, t,
                                 cheb ? cheb->tab : nullptr};
-    return launch_resident_gmres<SysF32>(a, ks, A, n, plan, st, launched);
+    return launch_resident_gmres<SysF32>(a, ks, A, n, plan, st);
 }
 
 }  // namespace sa

@@ -196,12 +196,12 @@ resident_cg_cluster_kernel(const DevArgs* __restrict__ a, KState* ks, typename S
     tm.sync();                                     // no block leaves while another may store to it
 }
 
-// Launch of one CG solve by a resident team; false when none fits (the caller
-// takes the streaming kernels).  *launched: the launch's own status.
+// Launch of one CG solve by a resident team; false when none fits or the driver
+// refuses the launch (the caller takes the streaming kernels).
 template <class Sys>
 static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r, typename Sys::T* q,
-                               typename Sys::T* x, TeamSlot* slots, int n, int W, int reach, cudaStream_t st,
-                               cudaError_t* launched) {
+                               typename Sys::T* x, TeamSlot* slots, int n, int W, int reach,
+                               cudaStream_t st) {
     using T = typename Sys::T;
     int dev = 0, sms = 0, optin = 0;
     cudaGetDevice(&dev);
@@ -247,8 +247,8 @@ static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r,
                 cudaGetLastError();
                 continue;
             }
-            *launched = cudaLaunchKernelEx(&cfg, k, a, ks, r, q, x, (const ResLayout)L);
-            return true;
+            if (cudaLaunchKernelEx(&cfg, k, a, ks, r, q, x, (const ResLayout)L) == cudaSuccess) return true;
+            cudaGetLastError();
         }
     }
     // At least four slices per block: the reductions cost more than rows save.
@@ -269,8 +269,11 @@ static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r,
     }
     cudaMemsetAsync(slots, 0, kTeamSlotBytes, st);
     void* args[] = {(void*)&a, (void*)&ks, (void*)&r, (void*)&q, (void*)&x, (void*)&slots, (void*)&L};
-    *launched = cudaLaunchCooperativeKernel((const void*)k, dim3(nblk), dim3(threads(L.per)), args,
-                                            bytes, st);
+    if (cudaLaunchCooperativeKernel((const void*)k, dim3(nblk), dim3(threads(L.per)), args, bytes, st) !=
+        cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
     return true;
 }
 

@@ -555,11 +555,10 @@ resident_gmres_kernel(const DevArgs* __restrict__ a, KState* ks,
 }
 
 // Launch of a whole GMRES solve by a resident grid; false when the size does not
-// fit (the caller takes the cycle graph).
+// fit or the driver refuses the launch (the caller takes the cycle graph).
 template <class Sys>
 static bool launch_resident_gmres(const DevArgs* a, KState* ks, const GmresArgs<typename Sys::T>& A,
-                                  int n, const SlotPlan& plan, cudaStream_t st,
-                                  cudaError_t* launched) {
+                                  int n, const SlotPlan& plan, cudaStream_t st) {
     using T = typename Sys::T;
     if (plan.list.count == 0 || plan.W > 9 || A.R > kResRestart) return false;
     int dev = 0, sms = 0, optin = 0, coop = 0;
@@ -593,7 +592,11 @@ static bool launch_resident_gmres(const DevArgs* a, KState* ks, const GmresArgs<
     cudaMemsetAsync(A.team, 0, kTeamSlotBytes, st);
     GmresArgs<T> args_copy = A;
     void* args[] = {(void*)&a, (void*)&ks, (void*)&args_copy, (void*)&L};
-    *launched = cudaLaunchCooperativeKernel((const void*)k, dim3(nblk), dim3(threads), args, bytes, st);
+    if (cudaLaunchCooperativeKernel((const void*)k, dim3(nblk), dim3(threads), args, bytes, st) !=
+        cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
     return true;
 }
 

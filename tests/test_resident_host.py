@@ -28,8 +28,10 @@ template <class F> static cudaError_t fake_limit(F, cudaFuncAttribute a, int v) 
 template <class F> static cudaError_t fake_blocks(int* b, F, int, size_t) { *b = 1; return cudaSuccess; }
 static cudaError_t fake_clusters(int* c, const void*, const cudaLaunchConfig_t*) { *c = 1; return cudaSuccess; }
 static cudaError_t fake_memset(void*, int, size_t, cudaStream_t) { return cudaSuccess; }
-static cudaError_t fake_last() { return cudaSuccess; }
-template <class... A> static cudaError_t fake_launch(A&&...) { return cudaSuccess; }
+static cudaError_t refusal = cudaSuccess, pending = cudaSuccess;    // of launches
+static int launches = 0;
+static cudaError_t fake_last() { const cudaError_t e = pending; pending = cudaSuccess; return e; }
+template <class... A> static cudaError_t fake_launch(A&&...) { ++launches; return pending = refusal; }
 #define cudaGetDevice fake_device
 #define cudaDeviceGetAttribute fake_attribute
 #define cudaFuncSetAttribute fake_limit
@@ -64,16 +66,14 @@ static SlotPlan five(int reach) {
     return p;
 }
 template <class Sys> static bool cg(int n, int reach) {
-    cudaError_t e = cudaSuccess;
     return launch_resident_cg<Sys>(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, n, 5, reach,
-                                   nullptr, &e) && e == cudaSuccess;
+                                   nullptr);
 }
 template <class Sys> static bool gmres(int n, int reach, int sweeps) {
-    cudaError_t e = cudaSuccess;
     GmresArgs<typename Sys::T> A = {};
     A.R = 30;
     A.sweeps = sweeps;
-    return launch_resident_gmres<Sys>(nullptr, nullptr, A, n, five(reach), nullptr, &e) && e == cudaSuccess;
+    return launch_resident_gmres<Sys>(nullptr, nullptr, A, n, five(reach), nullptr);
 }
 
 // The limit of a kernel's dynamic shared memory belongs to the process: whatever
@@ -102,8 +102,23 @@ static void counter_wraps() {
     }
 }
 
+// A launch that the driver refuses is no solve: the caller takes the streaming
+// kernels, and no error is left behind for its next check.
+static void refused() {
+    refusal = cudaErrorCooperativeLaunchTooLarge;
+    for (int n : {4096, 30000, 262144}) {
+        launches = 0;
+        CHECK(!cg<SysF64>(n, 100) && !cg<SysF32>(n, 100) && launches >= 2 && pending == cudaSuccess);
+    }
+    launches = 0;
+    CHECK(!gmres<SysF64>(10000, 100, 0) && !gmres<SysF32>(10000, 100, 3) && launches == 2 &&
+          pending == cudaSuccess);
+    refusal = cudaSuccess;
+}
+
 int main() {
     one_limit();
+    refused();
     counter_wraps();
     // The sizes of the offset-view solves: x does not fit in shared memory.
     CHECK(grid_layout(1001 * 1001, 5, 1001).x_in == 0);
