@@ -241,7 +241,7 @@ int build_sell(seq_ctx* ctx, const seq_csr* A) {
     ctx->plan = SlotPlan{};
     const int n = A->n, ns = (n + 31) / 32;
     launch_slot_stats(A->rowptr, A->colind, n, A->nnz, ctx->sell_width, ctx->d_stats, ctx->stream);
-    ctx->launches += 1;
+    ctx->launches += 2;
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(ctx->h_stats, ctx->d_stats, sizeof(SlotStats), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));

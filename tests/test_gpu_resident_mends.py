@@ -115,3 +115,16 @@ def test_two_threads_of_different_sizes(krylov, sizes):
     for t in threads:
         t.join()
     assert not wrong, (len(wrong), wrong[:3])
+
+
+@pytest.mark.parametrize("krylov", ["cg", "gmres"])
+def test_resident_solve_counts_its_launches(krylov):
+    """Two launches for the matrix's offsets, one for its copy, one for the solve."""
+    import paper_2309_02156_gb300 as sa
+    rng = np.random.default_rng(3)
+    n = 5001
+    seq = sa.Sequence(n, 2, 8, zeta=2, guess="zero", krylov=krylov)
+    info = seq.solve(_csr(_spd(n, [1, 70], rng)), _dev(rng.standard_normal(n), np.float64), 1e-10,
+                     torch.zeros(n, dtype=torch.float64, device=DEV))
+    seq.close()
+    assert info["launches"] == 4
