@@ -235,7 +235,7 @@ int reserve_copy(seq_ctx* ctx, size_t entries, bool columns, size_t slots) {
 // when it exists and has at most a quarter more entries than SELL-32 (it
 // stores no columns: 10.0 bytes per FP64 entry and 5.3 per FP32 one with that
 // padding, against 12 and 8); else SELL-32; neither (CSR is used) when
-// padding would more than double the storage.
+// padding would more than double the storage or no kernel of the solve reads it.
 int build_sell(seq_ctx* ctx, const seq_csr* A) {
     ctx->sell_ok = false;
     ctx->plan = SlotPlan{};
@@ -252,6 +252,11 @@ int build_sell(seq_ctx* ctx, const seq_csr* A) {
     const size_t el = ctx->mixed ? sizeof(float) : sizeof(double);
     const float* v32 = A->values_f32 ? A->values_f32 : ctx->val32;
     const SlotPlan plan = plan_slots(*ctx->h_stats, n);
+    // A CG that no resident team takes and that is too small for the grid's kernels
+    // runs in one block, from the CSR arrays: nothing would read a copy.
+    if (ctx->cfg.krylov == SEQ_CG && n < kGridCgMinRows &&
+        !(plan.W && resident_cg_fits_here(n, plan.W, plan.reach, el)))
+        return SEQ_OK;
     if (plan.W) {
         total = 32LL * ns * plan.W;
         int rc = reserve_copy(ctx, (size_t)total, false, (size_t)ns * plan.W);

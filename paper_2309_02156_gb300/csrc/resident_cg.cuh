@@ -196,6 +196,37 @@ resident_cg_cluster_kernel(const DevArgs* __restrict__ a, KState* ks, typename S
     tm.sync();                                     // no block leaves while another may store to it
 }
 
+// What the current device gives a resident team: blocks of a grid, bytes of
+// shared memory of a block.  The bytes leave out the kernel's static shared
+// memory; they are also its limit, which belongs to the process and is set by
+// other threads too: always to the same value, not to a launch's size.
+struct TeamRoom {
+    int sms;
+    size_t budget;
+};
+static TeamRoom team_room() {
+    int dev = 0, sms = 0, optin = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return {sms < kTeamMax ? sms : kTeamMax, (size_t)optin - 2048};
+}
+
+// Rows up to which the team is a cluster; the layout of the grid's blocks, at
+// least four slices in each: the reductions cost more than rows save.
+inline int cluster_rows(size_t el) { return el == 8 ? kClusterCgRows64 : kClusterCgRows32; }
+inline bool grid_layout(int n, int W, int reach, size_t el, const TeamRoom& room, ResLayout* L) {
+    const int nblk = ((n + 31) / 32 + 3) / 4;
+    return res_layout(n, W, reach, nblk < room.sms ? nblk : room.sms, el, room.budget, L);
+}
+
+// Whether a resident team has room for the solve.
+inline bool resident_cg_fits(int n, int W, int reach, size_t el, const TeamRoom& room) {
+    ResLayout L;
+    return (n <= cluster_rows(el) && res_layout(n, W, reach, 16, el, room.budget, &L)) ||
+           grid_layout(n, W, reach, el, room, &L);
+}
+
 // Launch of one CG solve by a resident team; false when none fits or the driver
 // refuses the launch (the caller takes the streaming kernels).
 template <class Sys>
@@ -203,15 +234,7 @@ static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r,
                                typename Sys::T* x, TeamSlot* slots, int n, int W, int reach,
                                cudaStream_t st) {
     using T = typename Sys::T;
-    int dev = 0, sms = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (sms > kTeamMax) sms = kTeamMax;
-    // Less the kernel's static shared memory.  A kernel's limit is the process's
-    // and other threads launch it too, so it is set to the same value each time,
-    // not to this launch's size.
-    const size_t budget = (size_t)optin - 2048;
+    const TeamRoom room = team_room();
     const int ns = (n + 31) / 32;
     // A warp per slice; in FP64 eight warps fill the FP64 pipe and more only
     // add to the reductions.
@@ -220,12 +243,12 @@ static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r,
         return t < 128 ? 128 : (t > most ? most : t);
     };
     ResLayout L;
-    if (n <= (sizeof(T) == 8 ? kClusterCgRows64 : kClusterCgRows32)) {
+    if (n <= cluster_rows(sizeof(T))) {
         for (int c = 16; c >= 8; c >>= 1) {
-            if (!res_layout(n, W, reach, c, sizeof(T), budget, &L)) continue;
+            if (!res_layout(n, W, reach, c, sizeof(T), room.budget, &L)) continue;
             auto k = resident_cg_cluster_kernel<Sys>;
             const size_t bytes = res_bytes(L, W, sizeof(T));
-            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget) != cudaSuccess ||
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room.budget) != cudaSuccess ||
                 (c > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
                 cudaGetLastError();
                 continue;
@@ -251,19 +274,17 @@ static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r,
             cudaGetLastError();
         }
     }
-    // At least four slices per block: the reductions cost more than rows save.
-    int nblk = (ns + 3) / 4;
-    if (nblk > sms) nblk = sms;
-    if (!res_layout(n, W, reach, nblk, sizeof(T), budget, &L)) return false;
-    nblk = (ns + L.per - 1) / L.per;
+    if (!grid_layout(n, W, reach, sizeof(T), room, &L)) return false;
+    const int nblk = (ns + L.per - 1) / L.per;
     auto k = resident_cg_grid_kernel<Sys>;
     const size_t bytes = res_bytes(L, W, sizeof(T));
-    int per_sm = 0, coop = 0;
+    int dev = 0, per_sm = 0, coop = 0;
+    cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     if (!coop ||
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget) != cudaSuccess ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room.budget) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads(L.per), bytes) != cudaSuccess ||
-        per_sm * sms < nblk) {
+        per_sm * room.sms < nblk) {
         cudaGetLastError();
         return false;
     }

@@ -128,3 +128,59 @@ def test_resident_solve_counts_its_launches(krylov):
                      torch.zeros(n, dtype=torch.float64, device=DEV))
     seq.close()
     assert info["launches"] == 4
+
+
+def _irregular(kind, n, rng):
+    """CSR arrays of a symmetric matrix without the slot form."""
+    if kind == "offsets25":
+        A = _spd(n, list(range(1, 13)), rng)
+    elif kind == "scattered":
+        A = _spd(n, [1], rng)
+        i, j = rng.integers(0, n, (2, 3 * n))
+        S = sp.coo_matrix((rng.uniform(-0.01, 0.01, 3 * n), (i, j)), shape=(n, n)).tocsr()
+        A = (A + S + S.T).tocsr()
+        A.sort_indices()
+    else:
+        A = _spd(n, [1, 70], rng)
+    ptr, ci, v = A.indptr, A.indices.copy(), A.data.copy()
+    if kind == "unsorted":
+        for i in range(n):
+            ci[ptr[i]:ptr[i + 1]] = ci[ptr[i]:ptr[i + 1]][::-1]
+            v[ptr[i]:ptr[i + 1]] = v[ptr[i]:ptr[i + 1]][::-1]
+    if kind == "repeated":                   # every diagonal entry in two halves
+        rows = np.repeat(np.arange(n), np.diff(ptr))
+        half = np.where(ci == rows, 0.5, 1.0)
+        order = np.argsort(np.concatenate([rows, np.arange(n)]), kind="stable")
+        ci = np.concatenate([ci, np.arange(n)])[order]
+        v = np.concatenate([v * half, 0.5 * A.diagonal()])[order]
+        ptr = ptr + np.arange(n + 1)
+    return A, (ptr, ci, v)
+
+
+# the largest size of the one-block form and the smallest of the grid's kernels,
+# which read the general layout; a long reach has the slot form and no room
+@pytest.mark.parametrize("n,kind", [(n, k) for n in (1000, 65535, 65536) for k in
+                                    ("unsorted", "repeated", "offsets25", "scattered", "far")
+                                    if n > 1000 or k != "far"])
+@pytest.mark.parametrize("precision", ["f64", "mixed_krylov"])
+def test_cg_without_a_resident_form(n, kind, precision):
+    """CG on matrices that no resident team takes: right, and below the grid's
+    sizes without a copy of the matrix (two launches look at its offsets, one
+    solves)."""
+    import paper_2309_02156_gb300 as sa
+    rng = np.random.default_rng(n)
+    if kind == "far":
+        A = _spd(n, [1, n - 5000], rng)
+        arrays = A.indptr, A.indices, A.data
+    else:
+        A, arrays = _irregular(kind, n, rng)
+    b = rng.standard_normal(n)
+    seq = sa.Sequence(n, 2, 8, zeta=2, guess="zero", max_iters=500, krylov="cg", precision=precision)
+    Ad = sa.CSR(_dev(arrays[0], np.int32), _dev(arrays[1], np.int32), _dev(arrays[2], np.float64))
+    x = torch.zeros(n, dtype=torch.float64, device=DEV)
+    info = seq.solve(Ad, _dev(b, np.float64), 1e-12, x)
+    seq.close()
+    assert info["status"] == 0
+    assert np.linalg.norm(b - A @ x.cpu().numpy()) <= 1.01e-12 * np.linalg.norm(b)
+    if n < 65536 and precision == "f64":
+        assert info["launches"] == 3

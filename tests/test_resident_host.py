@@ -47,13 +47,10 @@ using namespace sa;
 static int bad = 0;
 #define CHECK(c) do { if (!(c)) { printf("line %d: %s\n", __LINE__, #c); bad = 1; } } while (0)
 
-// Layout of the FP64 grid team on 152 SMs, as launch_resident_cg makes it.
-static ResLayout grid_layout(int n, int W, int reach) {
-    const int ns = (n + 31) / 32;
-    int nblk = (ns + 3) / 4;
-    if (nblk > 152) nblk = 152;
+// Layout of the FP64 grid team.
+static ResLayout layout(int n, int W, int reach) {
     ResLayout L;
-    CHECK(res_layout(n, W, reach, nblk, 8, 232448 - 2048, &L));
+    CHECK(grid_layout(n, W, reach, 8, team_room(), &L));
     return L;
 }
 
@@ -102,6 +99,17 @@ static void counter_wraps() {
     }
 }
 
+// Room and launch agree: a solve is launched where it is said to fit.
+static void fits() {
+    for (int n : {33, 1000, 20000, 30000, 65000})
+        for (int reach : {0, 100, 9999, 14000, 16000, 28000, 40000}) {
+            if (reach >= n) continue;
+            CHECK(cg<SysF64>(n, reach) == resident_cg_fits(n, 5, reach, 8, team_room()));
+            CHECK(cg<SysF32>(n, reach) == resident_cg_fits(n, 5, reach, 4, team_room()));
+        }
+    CHECK(!cg<SysF64>(65000, 28000) && cg<SysF64>(65000, 9999));
+}
+
 // A launch that the driver refuses is no solve: the caller takes the streaming
 // kernels, and no error is left behind for its next check.
 static void refused() {
@@ -118,12 +126,13 @@ static void refused() {
 
 int main() {
     one_limit();
+    fits();
     refused();
     counter_wraps();
     // The sizes of the offset-view solves: x does not fit in shared memory.
-    CHECK(grid_layout(1001 * 1001, 5, 1001).x_in == 0);
-    CHECK(grid_layout(30000, 5, 14000).x_in == 0);
-    CHECK(grid_layout(30000, 5, 100).x_in == 1);
+    CHECK(layout(1001 * 1001, 5, 1001).x_in == 0);
+    CHECK(layout(30000, 5, 14000).x_in == 0);
+    CHECK(layout(30000, 5, 100).x_in == 1);
     return bad;
 }
 '''
