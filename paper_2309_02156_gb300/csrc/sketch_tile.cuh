@@ -168,7 +168,9 @@ __device__ __forceinline__ void sketch_team_tiles(
         }
         const int e0 = __shfl_sync(0xffffffffu, rs, 0);
         const int e1 = max(e0, __shfl_sync(0xffffffffu, re, max(wcnt - 1, 0)));
-        const bool staged = e1 - e0 <= kSkWarpStage;
+        // Row pointers that decrease may name entries outside [e0, e1): not staged.
+        const bool staged = e1 - e0 <= kSkWarpStage &&
+                            __all_sync(0xffffffffu, lane >= wcnt || (rs >= e0 && re <= e1));
         if (staged) {
             for (int e = e0 + lane; e < e1; e += 32) {
                 colW[e - e0] = __ldg(colind + e);

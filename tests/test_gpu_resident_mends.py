@@ -184,3 +184,33 @@ def test_cg_without_a_resident_form(n, kind, precision):
     assert np.linalg.norm(b - A @ x.cpu().numpy()) <= 1.01e-12 * np.linalg.norm(b)
     if n < 65536 and precision == "f64":
         assert info["launches"] == 3
+
+
+def test_sketch_with_row_pointers_that_decrease():
+    """Rows of entries that lie outside the span of their warp's first and last
+    row (an invalid matrix): read where the row pointers say, as elsewhere."""
+    import paper_2309_02156_gb300 as sa
+    from oracle import sketch
+    n, M, s, zeta, seed = 100, 3, 16, 4, 9
+    rng = np.random.default_rng(1)
+    A = _spd(n, [1, 7], rng)
+    ptr = A.indptr.copy()
+    ptr[4] += 100                # rows 3 and 61 run past their neighbours,
+    ptr[62] += 90
+    ptr[20] -= 60                # row 20 starts before them
+    cols = [rng.standard_normal(n) for _ in range(M)]
+    b = rng.standard_normal(n)
+    Y = np.zeros((n, M))
+    for i in range(n):
+        for e in range(ptr[i], max(ptr[i], ptr[i + 1])):
+            Y[i] += A.data[e] * np.array([c[A.indices[e]] for c in cols])
+    seq = sa.Sequence(n, M, s, zeta=zeta, seed=seed)
+    for c in cols:
+        seq.push(_dev(c, np.float64))
+    Ad = sa.CSR(_dev(ptr, np.int32), _dev(A.indices, np.int32), _dev(A.data, np.float64))
+    seq.guess(Ad, _dev(b, np.float64), torch.empty(n, dtype=torch.float64, device=DEV))
+    W, _ = seq.last_sketch()
+    seq.close()
+    S = sketch.sparse_sign_matrix(n, s, zeta, seed)
+    ref = S @ np.column_stack([Y, b])
+    assert np.all(np.abs(W.reshape(s, M + 1) - ref) <= 1e-11 * np.linalg.norm(ref, axis=0))
