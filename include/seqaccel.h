@@ -413,7 +413,8 @@ int seq_batch_set_schedule(seq_batch* batch, int32_t threads, int32_t blocks_per
  * column offsets run at most 512 threads per SM. */
 int seq_batch_set_cluster(seq_batch* batch, int32_t ctas, int32_t threads, int32_t order_kind);
 
-/* The schedule in use: out[0] threads per block, out[1] blocks per SM,
+/* The schedule in use: out[0] threads per block (those that run: fewer than were
+ * set where the patterns share their column offsets), out[1] blocks per SM,
  * out[2] order (0 largest first, 1 given), out[3] CTAs per sequence. */
 int seq_batch_get_schedule(const seq_batch* batch, int32_t* out);
 

@@ -214,3 +214,27 @@ def test_sketch_with_row_pointers_that_decrease():
     S = sketch.sparse_sign_matrix(n, s, zeta, seed)
     ref = S @ np.column_stack([Y, b])
     assert np.all(np.abs(W.reshape(s, M + 1) - ref) <= 1e-11 * np.linalg.norm(ref, axis=0))
+
+
+@pytest.mark.parametrize("regular", [True, False])
+def test_batch_reports_the_threads_that_run(regular):
+    """Patterns that share their column offsets run at most 512 threads per SM."""
+    import paper_2309_02156_gb300 as sa
+    rng = np.random.default_rng(5)
+    arrays = []
+    for n in (33, 3000, 5001):
+        A = _spd(n, [1, 70], rng)
+        arrays.append((A.indptr, A.indices, A.data) if regular else _irregular("unsorted", n, rng)[1])
+    bt = sa.Batch([(_dev(a[0], np.int32), _dev(a[1], np.int32)) for a in arrays], M=4, s=16)
+    for threads, per_sm in ((256, 1), (512, 1), (1024, 1), (512, 2), (1024, 2)):
+        bt.set_schedule(threads, per_sm, 0)
+        got = bt.schedule()
+        assert got["threads"] == (min(threads, 512 // per_sm) if regular else threads)
+        assert got["blocks_per_sm"] == per_sm
+    bt.set_cluster(4, 1024, 0)
+    assert bt.schedule()["threads"] == (512 if regular else 1024)
+    xs = [torch.zeros(len(a[0]) - 1, dtype=torch.float64, device=DEV) for a in arrays]
+    chosen = bt.autotune([_dev(a[2], np.float64) for a in arrays],
+                         [_dev(rng.standard_normal(len(a[0]) - 1), np.float64) for a in arrays], xs, 1e-8)
+    assert chosen["threads"] * chosen["blocks_per_sm"] <= (512 if regular else 1024)
+    bt.close()
