@@ -255,7 +255,7 @@ int build_sell(seq_ctx* ctx, const seq_csr* A) {
     // A CG that no resident team takes and that is too small for the grid's kernels
     // runs in one block, from the CSR arrays: nothing would read a copy.
     if (ctx->cfg.krylov == SEQ_CG && n < kGridCgMinRows &&
-        !(plan.W && resident_cg_fits_here(n, plan.W, plan.reach, el)))
+        !(plan.W && resident_cg_takes_here(n, plan.W, plan.reach, el)))
         return SEQ_OK;
     if (plan.W) {
         total = 32LL * ns * plan.W;

@@ -164,7 +164,7 @@ void launch_slot_fill_f32(const int* rowptr, const int* colind, const float* val
 constexpr int kClusterCgRows64 = 22528;
 constexpr int kClusterCgRows32 = 131072;
 struct TeamSlot;
-bool resident_cg_fits_here(int n, int W, int reach, size_t el);   // room on the current device
+bool resident_cg_takes_here(int n, int W, int reach, size_t el);   // on the current device
 constexpr int kTeamBlocks = 160;                                // most blocks of a grid team
 constexpr size_t kTeamSlotBytes = 16 * 2 * kTeamBlocks + 128;   // slots, counter
 // A whole GMRES solve by a resident grid (resident_gmres.cuh), up to these many

@@ -577,8 +577,8 @@ void launch_cg_block_f32(const DevArgs* a, KState* ks, float* r, float* p, float
     cg_block_kernel<SysF32><<<1, 1024, 0, st>>>(a, ks, r, p, q);
 }
 
-bool resident_cg_fits_here(int n, int W, int reach, size_t el) {
-    return resident_cg_fits(n, W, reach, el, team_room());
+bool resident_cg_takes_here(int n, int W, int reach, size_t el) {
+    return resident_cg_takes(n, W, reach, el, team_room());
 }
 
 bool launch_resident_cg_f64(const DevArgs* a, KState* ks, double* r, double* q, double* x, TeamSlot* slots,

@@ -220,14 +220,29 @@ inline bool grid_layout(int n, int W, int reach, size_t el, const TeamRoom& room
     return res_layout(n, W, reach, nblk < room.sms ? nblk : room.sms, el, room.budget, L);
 }
 
-// Whether a resident team has room for the solve.
-inline bool resident_cg_fits(int n, int W, int reach, size_t el, const TeamRoom& room) {
-    ResLayout L;
-    return (n <= cluster_rows(el) && res_layout(n, W, reach, 16, el, room.budget, &L)) ||
-           grid_layout(n, W, reach, el, room, &L);
+// Whether the streaming kernels are faster although the grid has room.  A block
+// forms the direction on the rows within reach too, at 1.0 ns per iteration for
+// each of those 2 reach rows in FP64 (256 threads); without them the grid is
+// 8.5 us + n / 128 ns ahead of the streaming kernels.  FP64, us per iteration,
+// streaming and resident: 262,144 rows, reach 512, 23.3 and 12.1, reach 4,096
+// (64^3) 25.0 and 20.5; 360,000 rows, reach 6,000, 26.5 and 26.0; 512,000 rows,
+// reach 6,400 (80^3), 31.9 and 32.5; 200,000 rows, reach 10,000, 21.8 and 31.4;
+// 1,000,000 rows, reach 1,000, 42.0 and 26.3, reach 8,000, 41.8 and 42.0, reach
+// 10,000 (100^3), 57.6 and 65.4; 3,240,000 rows, reach 1,800, 150 and 124.  In
+// FP32 the grid is ahead wherever it has room (1,000,000 rows, reach 10,000: 30.2
+// and 18.2), as it is of the one-block form that serves fewer rows.
+inline bool long_halo(int n, int reach, size_t el) {
+    return el == 8 && n >= kGridCgMinRows && 2LL * reach > 8500 + n / 128;
 }
 
-// Launch of one CG solve by a resident team; false when none fits or the driver
+// Whether a resident team takes the solve.
+inline bool resident_cg_takes(int n, int W, int reach, size_t el, const TeamRoom& room) {
+    ResLayout L;
+    return (n <= cluster_rows(el) && res_layout(n, W, reach, 16, el, room.budget, &L)) ||
+           (!long_halo(n, reach, el) && grid_layout(n, W, reach, el, room, &L));
+}
+
+// Launch of one CG solve by a resident team; false when none takes it or the driver
 // refuses the launch (the caller takes the streaming kernels).
 template <class Sys>
 static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r, typename Sys::T* q,
@@ -274,7 +289,7 @@ static bool launch_resident_cg(const DevArgs* a, KState* ks, typename Sys::T* r,
             cudaGetLastError();
         }
     }
-    if (!grid_layout(n, W, reach, sizeof(T), room, &L)) return false;
+    if (long_halo(n, reach, sizeof(T)) || !grid_layout(n, W, reach, sizeof(T), room, &L)) return false;
     const int nblk = (ns + L.per - 1) / L.per;
     auto k = resident_cg_grid_kernel<Sys>;
     const size_t bytes = res_bytes(L, W, sizeof(T));

@@ -238,3 +238,36 @@ def test_batch_reports_the_threads_that_run(regular):
                          [_dev(rng.standard_normal(len(a[0]) - 1), np.float64) for a in arrays], xs, 1e-8)
     assert chosen["threads"] * chosen["blocks_per_sm"] <= (512 if regular else 1024)
     bt.close()
+
+
+# both sides of every line in the choice of CG's form: cluster and grid (FP64 22,528
+# rows, FP32 131,072), one block and the grid's kernels (65,536), and the reach from
+# which FP64 takes the streaming kernels (4,524 at 70,000 rows)
+@pytest.mark.parametrize("n,offsets,precision", [
+    (22528, [1, 150], "f64"), (22529, [1, 150], "f64"), (131072, [1, 362], "mixed_krylov"),
+    (131073, [1, 362], "mixed_krylov"), (136900, [1, 370], "mixed_krylov"), (65535, [1, 5000], "f64"),
+    (65536, [1, 5000], "f64"), (70000, [1, 4523], "f64"), (70000, [1, 4524], "f64"),
+    (70000, [1, 4524], "mixed_krylov"), (262144, [1, 64, 4096], "f64"), (200000, [1, 10000], "f64")])
+def test_cg_at_the_lines_of_its_forms(n, offsets, precision):
+    import paper_2309_02156_gb300 as sa
+    rng = np.random.default_rng(n)
+    A = _spd(n, offsets, rng)
+    b = rng.standard_normal(n)
+    Ad, bd = _csr(A), _dev(b, np.float64)
+    for bad, status in ((None, 0), ("cap", 1), ("nan", -5), ("indefinite", -4)):
+        seq = sa.Sequence(n, 2, 8, zeta=2, guess="zero", krylov="cg", precision=precision,
+                          max_iters=3 if bad == "cap" else 500)
+        M, c = (_csr((-A).tocsr()), bd) if bad == "indefinite" else (Ad, bd.clone())
+        if bad == "nan":
+            c[n // 2] = float("nan")
+        x = torch.zeros_like(bd)
+        if status < 0:
+            with pytest.raises(sa.SeqError) as e:
+                seq.solve(M, c, 1e-12, x)
+            assert e.value.code == status
+        else:
+            info = seq.solve(M, c, 1e-12, x)
+            r = np.linalg.norm(b - A @ x.cpu().numpy()) / np.linalg.norm(b)
+            assert info["status"] == status
+            assert r <= 1.01e-12 if status == 0 else info["iters"] == 3
+        seq.close()

@@ -99,15 +99,20 @@ static void counter_wraps() {
     }
 }
 
-// Room and launch agree: a solve is launched where it is said to fit.
-static void fits() {
-    for (int n : {33, 1000, 20000, 30000, 65000})
-        for (int reach : {0, 100, 9999, 14000, 16000, 28000, 40000}) {
+// Rule and launch agree: a solve is launched where a team is said to take it.
+static void takes() {
+    for (int n : {33, 1000, 20000, 30000, 65000, 65536, 262144, 1000000})
+        for (int reach : {0, 100, 4000, 5000, 6000, 9999, 14000, 16000, 28000, 40000}) {
             if (reach >= n) continue;
-            CHECK(cg<SysF64>(n, reach) == resident_cg_fits(n, 5, reach, 8, team_room()));
-            CHECK(cg<SysF32>(n, reach) == resident_cg_fits(n, 5, reach, 4, team_room()));
+            CHECK(cg<SysF64>(n, reach) == resident_cg_takes(n, 5, reach, 8, team_room()));
+            CHECK(cg<SysF32>(n, reach) == resident_cg_takes(n, 5, reach, 4, team_room()));
         }
     CHECK(!cg<SysF64>(65000, 28000) && cg<SysF64>(65000, 9999));
+    // the line of the long reaches: 64^3, 80^3, 100^3, flat grids; FP32 has none
+    CHECK(cg<SysF64>(262144, 4096) && !cg<SysF64>(512000, 6400) && !cg<SysF64>(1000000, 10000));
+    CHECK(cg<SysF64>(1000000, 8000) && !cg<SysF64>(200000, 10000) && cg<SysF64>(65535, 10000));
+    CHECK(cg<SysF64>(70000, 4523) && !cg<SysF64>(70000, 4524));
+    CHECK(cg<SysF32>(512000, 6400) && cg<SysF32>(1000000, 10000) && cg<SysF32>(200000, 10000));
 }
 
 // A launch that the driver refuses is no solve: the caller takes the streaming
@@ -126,7 +131,7 @@ static void refused() {
 
 int main() {
     one_limit();
-    fits();
+    takes();
     refused();
     counter_wraps();
     // The sizes of the offset-view solves: x does not fit in shared memory.
