@@ -24,17 +24,14 @@
 #include <vector>
 
 #include "../../include/seqaccel.h"
+#include "batch_layout.cuh"
 #include "common.cuh"
 #include "internal.h"
 #include "resident.cuh"
-#include "sketch_tile.cuh"
 
 namespace sa {
 namespace {
 
-constexpr int kBatchMaxM = 16;
-constexpr int kBatchMaxS = 64;
-constexpr int kSketchTeams = 4;           // teams of four warps that sketch a sequence
 constexpr double kTheta = 0.5;
 constexpr int kOk = 0;
 
@@ -99,26 +96,20 @@ __device__ __forceinline__ Acc row_dot(const int* __restrict__ rowptr, const int
     return acc;
 }
 
-// Doubles of the sketch's workspace: the teams' regions and FP64 accumulators.
-__host__ __device__ inline size_t sketch_ws_doubles(int s, int ncol) {
-    return kSketchTeams * (sketch_team_bytes(s, ncol) / 8 + (size_t)s * ncol);
-}
-
 // The sketched block W (s x (M+1), physical history slots, b last) of the
-// sequence's slices [s_lo, s_hi), summed into Wsum (shared).  The tiles, the
+// sequence's slices [s_lo, s_hi), in shared memory (returned).  The tiles, the
 // products spread over all lanes and the exact fixed-point additions are those
 // of the single-sequence kernel; a team's integers go to its FP64 accumulator
 // every kSkMaxTiles tiles, and the teams are added in order.  FP64 additions per
 // row and sketch entry, as before, held the FP64 pipe for 512 of the 832 cycles
 // a row took: 8 sequences of 122,500 rows in clusters of 8, guess 3.5 -> 1.8 ms.
-__device__ void block_sketch(const BatchSeq& q, double* ws, double* Wsum, int& bad, int s_lo,
-                             int s_hi) {
+__device__ double* block_sketch(const BatchSeq& q, double* ws, int& bad, int s_lo, int s_hi) {
     __shared__ int zk[kMaxZeta * (kBatchMaxM + 1)];
     const int ncol = q.M + 1, wsz = q.s * ncol;
     const int nt = min(kSketchTeams, (int)blockDim.x / kSkTeamThreads);
     const int team = threadIdx.x / kSkTeamThreads, tt = threadIdx.x % kSkTeamThreads;
     const size_t tb = sketch_team_bytes(q.s, ncol) / 8;
-    double* acc = ws + kSketchTeams * tb;
+    double* acc = ws + sketch_regions_doubles(q.s, ncol);
     sketch_pairs(zk, q.zeta, ncol);
     for (int i = threadIdx.x; i < nt * wsz; i += blockDim.x) acc[i] = 0.0;
     __syncthreads();
@@ -146,9 +137,10 @@ __device__ void block_sketch(const BatchSeq& q, double* ws, double* Wsum, int& b
     for (int i = threadIdx.x; i < wsz; i += blockDim.x) {
         double t = acc[i];
         for (int w = 1; w < nt; ++w) t += acc[(size_t)w * wsz + i];
-        Wsum[i] = t * inv;
+        acc[i] = t * inv;
     }
     __syncthreads();
+    return acc;
 }
 
 // Column-scaled, pivoted Householder least squares of the s x m block (the
@@ -830,16 +822,6 @@ __device__ __noinline__ int resident_cg32(const BatchSeq& q, double itol, int ma
     return it;
 }
 
-// Shared-memory bytes of one block for sequences with at most s rows of
-// sketch and M history columns.
-size_t batch_smem_bytes(int s, int M) {
-    const int ncol = M + 1, wsz = s * ncol;
-    const size_t d = sketch_ws_doubles(s, ncol) + wsz + (2 * s * M + 3 * s + 5 * M) + kBatchMaxM;
-    const size_t guess = d * sizeof(double);
-    const size_t stage = sizeof(double) * 32 * (size_t)kTileChunks * 32;   // up to 32 warps
-    return guess > stage ? guess : stage;
-}
-
 // One time step of every sequence.  Blocks take sequences from the queue
 // until it is empty; each sequence is processed by one block from start to
 // end (no inter-block waiting).  MAXT: the largest block size the
@@ -876,13 +858,12 @@ batched_step_kernel(BatchSeq* seqs, const int* __restrict__ order, int count, in
         int bad = 0, rank = 0;
         double rho = 0.0;
         // 1. guess
-        double* Wsum = smem + sketch_ws_doubles(s, M + 1);
-        double* ws = Wsum + s * (M + 1);
-        double* yphys = ws + (2 * s * M + 3 * s + 5 * M);
+        double* ws = smem;                     // batch_layout.cuh
+        double* yphys = ws + lsq_ws_doubles(s, M);
         if (m == 0) {
             for (int i = tid; i < n; i += bd) q.x[i] = 0.0;
         } else {
-            block_sketch(q, smem, Wsum, bad, 0, (n + 31) >> 5);
+            const double* Wsum = block_sketch(q, smem, bad, 0, (n + 31) >> 5);
             block_lsq(Wsum, s, M, m, (q.pushes - m) % M, 1e-12, ws, yphys, &rank, &rho);
             for (int i = tid; i < n; i += bd) {
                 const double* row = q.X + (size_t)i * q.ldx;
@@ -967,16 +948,6 @@ batched_step_kernel(BatchSeq* seqs, const int* __restrict__ order, int count, in
     }
 }
 
-// Shared-memory bytes of one CTA of the cluster form: the single-block layout
-// plus the cluster total of W.
-size_t batch_cluster_smem_bytes(int s, int M) {
-    const size_t base = batch_smem_bytes(s, M);
-    const int wsz = s * (M + 1);
-    const size_t d = sketch_ws_doubles(s, M + 1) + wsz + (2 * s * M + 3 * s + 5 * M) + kBatchMaxM;
-    const size_t need = (d + (size_t)wsz) * sizeof(double);
-    return base > need ? base : need;
-}
-
 // One time step of every sequence, one cluster per sequence (see cl_sync and
 // cl_total above).  The steps and their arithmetic are those of
 // batched_step_kernel; rows are split over the cluster's CTAs and block
@@ -1020,14 +991,13 @@ batched_cluster_kernel(BatchSeq* seqs, const int* __restrict__ order, int count,
         double rho = 0.0;
         // 1. guess
         const int ncol = M + 1, wsz = s * ncol;
-        double* Wsum = smem + sketch_ws_doubles(s, ncol);
-        double* ws = Wsum + wsz;
-        double* yphys = ws + (2 * s * M + 3 * s + 5 * M);
+        double* ws = smem;                     // batch_layout.cuh
+        double* yphys = ws + lsq_ws_doubles(s, M);
         double* Wtot = yphys + kBatchMaxM;
         if (m == 0) {
             for (int i = r_lo + tid; i < r_hi; i += bd) q.x[i] = 0.0;
         } else {
-            block_sketch(q, smem, Wsum, bad, s_lo, s_hi);
+            const double* Wsum = block_sketch(q, smem, bad, s_lo, s_hi);
             cl_sync();
             for (int i = tid; i < wsz; i += bd) {
                 double t = 0.0;
@@ -1161,7 +1131,6 @@ struct seq_batch {
     int threads = 512, blocks_per_sm = 1, order_kind = 0;  // 0: largest first, 1: given order
     int run_threads = 512;                // threads of the captured launch (step_launch)
     int cluster = 1;                      // CTAs per sequence (1: one block per sequence)
-    size_t smem_cluster = 0;              // least shared memory of a CTA (cluster form)
     int autopush = 1;
     cudaGraphExec_t graph = nullptr;
     size_t smem = 0;                      // least shared memory of a block
@@ -1223,7 +1192,7 @@ struct StepLaunch {
 StepLaunch step_launch(const seq_batch* bt) {
     const bool cl = bt->cluster > 1;
     const int bps = bt->blocks_per_sm;
-    const size_t need = cl ? bt->smem_cluster : bt->smem;
+    const size_t need = bt->smem;
     const int fewer = std::min(bt->threads, 512 / bps);
     const bool small = fewer * bps <= 256;
     const StepKernel kern = cl ? (small ? batched_cluster_kernel<256, true>
@@ -1388,7 +1357,6 @@ int seq_batch_create(int32_t count, const seq_csr* patterns, int32_t M, int32_t 
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&bt->sms, cudaDevAttrMultiProcessorCount, dev);
     bt->smem = batch_smem_bytes(s, M);
-    bt->smem_cluster = batch_cluster_smem_bytes(s, M);
     bt->host.resize(count);
     int rc = SEQ_OK;
     const int ldx = (M + 1) & ~1;
@@ -1561,8 +1529,7 @@ int seq_batch_autotune(seq_batch* bt, const double* const* values, const double*
             for (int ti = 0; ti < 3; ++ti) {
                 for (int bps = 1; bps <= 2; ++bps) {
                     if (cl > 1 && (bps > 1 || thr[ti] < 512)) continue;
-                    const size_t need = cl > 1 ? bt->smem_cluster : bt->smem;
-                    if ((size_t)bps * need > 220 * 1024) continue;
+                    if ((size_t)bps * bt->smem > 220 * 1024) continue;
                     bt->threads = thr[ti];
                     bt->blocks_per_sm = bps;
                     bt->order_kind = oi;

@@ -271,3 +271,37 @@ def test_cg_at_the_lines_of_its_forms(n, offsets, precision):
             assert info["status"] == status
             assert r <= 1.01e-12 if status == 0 else info["iters"] == 3
         seq.close()
+
+
+@pytest.mark.parametrize("schedule", [(1, 1024), (2, 512), ("cluster", 4)])
+@pytest.mark.parametrize("regular", [True, False])
+def test_batch_guess_of_the_largest_sketch(schedule, regular):
+    """M = 16, s = 64, the largest workspace: solutions within the span of the
+    history are found by the guess (64 random rows of 16 random columns: condition
+    of a few, so to a thousand roundings), and by one sketch column less."""
+    import paper_2309_02156_gb300 as sa
+    for M, s in ((16, 64), (15, 63)):
+        rng = np.random.default_rng(M)
+        arrays, hist, bs = [], [], []
+        for n in (64, 1000, 5001):
+            A = _spd(n, [1, 7], rng)
+            X = rng.standard_normal((n, M))
+            arrays.append((A.indptr, A.indices, A.data) if regular else _irregular("unsorted", n, rng)[1])
+            if not regular:
+                p, c, v = arrays[-1]
+                A = sp.csr_matrix((v, c, p), shape=(n, n))
+            hist.append(X)
+            bs.append(A @ (X @ rng.standard_normal(M)))
+        bt = sa.Batch([(_dev(a[0], np.int32), _dev(a[1], np.int32)) for a in arrays], M=M, s=s)
+        if schedule[0] == "cluster":
+            bt.set_cluster(schedule[1], 512, 0)
+        else:
+            bt.set_schedule(schedule[1], schedule[0], 0)
+        for k, X in enumerate(hist):
+            for j in range(M):
+                bt.push(k, _dev(X[:, j], np.float64))
+        xs = [_dev(np.zeros(len(b)), np.float64) for b in bs]
+        infos = bt.step([_dev(a[2], np.float64) for a in arrays], [_dev(b, np.float64) for b in bs], xs, 1e-8)
+        bt.close()
+        for i in infos:
+            assert i["status"] == 0 and i["iters"] == 0 and i["guess_relres"] <= 1e3 * 2.0 ** -52

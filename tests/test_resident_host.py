@@ -157,3 +157,37 @@ def test_host_decisions(tmp_path):
     assert r.returncode == 0, r.stderr
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout
+
+
+BATCH = r'''
+#include <cstdio>
+#include "batch_layout.cuh"
+using namespace sa;
+int main() {
+    int bad = 0;
+    for (int M = 1; M <= kBatchMaxM; ++M)
+        for (int s = 1; s <= kBatchMaxS; ++s) {
+            // two blocks on an SM (228 KB, 1 KB of each reserved, 4 KB for static arrays)
+            if (2 * (batch_smem_bytes(s, M) + 5 * 1024) > 228 * 1024) bad = printf("room: %d %d\n", M, s);
+            // what follows the sketch lies below its sum
+            if (after_sketch_doubles(s, M) > sketch_regions_doubles(s, M + 1)) bad = printf("over: %d %d\n", M, s);
+        }
+    return bad != 0;
+}
+'''
+
+
+def test_two_batch_blocks_fit_on_an_sm(tmp_path):
+    """Every size of a batch leaves room for the two blocks per SM that a schedule
+    may name."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    src, exe = tmp_path / "batch.cu", tmp_path / "batch"
+    src.write_text(BATCH)
+    r = subprocess.run([nvcc, "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-I",
+                        os.path.join(ROOT, "paper_2309_02156_gb300", "csrc"), str(src), "-o", str(exe)],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout
