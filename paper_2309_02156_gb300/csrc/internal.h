@@ -168,12 +168,15 @@ bool resident_cg_takes_here(int n, int W, int reach, size_t el);   // on the cur
 constexpr int kTeamBlocks = 160;                                // most blocks of a grid team
 constexpr size_t kTeamSlotBytes = 16 * 2 * kTeamBlocks + 128;   // slots, counter
 // A whole GMRES solve by a resident grid (resident_gmres.cuh), up to these many
-// rows: above them the streaming kernels of the cycle graph use the chip as well
-// and their launches weigh less.  Per Arnoldi step (cycle graph, resident), us:
-// FP64 10,000 rows 39.7, 27.3; 40,000 45.4, 35.2; 90,000 47.1, 42.2; 131,044
-// 53.2, 54.2.  FP32 22,500 rows 25.6, 21.1; 131,044 30.3, 25.2; 160,000 31,
-// 26.8 (near 200,000 rows the basis fills the shared memory).  FP32 with eight
-// Chebyshev sweeps 40,000 rows 50.2, 44.0; 90,000 50.6, 52.0.
+// rows and within a reach (long_fetch): above them the streaming kernels of the
+// cycle graph use the chip as well and their launches weigh less.  Per Arnoldi
+// step of full cycles (cycle graph, resident), us: FP64 10,000 rows 35.5, 26.3;
+// 56,000 37.6, 34.3; 77,000 39.2, 36.9; 92,000 40.8, 41.5.  FP32 10,000 rows 19.8,
+// 19.4; 56,000 21.5, 20.3; 110,000 22.5, 22.2; 150,000 23.5, 23.5; 190,000 24.0,
+// 25.9; eight Chebyshev sweeps 10,000 rows 38.7, 39.2; 56,000 40.8, 43.3.  Solves
+// whose last cycle ends early gain more (eight iterations, FP32: 190,000 rows 373
+// and 318 us; eight sweeps, 56,000 rows, 703 and 525): the line lies where a full
+// cycle's step is a twentieth slower.
 constexpr int kResGmresRows64 = 92160;
 constexpr int kResGmresRows32 = 196608;
 constexpr int kResGmresRows32Pre = 73728;

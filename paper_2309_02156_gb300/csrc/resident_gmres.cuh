@@ -554,6 +554,29 @@ resident_gmres_kernel(const DevArgs* __restrict__ a, KState* ks,
     }
 }
 
+// Whether the streaming kernels are faster although the size fits.  Every block
+// fetches the neighbours' rows of every product's vector, 2 reach of them and one
+// product per sweep and one for the step: 1.4 to 2 us for 1,000 rows of reach.
+// What a step has to spend on that: in FP64 9 us where a block has at most eight
+// slices (one pass of its warps), 3 us up to sixteen (1.6 with more than
+// five offsets), above that nothing once there are sweeps; in FP32 1.5 us.  Per step of full cycles, streaming and
+// resident, us (five offsets): FP64 10,000 rows, reach 4,000, 35.5 and 33.8;
+// 56,000 rows, reach 1,500, 37.6 and 35.6; 85,184 rows, reach 1,936 (44^3), 40.4
+// and 45.5; four sweeps 22,500 rows, reach 1,500, 48.4 and 47.4, reach 3,000 48.4
+// and 58.7; eight sweeps 10,000 rows, reach 1,000, 61.1 and 60.3, reach 2,000 61.2
+// and 76.3; 77,000 rows, reach 277, 69.2 and 72.4; 56,000 rows, reach 236, nine
+// offsets, 65.6 and 74.9; 92,000 rows, reach 303, 73.3 and 84.9.  FP32 22,500 rows, reach 1,500, 20.1 and 21.5, reach 3,000 20.2 and
+// 25.1; eight sweeps 36,864 rows, reach 192, 39.5 and 42.2, reach 1,000 39.8 and
+// 52.3, 10,000 rows, reach 4,000, 39.3 and 98.8.  A cycle that ends early costs the
+// streaming kernels the launches of the rest: eight iterations with eight sweeps,
+// 56,000 rows, reach 236, FP64 860 and 613, FP32 703 and 525, so a step may cost up
+// to a twentieth more.
+inline bool long_fetch(int W, int reach, int sweeps, int per, size_t el) {
+    const long long rows = (sweeps + 1LL) * reach;
+    if (el == 4) return rows > (sweeps > 0 ? 2500 : 1800);
+    return rows > (per <= 8 ? 9000 : per <= 16 ? (W <= 5 ? 3000 : 1600) : sweeps <= 1 ? 1000 : 0);
+}
+
 // Launch of a whole GMRES solve by a resident grid; false when the size does not
 // fit or the driver refuses the launch (the caller takes the cycle graph).
 template <class Sys>
@@ -574,7 +597,8 @@ static bool launch_resident_gmres(const DevArgs* a, KState* ks, const GmresArgs<
     GmresLayout L;
     const size_t budget = (size_t)optin - 20480;   // less the static arrays; also the kernel's limit
     if (!gmres_layout(n, plan.W, plan.reach, nblk, A.R, A.sweeps, sizeof(T), budget, &L)) return false;
-    if (n > (sizeof(T) == 8 ? kResGmresRows64 : A.sweeps > 0 ? kResGmresRows32Pre : kResGmresRows32))
+    if (n > (sizeof(T) == 8 ? kResGmresRows64 : A.sweeps > 0 ? kResGmresRows32Pre : kResGmresRows32) ||
+        long_fetch(plan.W, plan.reach, A.sweeps, L.per, sizeof(T)))
         return false;
     nblk = (ns + L.per - 1) / L.per;
     int threads = 32 * L.per;

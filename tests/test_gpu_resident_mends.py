@@ -305,3 +305,45 @@ def test_batch_guess_of_the_largest_sketch(schedule, regular):
         bt.close()
         for i in infos:
             assert i["status"] == 0 and i["iters"] == 0 and i["guess_relres"] <= 1e3 * 2.0 ** -52
+
+
+# both sides of every line between the resident GMRES and the cycle graph (the last
+# column: one launch per solve)
+@pytest.mark.parametrize("n,reach,sweeps,precision,resident", [
+    (92160, 303, 0, "f64", True), (92161, 303, 0, "f64", False), (38913, 3000, 0, "f64", True),
+    (38913, 3001, 0, "f64", False), (77825, 1000, 0, "f64", True), (77825, 1001, 0, "f64", False),
+    (30000, 1000, 8, "f64", True), (30000, 1001, 8, "f64", False), (40000, 333, 8, "f64", True),
+    (40000, 334, 8, "f64", False), (77824, 277, 8, "f64", True), (77825, 277, 8, "f64", False),
+    (20000, 1800, 0, "mixed_krylov", True), (20000, 1801, 0, "mixed_krylov", False),
+    (196608, 443, 0, "mixed_krylov", True), (196609, 443, 0, "mixed_krylov", False),
+    (20000, 277, 8, "mixed_krylov", True), (20000, 278, 8, "mixed_krylov", False),
+    (73728, 271, 8, "mixed_krylov", True), (73729, 271, 8, "mixed_krylov", False)])
+@pytest.mark.parametrize("kind", ["jacobi", "chebyshev"])
+def test_gmres_at_the_lines_of_its_forms(n, reach, sweeps, precision, resident, kind):
+    import paper_2309_02156_gb300 as sa
+    if not sweeps and kind == "chebyshev":
+        pytest.skip("no sweeps")
+    rng = np.random.default_rng(n + reach)
+    A = _spd(n, [1, reach], rng)
+    b = rng.standard_normal(n)
+    Ad, bd = _csr(A), _dev(b, np.float64)
+    for bad, status in ((None, 0), ("cap", 1), ("nan", -5)):
+        seq = sa.Sequence(n, 2, 8, zeta=2, guess="zero", krylov="gmres", precision=precision,
+                          max_iters=3 if bad == "cap" else 500, precond_sweeps=sweeps, precond_kind=kind)
+        c = bd.clone()
+        if bad == "nan":
+            c[n // 2] = float("nan")
+        x = torch.zeros_like(bd)
+        if status < 0:
+            with pytest.raises(sa.SeqError) as e:
+                seq.solve(Ad, c, 1e-12, x)
+            assert e.value.code == status
+        else:
+            info = seq.solve(Ad, c, 1e-12, x)
+            r = np.linalg.norm(b - A @ x.cpu().numpy()) / np.linalg.norm(b)
+            assert (info["launches"] < 100) == resident
+            if bad == "cap" and info["status"] == 0:      # three iterations were enough
+                status = 0
+            assert info["status"] == status
+            assert r <= 1.01e-12 if status == 0 else r > 1e-12 and info["iters"] == 3
+        seq.close()

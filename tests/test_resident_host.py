@@ -191,3 +191,38 @@ def test_two_batch_blocks_fit_on_an_sm(tmp_path):
     assert r.returncode == 0, r.stderr
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout
+
+
+# Lines of the resident GMRES: the sizes, and the reach at which fetching the
+# neighbours' rows costs more than the streaming kernels' launches.
+GMRES_LINES = r'''
+int main() {
+    CHECK(gmres<SysF64>(10000, 4500, 0) && gmres<SysF64>(92160, 303, 0) && !gmres<SysF64>(92161, 303, 0));
+    CHECK(gmres<SysF64>(38912, 3001, 0) && gmres<SysF64>(38913, 3000, 0) && !gmres<SysF64>(38913, 3001, 0));
+    CHECK(gmres<SysF64>(77825, 1000, 0) && !gmres<SysF64>(77825, 1001, 0));
+    CHECK(gmres<SysF64>(30000, 1000, 8) && !gmres<SysF64>(30000, 1001, 8));
+    CHECK(gmres<SysF64>(40000, 333, 8) && !gmres<SysF64>(40000, 334, 8));
+    CHECK(gmres<SysF64>(77824, 279, 8) && !gmres<SysF64>(77825, 279, 8) && gmres<SysF64>(77825, 279, 1));
+    CHECK(!long_fetch(9, 177, 8, 16, 8) && long_fetch(9, 178, 8, 16, 8) && !long_fetch(5, 178, 8, 16, 8));
+    CHECK(gmres<SysF32>(20000, 1800, 0) && !gmres<SysF32>(20000, 1801, 0));
+    CHECK(gmres<SysF32>(196608, 443, 0) && !gmres<SysF32>(196609, 443, 0));
+    CHECK(gmres<SysF32>(20000, 277, 8) && !gmres<SysF32>(20000, 278, 8));
+    CHECK(gmres<SysF32>(73728, 271, 8) && !gmres<SysF32>(73729, 271, 8));
+    return bad;
+}
+'''
+
+
+def test_gmres_lines(tmp_path):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    src, exe = tmp_path / "lines.cu", tmp_path / "lines"
+    src.write_text(PROGRAM.split("int main()")[0] + GMRES_LINES)
+    r = subprocess.run([nvcc, "-std=c++17", "--expt-relaxed-constexpr", "-gencode",
+                        "arch=compute_103a,code=sm_103a", "-I",
+                        os.path.join(ROOT, "paper_2309_02156_gb300", "csrc"), str(src), "-o", str(exe)],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout
