@@ -1,7 +1,8 @@
-// Shared memory of a block of the batched step while it forms the guess.
+// Shared memory of a block of the batched step: the guess, then the resident CG.
 #pragma once
 
 #include "common.cuh"
+#include "resident.cuh"
 #include "sketch_tile.cuh"
 
 namespace sa {
@@ -31,6 +32,19 @@ inline size_t batch_smem_bytes(int s, int M) {
     const size_t guess = 8 * (sketch_regions_doubles(s, ncol) + kSketchTeams * (size_t)s * ncol);
     const size_t stage = sizeof(double) * 32 * (size_t)kTileChunks * 32;   // up to 32 warps
     return guess > stage ? guess : stage;
+}
+
+// Layout of a sequence's resident CG over `ctas` CTAs; false: it takes the form
+// whose vectors lie in global memory.  A CTA of a cluster also forms the direction
+// on the rows within reach on both sides: with more of those than rows of its own
+// it is slower for it (clusters of 8 and of 4, 64 sequences, ms a step, global
+// form and resident: 10,000 rows, reach 5,000, 1.12 and 1.41, 0.67 and 0.74, reach
+// 2,000 1.19 and 1.26, 0.71 and 0.72, reach 100 1.17 and 1.11, 0.70 and 0.65;
+// 64,000 rows, reach 1,600, 3.02 and 2.83, 2.37 and 2.23).
+__host__ __device__ inline bool batch_resident(int n, int W, int reach, int ctas, size_t budget,
+                                               ResLayout* L) {
+    return res_layout(n, W, reach, ctas, sizeof(float), budget, L) &&
+           (ctas == 1 || 2LL * reach <= 32LL * L->per);
 }
 
 }  // namespace sa

@@ -27,7 +27,6 @@
 #include "batch_layout.cuh"
 #include "common.cuh"
 #include "internal.h"
-#include "resident.cuh"
 
 namespace sa {
 namespace {
@@ -878,7 +877,7 @@ batched_step_kernel(BatchSeq* seqs, const int* __restrict__ order, int count, in
         double* stage_d = smem;
         ResLayout L;
         const bool resident =
-            RES && q.slot && res_layout(n, q.slot_w, q.reach, 1, 4, smem_bytes, &L);
+            RES && q.slot && batch_resident(n, q.slot_w, q.reach, 1, smem_bytes, &L);
         const int lane = tid & 31, warp = tid >> 5, nw = bd >> 5;
         // 2. FP64 refinement around FP32 CG
         double bb_l = 0.0;
@@ -1018,7 +1017,7 @@ batched_cluster_kernel(BatchSeq* seqs, const int* __restrict__ order, int count,
         double* stage_d = smem;
         ResLayout L;
         const bool resident =
-            RES && q.slot && res_layout(n, q.slot_w, q.reach, (int)nr, 4, smem_bytes, &L);
+            RES && q.slot && batch_resident(n, q.slot_w, q.reach, (int)nr, smem_bytes, &L);
         const int lane = tid & 31, warp = tid >> 5, nw = bd >> 5;
         // 2. FP64 refinement around FP32 CG (the x of other CTAs is complete
         // after the cluster total below)
@@ -1217,7 +1216,7 @@ StepLaunch step_launch(const seq_batch* bt) {
         if (!q.slot) continue;
         slot += q.n;
         if (most >= (long long)need &&
-            res_layout(q.n, q.slot_w, q.reach, bt->cluster, sizeof(float), (size_t)most, &L))
+            batch_resident(q.n, q.slot_w, q.reach, bt->cluster, (size_t)most, &L))
             fits += q.n;
     }
     if (fits >= 0.6 * all) return {kern, (size_t)most, fewer};

@@ -347,3 +347,25 @@ def test_gmres_at_the_lines_of_its_forms(n, reach, sweeps, precision, resident, 
             assert info["status"] == status
             assert r <= 1.01e-12 if status == 0 else r > 1e-12 and info["iters"] == 3
         seq.close()
+
+
+@pytest.mark.parametrize("ctas,reaches", [(8, (600, 1280, 1281, 5000)), (4, (2560, 2561)), (1, (9999, 10001))])
+def test_batch_with_long_reaches(ctas, reaches):
+    """Reaches at both sides of half a CTA's rows (20,480 rows: 2,560 a CTA of 8)."""
+    import paper_2309_02156_gb300 as sa
+    rng = np.random.default_rng(ctas)
+    n = 20480
+    for r in reaches:
+        A = _spd(n, [1, r], rng)
+        bs = [rng.standard_normal(n) for _ in range(3)]
+        bt = sa.Batch([(_dev(A.indptr, np.int32), _dev(A.indices, np.int32))] * 3, M=2, s=8, zeta=2)
+        if ctas > 1:
+            bt.set_cluster(ctas, 512, 0)
+        else:
+            bt.set_schedule(512, 1, 0)
+        xs = [_dev(np.zeros(n), np.float64) for _ in bs]
+        infos = bt.step([_dev(A.data, np.float64)] * 3, [_dev(b, np.float64) for b in bs], xs, 1e-11)
+        bt.close()
+        for b, x, i in zip(bs, xs, infos):
+            assert i["status"] == 0
+            assert np.linalg.norm(b - A @ x.cpu().numpy()) <= 1.01e-11 * np.linalg.norm(b)

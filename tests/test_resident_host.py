@@ -172,6 +172,11 @@ int main() {
             // what follows the sketch lies below its sum
             if (after_sketch_doubles(s, M) > sketch_regions_doubles(s, M + 1)) bad = printf("over: %d %d\n", M, s);
         }
+    // a cluster's CTAs keep a sequence on the chip up to a reach of half their rows
+    ResLayout L;
+    const size_t room = 220 * 1024;
+    if (!batch_resident(20480, 5, 1280, 8, room, &L) || batch_resident(20480, 5, 1281, 8, room, &L) ||
+        !batch_resident(3000, 5, 1499, 1, room, &L)) bad = printf("reach");
     return bad != 0;
 }
 '''
