@@ -179,13 +179,14 @@ int seq_guess(seq_ctx* ctx, const seq_csr* A, const double* b_dev,
  * is one restart cycle).  CG runs as one launch with its vectors on the chip
  * where the matrix's rows share their column offsets (stencils, bands): a
  * thread-block cluster for small n, a cooperative grid above.  Other matrices
- * take one thread block for n < 65,536 and the whole GPU above (three kernels
- * per iteration, captured as a CUDA graph of 16 iterations); the algorithm and
- * its stopping test are the same.  GMRES on such matrices up to about 90,000
- * rows (FP32 inner solves: 70,000 to 200,000) is one launch too, with its basis
- * on the chip.  With b = 0 the
- * test is ||b - A x|| <= 0 and x = 0 passes it.  Does not push x.
- * Synchronises.
+ * (and long reaches |column - row| where that is faster) take one thread block
+ * for n < 65,536 and the whole GPU above (three kernels per iteration, captured
+ * as a CUDA graph of 16 iterations); the algorithm and its stopping test are the
+ * same.  GMRES on such matrices up to about 90,000 rows (FP32 inner solves:
+ * 70,000 to 200,000), less with a long reach or many sweeps, is one launch too,
+ * with its basis on the chip.  A launch of these forms that the driver refuses
+ * falls back to the others.  With b = 0 the test is ||b - A x|| <= 0 and x = 0
+ * passes it.  Does not push x.  Synchronises.
  * Errors: SEQ_EINVAL, SEQ_EBREAKDOWN (CG p^T A p <= 0, singular Hessenberg),
  * SEQ_ENONFINITE (NaN or Inf met), SEQ_ETIMEOUT (host cycle bound, or a bounded
  * wait between thread blocks ran out), SEQ_ECUDA. */
@@ -407,10 +408,10 @@ int seq_batch_set_schedule(seq_batch* batch, int32_t threads, int32_t blocks_per
  * distributed shared memory (same steps and arithmetic, rows split).  Fewer
  * sequences are in flight at once, so their working sets stay in L2 between
  * CG iterations, or in the CTAs' shared memory where the patterns' rows share
- * their column offsets and the CTAs have room.  ctas = 1 is the one-block
- * schedule with `threads`.  The autotuner also tries clusters of 4 and 8 (512
- * and 1024 threads).  In every schedule blocks whose patterns share their
- * column offsets run at most 512 threads per SM. */
+ * their column offsets, the CTAs have room and the reach is at most half a CTA's
+ * rows.  ctas = 1 is the one-block schedule with `threads`.  The autotuner also
+ * tries clusters of 4 and 8 (512 and 1024 threads).  In every schedule blocks
+ * whose patterns share their column offsets run at most 512 threads per SM. */
 int seq_batch_set_cluster(seq_batch* batch, int32_t ctas, int32_t threads, int32_t order_kind);
 
 /* The schedule in use: out[0] threads per block (those that run: fewer than were
