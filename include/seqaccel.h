@@ -411,7 +411,8 @@ int seq_batch_set_schedule(seq_batch* batch, int32_t threads, int32_t blocks_per
  * their column offsets, the CTAs have room and the reach is at most half a CTA's
  * rows.  ctas = 1 is the one-block schedule with `threads`.  The autotuner also
  * tries clusters of 4 and 8 (512 and 1024 threads).  In every schedule blocks
- * whose patterns share their column offsets run at most 512 threads per SM. */
+ * whose patterns share five column offsets at most, or whose vectors fit on the
+ * chip, run at most 512 threads per SM. */
 int seq_batch_set_cluster(seq_batch* batch, int32_t ctas, int32_t threads, int32_t order_kind);
 
 /* The schedule in use: out[0] threads per block (those that run: fewer than were

@@ -1179,10 +1179,12 @@ cudaError_t lift_smem_limit(StepKernel kern) {
 // resident CG's shared memory takes away (measured 2 times slower), while one
 // that fits gains a factor of about 3: the resident kernel is taken when at
 // least 60% of the rows lie in sequences that fit.
-// Where most rows are in slot form the products need no index loads, and 512
-// threads per SM with 128 registers keep more values in flight than 1,024 with
-// 64 do (64 sequences, ms a step: clusters of 8 33 against 41, one block each
-// 244 against 304): such a launch runs at most 512.
+// Where most rows have common offsets, five at most, the products need no index
+// loads, and 512 threads per SM with 128 registers keep more values in flight than
+// 1,024 with 64 do (64 sequences, ms a step: clusters of 8 33 against 41, one block
+// each 244 against 304): such a launch runs at most 512.  Wider rows are taken slot
+// by slot and want the warps that were set (200 sequences of 80,000 rows, one block
+// each, 512 and 1,024 threads: seven offsets 73.4 and 46.0 ms, 23 offsets 359 and 283).
 struct StepLaunch {
     StepKernel kern;
     size_t smem;
@@ -1214,7 +1216,7 @@ StepLaunch step_launch(const seq_batch* bt) {
     for (const BatchSeq& q : bt->host) {
         all += q.n;
         if (!q.slot) continue;
-        slot += q.n;
+        if (q.list.count > 0 && q.slot_w <= kBW) slot += q.n;
         if (most >= (long long)need &&
             batch_resident(q.n, q.slot_w, q.reach, bt->cluster, (size_t)most, &L))
             fits += q.n;

@@ -369,3 +369,21 @@ def test_batch_with_long_reaches(ctas, reaches):
         for b, x, i in zip(bs, xs, infos):
             assert i["status"] == 0
             assert np.linalg.norm(b - A @ x.cpu().numpy()) <= 1.01e-11 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("offsets,threads", [([1, 264], 512), ([1, 2, 264], 1024), (list(range(1, 12)), 1024)])
+def test_batch_threads_of_sequences_off_the_chip(offsets, threads):
+    """70,000 rows do not fit one block's shared memory: five common offsets run 512
+    threads, wider rows the threads that were set."""
+    import paper_2309_02156_gb300 as sa
+    rng = np.random.default_rng(len(offsets))
+    n = 70000
+    A = _spd(n, offsets, rng)
+    b = rng.standard_normal(n)
+    bt = sa.Batch([(_dev(A.indptr, np.int32), _dev(A.indices, np.int32))], M=2, s=8, zeta=2)
+    bt.set_schedule(1024, 1, 0)
+    assert bt.schedule()["threads"] == threads
+    x = _dev(np.zeros(n), np.float64)
+    info = bt.step([_dev(A.data, np.float64)], [_dev(b, np.float64)], [x], 1e-11)[0]
+    bt.close()
+    assert info["status"] == 0 and np.linalg.norm(b - A @ x.cpu().numpy()) <= 1.01e-11 * np.linalg.norm(b)
